@@ -141,6 +141,7 @@ extern "C" mhc_status mhc_correlator_backward(mhc_plan_t plan, const double* con
   if (st != MHC_OK) return st;
   BwdArgs b;
   if ((st = fill_fwd_args(p, S_f, w_src_dev, w_snk_dev, b.a)) != MHC_OK) return st;
+  b.a.fx = fx::Tables();  // the adjoint works on FP64 factors (kfac writes the format a.fx asks for)
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int F = p.F;
   int ysl = b.a.slots, mn_max = 1, Mmax = 0, Lmax = 1;  // ysl: the cached solves' slots

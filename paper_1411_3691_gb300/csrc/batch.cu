@@ -38,6 +38,7 @@ mhc_status ensure_device(Plan& p);
 mhc_status fill_fwd_args(Plan& p, const double* const* S_f, const double* w_src,
                          const double* w_snk, FwdArgs& a);
 void plan_slots(const Plan& p, int* yoff, int* total);
+size_t fx_layout(const Plan& p, char* base, fx::Tables* t);
 
 namespace {
 
@@ -124,10 +125,13 @@ struct mhc_batch_s {
   int64_t* d_kpref = nullptr;     // [count + 1] first two-sided block thread of each plan
   int64_t* d_nfam = nullptr;      // [count] families per plan
   int64_t k_total = 0;
+  int64_t* d_fxpref = nullptr;    // [count + 1] first block of each plan's fixed-point tables
+  int64_t fx_total = 0;
   int k_big = 0;                  // a two-sided plan has a flavour with n > 6
   // a plan given more than once (one plan, several propagator sets: gauge configurations,
-  // time slices) gets batch-owned block factors and guard flags for its later entries
-  std::vector<void*> own_kbuf, own_kguard;  // [count], null where the plan's own are used
+  // time slices) gets batch-owned block factors, guard flags and fixed-point tables for its
+  // later entries
+  std::vector<void*> own_kbuf, own_kguard, own_fx;  // [count], null where the plan's own are used
   cudaStream_t side = nullptr;    // second branch: the class kernels run concurrently
   cudaEvent_t fork = nullptr, join = nullptr;
   std::vector<const void*> key;  // S and out pointers the graph was captured with
@@ -184,7 +188,7 @@ BatchShape make_shape(const mhc_batch_s& b, const int (&Tc)[kClasses]) {
     for (auto& x : all[c]) sh.items.push_back(x.it);
     const int64_t n = (int64_t)all[c].size();
     if (n == 0) continue;
-    sh.cls_smem[c] = forward_smem_bytes(max_slots[c], Tc[c]);
+    sh.cls_smem[c] = forward_smem_bytes(max_slots[c], Tc[c], kClassNc[c]);
     const int occ = c == 0 ? batch_occupancy_nc8(Tc[c], sh.cls_smem[c])
                            : (c == 1 ? batch_occupancy_nc18(Tc[c], sh.cls_smem[c])
                                      : batch_occupancy_nc32(Tc[c], sh.cls_smem[c]));
@@ -287,6 +291,7 @@ mhc_status fill_descs(mhc_batch_s& b, const BatchShape& sh, const double* const*
   desc.resize(b.count);
   b.own_kbuf.resize(b.count, nullptr);
   b.own_kguard.resize(b.count, nullptr);
+  b.own_fx.resize(b.count, nullptr);
   for (int k = 0; k < b.count; k++) {
     const Plan& p = *b.plans[k];
     mhc_status st = fill_fwd_args(*b.plans[k], S[k], nullptr, nullptr, desc[k]);
@@ -294,6 +299,15 @@ mhc_status fill_descs(mhc_batch_s& b, const BatchShape& sh, const double* const*
     desc[k].n_tiles = sh.n_tiles[k];
     bool repeat = false;
     for (int k2 = 0; k2 < k; k2++) repeat |= b.plans[k2] == b.plans[k];
+    if (repeat && desc[k].fx.nf > 0) {
+      fx::Tables t;
+      const size_t bytes = fx_layout(p, nullptr, &t);
+      if (!b.own_fx[k] && cudaMalloc(&b.own_fx[k], bytes) != cudaSuccess) {
+        set_error("mhc_batch: cudaMalloc failed for a repeated plan's fixed-point tables");
+        return MHC_ENOMEM;
+      }
+      fx_layout(p, reinterpret_cast<char*>(b.own_fx[k]), &desc[k].fx);
+    }
     if (repeat && desc[k].snk_orig) {
       if (!b.own_kbuf[k]) {
         const size_t nk = (size_t)p.n_fam * p.n_qfam * desc[k].kstride * sizeof(double2);
@@ -346,6 +360,8 @@ cudaError_t launch_class(const mhc_batch_s& b, const BatchShape& sh, int c, cuda
 }
 
 cudaError_t launch_kfac(const mhc_batch_s& b, const BatchShape& sh, cudaStream_t s) {
+  const cudaError_t e = launch_fxprep_batch(b.d_desc, b.d_fxpref, b.count, b.fx_total, s);
+  if (e != cudaSuccess) return e;
   if (sh.ncmax <= 8) return launch_kfac_batch_nc8(b.d_desc, b.d_kpref, b.d_nfam, b.count, b.k_total, b.k_big, s);
   if (sh.ncmax <= 18) return launch_kfac_batch_nc18(b.d_desc, b.d_kpref, b.d_nfam, b.count, b.k_total, b.k_big, s);
   return launch_kfac_batch_nc32(b.d_desc, b.d_kpref, b.d_nfam, b.count, b.k_total, b.k_big, s);
@@ -395,12 +411,14 @@ void destroy(mhc_batch_s* b) {
   }
   if (b->exec) cudaGraphExecDestroy(b->exec);
   void* ptrs[] = {b->d_desc, b->d_items, b->d_part_off, b->d_partials, b->d_head, b->d_outs,
-                  b->d_kpref, b->d_nfam};
+                  b->d_kpref, b->d_nfam, b->d_fxpref};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (void* p : b->own_kbuf)
     if (p) cudaFree(p);
   for (void* p : b->own_kguard)
+    if (p) cudaFree(p);
+  for (void* p : b->own_fx)
     if (p) cudaFree(p);
   if (b->cap) cudaStreamDestroy(b->cap);
   if (b->side) cudaStreamDestroy(b->side);
@@ -437,21 +455,27 @@ mhc_status mhc_batch_create(mhc_batch_t* out, int32_t count, const mhc_plan_t* p
     }
     b->plans.push_back(p);
   }
-  std::vector<int64_t> kpref(1, 0), nfam;
+  std::vector<int64_t> kpref(1, 0), nfam, fxpref(1, 0);
   for (int k = 0; k < count; k++) {
     const Plan& p = *b->plans[k];
     nfam.push_back(p.n_fam);
+    int64_t nb = p.dev.fx ? p.n_fam : 0;
+    for (int f = 0; f < p.F && p.dev.fx; f++) nb += p.n_f[f] > 0 ? p.L_f[f] : 0;
+    fxpref.push_back(fxpref.back() + nb);
     kpref.push_back(kpref.back() + (p.dev.two_sided ? p.n_fam * p.n_qfam * p.F : 0));
     for (int f = 0; f < p.F; f++) b->k_big |= (p.dev.two_sided && p.n_f[f] > 6) ? 1 : 0;
   }
   b->k_total = kpref.back();
+  b->fx_total = fxpref.back();
   if (cudaMalloc(&b->d_kpref, sizeof(int64_t) * (count + 1)) != cudaSuccess ||
+      cudaMalloc(&b->d_fxpref, sizeof(int64_t) * (count + 1)) != cudaSuccess ||
       cudaMalloc(&b->d_nfam, sizeof(int64_t) * count) != cudaSuccess) {
     destroy(b);
     set_error("mhc_batch_create: CUDA allocation failed");
     return MHC_ENOMEM;
   }
   cudaMemcpy(b->d_kpref, kpref.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice);
+  cudaMemcpy(b->d_fxpref, fxpref.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice);
   cudaMemcpy(b->d_nfam, nfam.data(), sizeof(int64_t) * count, cudaMemcpyHostToDevice);
   if (cudaMalloc(&b->d_desc, sizeof(FwdArgs) * count) != cudaSuccess ||
       cudaMalloc(&b->d_head, sizeof(unsigned long long) * kClasses) != cudaSuccess ||

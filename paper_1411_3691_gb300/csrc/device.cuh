@@ -63,6 +63,16 @@ __device__ __forceinline__ cd crcp(cd z) {
 
 __device__ __forceinline__ cd ldS(const cd* __restrict__ p) { return __ldg(p); }
 
+}  // namespace dev
+
+// fixed-point limbs of block factors (fx.cuh)
+namespace fx {
+__device__ __forceinline__ int4 factor_limbs(dev::cd z, int e);
+__device__ __forceinline__ bool exponents_ok(int eu, int er);
+}  // namespace fx
+
+namespace dev {
+
 // ------------------------------------------------------------------------------------
 // Shared-row factorisation of one (family, sink, flavour) block.
 //
@@ -649,7 +659,7 @@ template <int NC, int NFIX, int RHO>
 __device__ __forceinline__ bool kfac_block(const cd* __restrict__ S, int L, int n_rt,
                                            const int32_t* __restrict__ arow,
                                            const int32_t* __restrict__ scol, cd* __restrict__ K,
-                                           int kp) {
+                                           int kp, bool fxf) {
   constexpr int UNR = NFIX ? NC : 1;
   const int n = NFIX ? NFIX : n_rt;
   const int M = n - RHO;
@@ -704,6 +714,24 @@ __device__ __forceinline__ bool kfac_block(const cd* __restrict__ S, int L, int 
   }
   if (M > 0 && (zero || emax - emin > kp)) return true;
   const cd sd = parity ? cneg(det) : det;
+  if (fxf && RHO == 1) {  // the same factors as limbs (fx.cuh, solve)
+    int4* X = reinterpret_cast<int4*>(K);
+#pragma unroll UNR
+    for (int i = 0; i < M; i++) {
+      int eu = -4096;
+#pragma unroll UNR
+      for (int u = i + 1; u < M; u++) eu = max(eu, expo(B[i][u]));
+      const int er = expo(B[i][i]) + 1;
+      eu = max(eu + 1, -er);
+      if (!fx::exponents_ok(eu, er)) return true;
+#pragma unroll UNR
+      for (int u = 0; u < M; u++) X[i * M + u] = fx::factor_limbs(B[i][u], u < i ? 1 : u == i ? er : eu);
+      X[M * M + i] = make_int4(arow[perm[i]] * L, eu, er, 0);
+    }
+    K[M * M + M] = cneg(sd);
+    K[M * M + M + 1] = sd;
+    return false;
+  }
 #pragma unroll UNR
   for (int i = 0; i < M; i++) {
 #pragma unroll UNR
@@ -946,7 +974,8 @@ template <int G>
 __device__ __forceinline__ bool group_kfac_block(const cd* __restrict__ S, int L, int n, int rho,
                                                  const int32_t* __restrict__ arow,
                                                  const int32_t* __restrict__ scol, cd* __restrict__ K,
-                                                 int kp, int g, unsigned gm, cd* Bs, cd* Ws, int* Ps) {
+                                                 int kp, int g, unsigned gm, cd* Bs, cd* Ws, int* Ps, int pn,
+                                                 bool fxf) {
   const int M = n - rho;
   const int C = rho == 2 ? M + 1 : M;
   const int P = group_pitch(C);
@@ -975,11 +1004,36 @@ __device__ __forceinline__ bool group_kfac_block(const cd* __restrict__ S, int L
       __syncwarp(gm);
     }
   }
-  for (int e = g; e < M * M; e += G) {
-    const int i = e / M, u = e - i * M;
-    K[e] = Bs[i * P + u];
+  if (fxf) {  // the same factors as limbs (fx.cuh, solve); Ps + pn, Ps + 2 pn: eU_i, er_i
+    int4* X = reinterpret_cast<int4*>(K);
+    bool bad = false;
+    int enu = -4096;  // exponent above -U1^{-1} u
+    for (int i = g; i < M; i += G) {
+      int eu = -4096;
+      for (int u = i + 1; u < M; u++) eu = max(eu, expo(Bs[i * P + u]));
+      const int er = expo(Bs[i * P + i]) + 1;
+      eu = max(eu + 1, -er);
+      bad |= !fx::exponents_ok(eu, er);
+      Ps[pn + i] = eu;
+      Ps[2 * pn + i] = er;
+      if (rho == 2) enu = max(enu, expo(Ws[i]) + 1);
+    }
+#pragma unroll
+    for (int off = 1; off < G; off <<= 1) enu = max(enu, __shfl_xor_sync(gm, enu, off));
+    if (__any_sync(gm, bad || enu > 900)) return true;
+    __syncwarp(gm);
+    for (int e = g; e < M * M; e += G) {
+      const int i = e / M, u = e - i * M;
+      X[e] = fx::factor_limbs(Bs[i * P + u], u < i ? 1 : Ps[(u == i ? 2 * pn : pn) + i]);
+    }
+    for (int i = g; i < M; i += G) X[M * M + i] = make_int4(arow[Ps[i]] * L, Ps[pn + i], Ps[2 * pn + i], enu);
+  } else {
+    for (int e = g; e < M * M; e += G) {
+      const int i = e / M, u = e - i * M;
+      K[e] = Bs[i * P + u];
+    }
+    for (int i = g; i < M; i += G) K[M * M + i] = make_double2((double)Ps[i], 0.0);
   }
-  for (int i = g; i < M; i += G) K[M * M + i] = make_double2((double)Ps[i], 0.0);
   if (rho == 1) {
     if (g == 0) {
       K[M * M + M] = cneg(sd);

@@ -7,26 +7,42 @@ namespace mhc {
 
 namespace {
 
-// Sum of the per-item partials in a fixed order (one block of 1024 threads).
-__global__ void __launch_bounds__(1024) reduce_kernel(const double2* __restrict__ partials,
-                                                      int64_t n, double* out) {
-  __shared__ double2 red[32];
-  double2 s = make_double2(0.0, 0.0);
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    s.x += partials[i].x;
-    s.y += partials[i].y;
-  }
-  s = dev::warp_sum(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
+// Sum of the per-item partials in a fixed order: every block sums a slice of its own, the last one
+// to finish (by a counter that it sets back) the blocks' sums.  One block took 12.5 us for the 8192 partials of the He-4 shapes.
+constexpr int kReduceBlocks = kReduceMaxBlocks, kReduceThreads = 256;
+__global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const double2* __restrict__ p, int64_t n, double2* blocks,
+                                                                unsigned* done, double* out) {
+  __shared__ double2 red[kReduceThreads / 32];
+  __shared__ bool last;
+  auto block_sum = [&](double2 s) {
+    s = dev::warp_sum(s);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
     double2 t = red[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-      t.x += red[w].x;
-      t.y += red[w].y;
-    }
-    out[0] = t.x;
-    out[1] = t.y;
+    for (int w = 1; w < kReduceThreads / 32; w++) t = dev::cadd(t, red[w]);
+    return t;
+  };
+  const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t i0 = per * blockIdx.x, i1 = i0 + per < n ? i0 + per : n;
+  double2 s = make_double2(0.0, 0.0);
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += kReduceThreads) s = dev::cadd(s, p[i]);
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    blocks[blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  s = make_double2(0.0, 0.0);
+  if (threadIdx.x < gridDim.x) s = __ldcg(blocks + threadIdx.x);
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    out[0] = s.x;
+    out[1] = s.y;
+    *done = 0;
   }
 }
 
@@ -42,12 +58,11 @@ __global__ void combine_cw(const double* __restrict__ t, double* __restrict__ ou
   }
 }
 
-size_t forward_smem_bytes(int slots, int tile) {
+size_t forward_smem_bytes(int slots, int tile, int ncmax) {
   const size_t cache = (size_t)slots * tile * sizeof(double2);
-  const size_t queue = (size_t)(tile / 32) * kQueueCap * kQueueEntryBytes;
-  const size_t z1 = (size_t)(tile / 32) * kZ1Bytes;
-  const size_t walk = (size_t)(tile / 32) * kWalkBytes;
-  return cache + queue + z1 + walk;
+  const size_t scratch = ncmax <= 8 ? WarpScratch<8>::kBytes : ncmax <= 18 ? WarpScratch<18>::kBytes : WarpScratch<32>::kBytes;
+  const size_t labels = (size_t)(slots + 2 * MHC_FMAX) * tile * sizeof(short);  // fwd::FxLane
+  return cache + (size_t)(tile / 32) * scratch + labels;
 }
 
 // fwd_kernel over items [0, items): one launch per layout range, each with its own y
@@ -67,7 +82,7 @@ static cudaError_t launch_fwd_items(const FwdArgs& a, int ncmax, int tile, int64
     ar.slots = g.slots;
     for (int f = 0; f < MHC_FMAX; f++) ar.yoff[f] = g.yoff[f];
     ar.item0 = g.first * a.n_tiles;
-    const cudaError_t e = one(ar, g.count * a.n_tiles, forward_smem_bytes(g.slots, tile));
+    const cudaError_t e = one(ar, g.count * a.n_tiles, forward_smem_bytes(g.slots, tile, ncmax));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -75,7 +90,8 @@ static cudaError_t launch_fwd_items(const FwdArgs& a, int ncmax, int tile, int64
 
 cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
                            size_t smem, double* out, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = launch_fxprep(a, s);
+  if (e != cudaSuccess) return e;
   if (a.snk_orig) {  // two-sided update: the LU factors of every (family, sink family) block first
     TraceRange trace("block factors");
     if (ncmax <= 8)
@@ -91,7 +107,7 @@ cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam,
     if ((e = launch_fwd_items(a, ncmax, tile, items, smem, s)) != cudaSuccess) return e;
   }
   TraceRange trace("reduce");
-  return launch_reduce(a.partials, items, out, s);
+  return launch_reduce(a, items, out, s);
 }
 
 cudaError_t launch_forward_cw(const FwdArgs& a0, const double* const* ws, const double* const* wk,
@@ -107,15 +123,18 @@ cudaError_t launch_forward_cw(const FwdArgs& a0, const double* const* ws, const 
     FwdArgs a = a0;
     a.w_src = ws[k >> 1];
     a.w_snk = wk[k & 1];
+    if ((k & 1) == 0 && (e = launch_fxprep(a, s)) != cudaSuccess) return e;  // the source weights' tables
     if ((e = launch_fwd_items(a, ncmax, tile, items, smem, s)) != cudaSuccess) return e;
-    if ((e = launch_reduce(a.partials, items, tmp + 2 * k, s)) != cudaSuccess) return e;
+    if ((e = launch_reduce(a, items, tmp + 2 * k, s)) != cudaSuccess) return e;
   }
   combine_cw<<<1, 32, 0, s>>>(tmp, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const double2* partials, int64_t items, double* out, cudaStream_t s) {
-  reduce_kernel<<<1, 1024, 0, s>>>(partials, items, out);
+cudaError_t launch_reduce(const FwdArgs& a, int64_t items, double* out, cudaStream_t s) {
+  const int64_t b = (items + kReduceThreads - 1) / kReduceThreads;
+  reduce_kernel<<<(unsigned)(b < kReduceBlocks ? b : kReduceBlocks), kReduceThreads, 0, s>>>(
+      a.partials, items, a.reduce_blocks, a.reduce_done, out);
   return cudaGetLastError();
 }
 

@@ -4,7 +4,9 @@
 // One thread block per work item (work family W, tile of `tile` sinks); one thread per
 // sink.  Per flavour a thread factorises the family's shared rows against its sink's
 // columns (shared_rows) and caches y = det(G) G^{-1} e_r in shared memory; then every
-// member of the family costs one O(n) dot product per flavour (member_det), Sec. 2.1.
+// member of the family costs one O(n) dot product per flavour, Sec. 2.1: in fixed point on the
+// integer pipe (fx_dots, fx_det2), or in FP64 (member_det) where the fixed-point value is out of
+// its range or near the lemma guard.
 // Two-sided blocks (a family against a sink family) take y from factors stored once per
 // block (kapply*).  Members whose lemma factor or whose family pivots fail the guards go
 // to a per-warp queue and are refactored from scratch 32 at a time -- pairs that share the
@@ -249,16 +251,33 @@ __device__ __forceinline__ dev::cd group_fresh(const FwdArgs& a, int W, int f, i
   return parity ? dev::cneg(det) : det;
 }
 
+// does the sink family's block hold fixed-point factors of the one-column kind
+__device__ __forceinline__ bool fx_block(const FwdArgs& a, int W, int Q, int f, bool qtwo) {
+  return a.fx.nf > 0 && qtwo && a.q_rank[(int64_t)Q * a.F + f] == 1 && a.fam_rank[(int64_t)W * a.F + f] <= 2 &&
+         !a.kguard[((int64_t)W * a.n_q + Q) * a.F + f];
+}
+
+// complex factor of a flavour's fixed-point solve: det B of a block solved in fixed point, sd of
+// a two-row family, else 1
+__device__ __forceinline__ dev::cd fx_factor(const FwdArgs& a, int W, int Q, int f, bool blk, const double2* Yf, int T) {
+  const int n = a.n_f[f];
+  if (a.fam_rank[(int64_t)W * a.F + f] == 2) return Yf[2 * n * T];
+  if (!blk) return make_double2(1.0, 0.0);
+  return a.kbuf[((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f] + (n - 1) * (n - 1) + n];
+}
+
 // Refactor one pair per lane (the lanes with have; e: the pair, j: its sink position):
 // the product of the flavours that passed, times fresh determinants of the flavours that
 // failed, accumulated into acc.  With a.rowdiff the row-difference update is tried first
 // for members of one- and two-row families.  Pairs that share a member and a two-sided sink
 // family with one or two changed columns (n <= 18) are factorised together (group_fresh);
 // the others one per lane.  Yw: the warp's cached solves (lane l at Yw + l, stride
-// blockDim.x); wk: the warp's scratch for group_fresh.  Called by the whole warp.
+// blockDim.x), in fixed point with exponents eyw when fxm; wk: the warp's scratch for group_fresh.
+// Called by the whole warp; a call, not inlined: the member loop keeps its registers and the
+// instruction cache its lines.
 template <int NCMAX>
-__device__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
-                              const double2* Yw, double2* wk, double2& acc, unsigned long long& rflops,
+__device__ __noinline__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
+                              const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc, unsigned long long& rflops,
                               unsigned long long& nrd) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -277,16 +296,28 @@ __device__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& 
       const int rho = a.fam_rank[(int64_t)W * a.F + f];
       if (!((cand >> f) & 1) || rho > 2 || n < rho + 1) continue;
       const double2* Yf = Yw + (size_t)a.yoff[f] * T + e.lane;
-      const int ey = dev::cached_scale(Yf, T, n, rho);
+      double2 yl[2 * NCMAX + 1];  // the solve of the pair's sink
+      if (fxm) {
+        const int e2 = eyw[f * T + e.lane], eq = e2 >> 1;
+        const double2 fac = fx_factor(a, W, Q, f, e2 & 1, Yf, T);
+        for (int q = 0; q < rho * n; q++) {
+          yl[q] = fx::value(reinterpret_cast<const int4*>(Yf)[q * T], eq);
+          if (rho == 1) yl[q] = dev::cmul(yl[q], fac);
+        }
+        if (rho == 2) yl[2 * n] = fac;
+      } else {
+        for (int q = 0; q < rho * n + (rho == 2); q++) yl[q] = Yf[q * T];
+      }
+      const int ey = dev::cached_scale(yl, 1, n, rho);
       bool f2 = true;
       const int32_t* mlab = a.mem_lab + ((int64_t)e.member * a.F + f) * MHC_MAX_RANK;
       const int32_t* arow = a.fam_arow + (int64_t)W * a.Tn + a.off_f[f];
       double2 d;
       if constexpr (NCMAX >= 10)  // two-row families need n_f >= 10
-        d = rho == 1 ? dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], Yf, T, ey, a.kc, &f2)
-                     : dev::rowdiff2_det(a.S[f], a.L_f[f], n, mlab, arow, cols + a.off_f[f], Yf, T, ey, a.kc, &f2);
+        d = rho == 1 ? dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2)
+                     : dev::rowdiff2_det(a.S[f], a.L_f[f], n, mlab, arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2);
       else
-        d = dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], Yf, T, ey, a.kc, &f2);
+        d = dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2);
       rflops += rho == 1 ? dev::rowdiff_flops(n) : dev::rowdiff2_flops(n);
       if (!f2) {
         prod = dev::cmul(prod, d);
@@ -334,17 +365,208 @@ __device__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& 
 // Refactor the first count queued pairs (one per lane).  Called by the whole warp.
 template <int NCMAX>
 __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int64_t jbase,
-                              const double2* Yw, double2* wk, double2& acc, unsigned long long& rflops,
-                              unsigned long long& nrd) {
+                              const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc,
+                              unsigned long long& rflops, unsigned long long& nrd) {
   const int lane = threadIdx.x & 31;
   const bool have = lane < count;
   QEntry e = {};
   if (have) e = q[lane];
-  process_pairs<NCMAX>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, wk, acc, rflops, nrd);
+  process_pairs<NCMAX>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, fxm, eyw, wk, acc, rflops, nrd);
+}
+
+// ---- solves and member dots in fixed point (fx.cuh) -------------------------------------
+// The warp's cached solves are fixed-point vectors in the y cache (rank 1: the n entries of y up
+// to a complex factor; rank 2: the 2 n entries of z1 and z2, sd stays FP64), with two shorts per
+// flavour and lane beside the column labels: the vector's exponent and how many binades its
+// largest entry lies below it.
+struct FxLane {
+  unsigned short* lab;  // [slot][T] column labels, at the lane
+  short* ey;            // [F][T] 2 e_y (an entry of 2^56 stands for 2^e_y), + 1 when the block's det B is a factor
+  short* low;           // [F][T] binades of the largest entry below 2^56
+};
+template <int NCMAX>
+__device__ __forceinline__ FxLane fx_lane(const FwdArgs& a, double2* smem, int T) {
+  char* base = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)(T >> 5) * WarpScratch<NCMAX>::kBytes;
+  unsigned short* lab = reinterpret_cast<unsigned short*>(base);
+  short* ey = reinterpret_cast<short*>(lab + (size_t)a.slots * T);
+  return FxLane{lab, ey, ey + MHC_FMAX * T};
+}
+
+// Solve of one flavour in fixed point; false: the lane takes the FP64 factorisation.  Ks: the
+// block's factors staged in shared memory, or null.
+__device__ __forceinline__ bool fx_solve(const FwdArgs& a, int W, int Q, int f, const int32_t* col, const int4* Ks,
+                                         double2* Yf, int T, short* ey, short* low) {
+  const int n = a.n_f[f], rho = a.fam_rank[(int64_t)W * a.F + f], M = n - rho;
+  const double2* K = a.kbuf + ((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f];
+  const int4* Kg = reinterpret_cast<const int4*>(K);
+  int4* z = reinterpret_cast<int4*>(Yf) + (rho == 2 ? n * T : 0);
+  const int c = col[n - 1], ea = a.fx.cexp[f][c];
+  if (ea > 900 || ea < -900) return false;
+  const int zlo = rho == 2 ? max(0, __ldg(Kg + M * M).w) : 0;
+  int u = zlo - 55, mag = 0;
+  if (M > 0) {
+    const int4* ac = a.fx.sc[f] + c;
+    const bool ok = Ks ? fx::solve<true>(M, ac, ea, zlo, Ks, z, T, &u, &mag)
+                       : fx::solve<false>(M, ac, ea, zlo, Kg, z, T, &u, &mag);
+    if (!ok) return false;
+  }
+  // the unit entries; u >= -55, and an entry 1 below the unit is lost against the others
+  const fx::Val unit{u <= 0 ? 1ll << -u : 0ll, 0ll};
+  const int4 one = fx::limbs(unit), zero = make_int4(0, 0, 0, 0);
+  mag = max(mag, fx::magnitude(unit));
+  if (rho == 2) {
+    z[M * T] = zero;
+    z[(M + 1) * T] = one;
+    int4* z1 = reinterpret_cast<int4*>(Yf);
+    for (int q = 0; q < M; q++) {
+      const int4 v = fx::quant(__ldg(K + M * M + M + q), u + fx::kFracBits, fx::kFracBits);
+      z1[q * T] = v;
+      mag = max(mag, fx::magnitude(fx::joined(v)));
+    }
+    z1[M * T] = one;
+    z1[(M + 1) * T] = zero;
+    Yf[2 * n * T] = __ldg(K + M * M + 2 * M);
+  } else {
+    z[M * T] = one;
+  }
+  int top = 64 - __clz(mag);  // bits of the largest entry (32 when below 2^32)
+  if (top > fx::kFracBits) {
+    const int sh = top - fx::kFracBits;
+    for (int q = 0; q < rho * n; q++) {
+      int4& v = reinterpret_cast<int4*>(Yf)[q * T];
+      const fx::Val x = fx::joined(v);
+      v = fx::limbs(x.re >> sh, x.im >> sh);
+    }
+    u += sh;
+    top = fx::kFracBits;
+  }
+  *ey = (short)(2 * (u + fx::kFracBits) + 1);
+  *low = (short)(fx::kFracBits - top);
+  return true;
+}
+
+// The block factors of flavour f of the warp's sinks, copied to its scratch: a solve walks them
+// row by row, every row waiting for a few loads, which from global memory cost hundreds of clocks
+// each.  Sinks stand in family order, so the warp's blocks are those of families Q0 .. Q1.  Returns
+// the lane's block, or null (kept in global memory) when they do not fit.  Called by the whole
+// warp; the caller's solves end before the next call.
+template <int NCMAX>
+__device__ __forceinline__ const int4* fx_stage(const FwdArgs& a, int W, int Q, int f, int lane, void* scratch) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int M = a.n_f[f] - a.fam_rank[(int64_t)W * a.F + f], blk = M * (M + 1);
+  const int Q0 = __shfl_sync(FULL, Q, 0), cnt = __shfl_sync(FULL, Q, 31) - Q0 + 1;
+  if (Q0 < 0 || cnt * blk > WarpScratch<NCMAX>::kBytes / 16) return nullptr;
+  const int4* src = reinterpret_cast<const int4*>(a.kbuf + ((int64_t)W * a.n_q + Q0) * a.kstride + a.koff[f]);
+  int4* dst = reinterpret_cast<int4*>(scratch);
+  __syncwarp();
+  for (int q = 0; q < cnt; q++)
+    for (int e = lane; e < blk; e += 32) dst[q * blk + e] = __ldg(src + (size_t)q * a.kstride + e);
+  __syncwarp();
+  return dst + (Q - Q0) * blk;
+}
+
+// A flavour's FP64 solve to fixed point, in place; ey: the member guard's scale exponent as the
+// FP64 producers define it.  false (and nothing changed): not finite, or without a normal exponent.
+__device__ __forceinline__ bool fx_from_fp64(int n, int rho, double2* Yf, int T, int ey, short* out_e, short* low) {
+  if (rho == 2) {
+    const double2 sd = Yf[2 * n * T];
+    if (!dev::finite2(sd) || dev::expo(sd) < -900) return false;
+    ey = (ey - dev::expo(sd)) >> 1;
+  }
+  if (ey >= 900 || ey <= -900) return false;
+  for (int q = 0; q < rho * n; q++) reinterpret_cast<int4*>(Yf)[q * T] = fx::quant(Yf[q * T], ey + 1, fx::kFracBits);
+  *out_e = (short)(2 * (ey + 1));
+  *low = 0;
+  return true;
+}
+
+// back to FP64 in place (the lanes of a warp that leaves the fixed-point path)
+static __device__ __noinline__ void fx_to_fp64(int n, int rho, double2* Yf, int T, int ey, dev::cd factor) {
+  for (int q = 0; q < rho * n; q++) {
+    const dev::cd v = fx::value(reinterpret_cast<const int4*>(Yf)[q * T], ey);
+    Yf[q * T] = rho == 1 ? dev::cmul(v, factor) : v;
+  }
+}
+
+// g . y of kN members' rows (rank 1).  The members share each load of y and give the integer pipe
+// independent sums; the rows' entries are one address for the lanes of a sink family but in its
+// changed column.
+template <int kN>
+__device__ __forceinline__ void fx_dots(int n, const int4* const (&r)[kN], const unsigned short* lab, const int4* Y,
+                                        int T, fx::Val (&v)[kN]) {
+  fx::Acc s[kN];
+#pragma unroll 1
+  for (int q = 0; q < n; q++) {
+    const int o = lab[q * T];
+    const int4 y = Y[q * T];
+#pragma unroll
+    for (int k = 0; k < kN; k++) fx::mac(s[k], __ldg(r[k] + o), y);
+  }
+#pragma unroll
+  for (int k = 0; k < kN; k++) v[k] = fx::finish(s[k]);
+}
+
+// det(B Z) of one member's two rows against z1, z2 (rank 2); a dot too large for the product's
+// limbs gives 0, which no threshold lets pass.
+__device__ __forceinline__ fx::Val fx_det2(int n, const int4* __restrict__ r1, const int4* __restrict__ r2,
+                                           const unsigned short* lab, const int4* Y, int T) {
+  fx::Acc s11, s12, s21, s22;
+#pragma unroll 1
+  for (int q = 0; q < n; q++) {
+    const int o = lab[q * T];
+    const int4 z1 = Y[q * T], z2 = Y[(n + q) * T];
+    const int4 a = __ldg(r1 + o), b = __ldg(r2 + o);
+    fx::mac(s11, a, z1);
+    fx::mac(s12, a, z2);
+    fx::mac(s21, b, z1);
+    fx::mac(s22, b, z2);
+  }
+  const fx::Val d11 = fx::finish(s11), d12 = fx::finish(s12), d21 = fx::finish(s21), d22 = fx::finish(s22);
+  const bool ok = max(max(fx::magnitude(d11), fx::magnitude(d12)), max(fx::magnitude(d21), fx::magnitude(d22))) < fx::kMulHi;
+  const fx::Val p = fx::mul(fx::split(d11), fx::split(d22)), m = fx::mul(fx::split(d12), fx::split(d21));
+  return ok ? fx::Val{p.re - m.re, p.im - m.im} : fx::Val{0, 0};  // half the determinant
+}
+
+// One member's determinant in FP64 from a fixed-point solve, with the FP64 lemma guard: the pairs
+// whose fixed-point value is out of range or near the guard.  The solve's entries carry at least
+// the accuracy of FP64 ones at their largest entry's scale, which is the guard's scale.
+static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S, int L, int n, int rho,
+                                            const int32_t* __restrict__ lab, const int32_t* __restrict__ col,
+                                            const int4* Y, int T, int e, dev::cd factor, int kc, bool* fail) {
+  const dev::cd* r1 = S + (size_t)lab[0] * L;
+  dev::cd d = make_double2(0.0, 0.0);
+  int eb = -4096, ez = -4096;
+  if (rho == 1) {
+    for (int q = 0; q < n; q++) {
+      const dev::cd y = dev::cmul(fx::value(Y[q * T], e), factor), b = dev::ldS(r1 + col[q]);
+      ez = max(ez, dev::expo(y));
+      eb = max(eb, dev::expo(b));
+      d = dev::cfma(b, y, d);
+    }
+    *fail = dev::expo(d) < eb + ez - kc;
+    return d;
+  }
+  const dev::cd* r2 = S + (size_t)lab[1] * L;
+  dev::cd d11 = d, d12 = d, d21 = d, d22 = d;
+  int e2 = -4096;
+  for (int q = 0; q < n; q++) {
+    const dev::cd z1 = fx::value(Y[q * T], e), z2 = fx::value(Y[(n + q) * T], e);
+    const dev::cd b1 = dev::ldS(r1 + col[q]), b2 = dev::ldS(r2 + col[q]);
+    ez = max(ez, max(dev::expo(z1), dev::expo(z2)));
+    eb = max(eb, dev::expo(b1));
+    e2 = max(e2, dev::expo(b2));
+    d11 = dev::cfma(b1, z1, d11);
+    d12 = dev::cfma(b1, z2, d12);
+    d21 = dev::cfma(b2, z1, d21);
+    d22 = dev::cfma(b2, z2, d22);
+  }
+  d = dev::cmul(factor, dev::cfms(d12, d21, dev::cmul(d11, d22)));
+  *fail = dev::expo(d) < eb + e2 + dev::expo(factor) + 2 * max(ez, 0) - kc;
+  return d;
 }
 
 // One work item (family W x sink tile) by the whole thread block; the block's sum goes
-// to *partial.  Shared by the per-plan launch and the persistent batched launch.
+// to *partial.  Shared by the per-plan launch and the persistent batched launch. 
 template <int NCMAX>
 __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, double2* smem,
                                          double2* partial) {
@@ -357,11 +579,20 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   const int Q = a.snk_orig ? a.snk_q[j] : -1;
   const bool qtwo = Q >= 0 && a.q_two[Q];
   const int mem0 = a.fam_info[4 * W], kW = a.fam_info[4 * W + 1];
-  QEntry* queue = reinterpret_cast<QEntry*>(smem + (size_t)a.slots * T) + warp * kQueueCap;
+  using WS = WarpScratch<NCMAX>;
+  char* scratch = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)warp * WS::kBytes;
+  QEntry* queue = reinterpret_cast<QEntry*>(scratch);
   double2* Y = smem + tid;
   const double2* Yw = smem + (tid & ~31);  // the warp's cached solves (lane l: Yw + l)
 
-  // ---- per flavour: factorise the shared rows against this sink ----------------------
+  // ---- per flavour: solve, or factorise the shared rows, for this sink ----------------
+  constexpr bool kFx = NCMAX <= 18;
+  const FxLane fl = fx_lane<NCMAX>(a, smem, T);
+  bool fxm = kFx && a.fx.nf > 0 && kW <= 2 * fx::kFlush, bad = false;
+  for (int f = 0; f < a.F; f++) fxm &= a.fam_rank[(int64_t)W * a.F + f] <= 2;
+  const short* eyw = fl.ey + (tid & ~31);
+  // flavours solved in fixed point; left to the FP64 factorisation; FP64 solves converted
+  unsigned infx = 0, solo = 0, made = 0;
   unsigned pguard = 0;
   dev::ScalesFor<NCMAX> eys;
   for (int f = 0; f < a.F; f++) {
@@ -371,27 +602,64 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
     const int rho = a.fam_rank[(int64_t)W * a.F + f];
     const int32_t* arow = a.fam_arow + (int64_t)W * a.Tn + a.off_f[f];
     const int sig = qtwo ? a.q_rank[(int64_t)Q * a.F + f] : 0;
-    if (qtwo && (rho == 1 || sig == 1 || (rho == 2 && sig == 2)) &&
-        !a.kguard[((int64_t)W * a.n_q + Q) * a.F + f]) {
-      const double2* K = a.kbuf + ((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f];
-      if (rho == 2 && sig == 2)
-        dev::dispatch_kapply22<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K,
-                                      Y + (size_t)a.yoff[f] * T, T, &ey);
-      else if (rho == 2)
-        dev::dispatch_kapply2<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K,
-                                     Y + (size_t)a.yoff[f] * T, T, &ey);
-      else if (sig == 2)
-        dev::dispatch_kapply12<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K,
-                                      Y + (size_t)a.yoff[f] * T, T, &ey);
-      else
-        dev::dispatch_kapply<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K,
-                                    Y + (size_t)a.yoff[f] * T, T, &ey);
-    } else {
-      const bool g = dev::dispatch_shared<NCMAX>(n, rho, a.S[f], a.L_f[f], arow, cols + a.off_f[f],
-                                                 Y + (size_t)a.yoff[f] * T, T, &ey, a.kp);
-      pguard |= (unsigned)g << f;
+    double2* Yf = Y + (size_t)a.yoff[f] * T;
+    bool done = false;
+    if constexpr (kFx) {
+      const bool blk = fx_block(a, W, Q, f, qtwo);
+      const int4* Ks = __any_sync(0xffffffffu, blk) ? fx_stage<NCMAX>(a, W, Q, f, lane, scratch) : nullptr;
+      if (blk) {
+        done = fx_solve(a, W, Q, f, cols + a.off_f[f], Ks, Yf, T, fl.ey + f * T + tid, fl.low + f * T + tid);
+        if (done) infx |= 1u << f; else solo |= 1u << f;
+      }
+    }
+    if (!done) {
+      if (!((solo >> f) & 1) && qtwo && (rho == 1 || sig == 1 || (rho == 2 && sig == 2)) &&
+          !a.kguard[((int64_t)W * a.n_q + Q) * a.F + f]) {
+        const double2* K = a.kbuf + ((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f];
+        if (rho == 2 && sig == 2)
+          dev::dispatch_kapply22<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K, Yf, T, &ey);
+        else if (sig == 2)
+          dev::dispatch_kapply12<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K, Yf, T, &ey);
+        else if (rho == 2)
+          dev::dispatch_kapply2<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K, Yf, T, &ey);
+        else
+          dev::dispatch_kapply<NCMAX>(n, a.S[f], a.L_f[f], arow, cols + a.off_f[f], K, Yf, T, &ey);
+      } else {
+        const bool g = dev::dispatch_shared<NCMAX>(n, rho, a.S[f], a.L_f[f], arow, cols + a.off_f[f], Yf, T, &ey, a.kp);
+        pguard |= (unsigned)g << f;
+      }
+      if constexpr (kFx) {
+        if (fxm && fx_from_fp64(n, rho, Yf, T, ey, fl.ey + f * T + tid, fl.low + f * T + tid)) made |= 1u << f;
+        bad |= fxm && !((made >> f) & 1);
+      }
     }
     eys.set(f, ey);
+  }
+
+  // ---- the member dots in fixed point, unless a sink of the warp has no usable solve (not
+  // finite, or its pivot guard fired) ------------------------------------------------------
+  int le = 0;                           // exponent of the lane's solves, all flavours
+  double2 lf = make_double2(1.0, 0.0);  // their factors
+  if constexpr (kFx) {
+    const bool keep = fxm && !__any_sync(0xffffffffu, bad || pguard != 0);
+    for (int f = 0; f < a.F; f++) {
+      const int n = a.n_f[f];
+      if (n == 0) continue;
+      const int rho = a.fam_rank[(int64_t)W * a.F + f];
+      double2* Yf = Y + (size_t)a.yoff[f] * T;
+      const int e = fl.ey[f * T + tid] >> 1;
+      const bool blk = (infx >> f) & 1;
+      if (keep) {
+        lf = dev::cmul(lf, fx_factor(a, W, Q, f, blk, Yf, T));
+        le += rho * e + (rho == 2);  // fx::mul halves
+        for (int q = 0; q < n; q++) fl.lab[(size_t)(a.yoff[f] + q) * T + tid] = (unsigned short)cols[a.off_f[f] + q];
+      } else if (blk || ((made >> f) & 1)) {
+        fx_to_fp64(n, rho, Yf, T, e, fx_factor(a, W, Q, f, blk, Yf, T));
+        eys.set(f, dev::cached_scale(Yf, T, n, rho));
+      }
+    }
+    fxm = keep;
+    __syncwarp();
   }
 
   // ---- rank-2 flavours against a one-column sink family shared by the warp's sinks: the
@@ -399,18 +667,14 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   // (two-row families need n_f >= 10: the classes below compile none of this)
   constexpr bool kZ1 = NCMAX >= 10;
   int zf0 = -1, zf1 = -1;
-  double2* z1d = reinterpret_cast<double2*>(reinterpret_cast<char*>(smem + (size_t)a.slots * T) +
-                                            (size_t)(T >> 5) * kQueueCap * kQueueEntryBytes +
-                                            (size_t)warp * kZ1Bytes);
+  double2* z1d = reinterpret_cast<double2*>(scratch + WS::kQueue);
   // the warp's scratch for the grouped refactors' multipliers (group_fresh)
-  double2* wk = reinterpret_cast<double2*>(reinterpret_cast<char*>(smem + (size_t)a.slots * T) +
-                                           (size_t)(T >> 5) * (kQueueCap * kQueueEntryBytes + kZ1Bytes) +
-                                           (size_t)warp * kWalkBytes);
+  double2* wk = reinterpret_cast<double2*>(scratch + WS::kQueue + WS::kZ1);
   // (the shuffle and the vote run on every lane: qtwo differs between lanes whose sinks
   // belong to a two-sided family and lanes whose sinks stand alone)
   const int Q0 = kZ1 ? __shfl_sync(0xffffffffu, Q, 0) : 0;
   const bool z1_warp = kZ1 && __all_sync(0xffffffffu, qtwo && Q == Q0);
-  if (kZ1 && z1_warp && kW <= 32) {
+  if (kZ1 && z1_warp && kW <= 32 && !fxm) {
     // the flavours are chosen from warp-uniform data only (W, Q), so every lane assigns the
     // same slots; such a flavour took kapply2 on every lane
     for (int f = 0; f < a.F && zf1 < 0; f++) {
@@ -440,7 +704,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   double2 acc = make_double2(0.0, 0.0), accq = make_double2(0.0, 0.0);
   int qn = 0;
   unsigned long long n_parent = 0, n_child = 0, n_rowdiff = 0, rflops = 0;
-  for (int c = 0; c < kW; c++) {
+  // one member in FP64: the lanes with part (the others' pairs are already summed)
+  auto member64 = [&](int c, bool part) {
     const int m = mem0 + c;
     unsigned fail = pguard;
     double2 prod = make_double2(1.0, 0.0);
@@ -453,7 +718,16 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       const int32_t* mlab = a.mem_lab + ((int64_t)m * a.F + f) * MHC_MAX_RANK;
       const double2* Yf = Y + (size_t)a.yoff[f] * T;
       double2 d;
-      if (kZ1 && (f == zf0 || f == zf1)) {
+      bool fixed = false;
+      if constexpr (kFx) {
+        if (fxm) {
+          d = fx_member64(a.S[f], a.L_f[f], n, rho, mlab, cols + a.off_f[f], reinterpret_cast<const int4*>(Yf), T,
+                          fl.ey[f * T + tid] >> 1, fx_factor(a, W, Q, f, (infx >> f) & 1, Yf, T), a.kc, &cf);
+          fixed = true;
+        }
+      }
+      if (fixed) {
+      } else if (kZ1 && (f == zf0 || f == zf1)) {
         const double2* zd = z1d + ((f == zf0 ? 0 : 32) + c) * 2;
         d = dev::dispatch_member_z1<NCMAX>(n, a.S[f], a.L_f[f], mlab, cols + a.off_f[f], Yf, T, eys.get(f),
                                            a.kc, &cf, zd[0], zd[1]);
@@ -468,10 +742,10 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         first = false;
       }
     }
-    const bool need = valid && fail != 0;
+    const bool need = valid && part && fail != 0;
     double wi = a.w_src[a.mem_term[m]];
     if (__popc(a.mem_par[m]) & 1) wi = -wi;
-    if (!fail) {
+    if (part && !fail) {
       acc.x = fma(wi, prod.x, acc.x);
       acc.y = fma(wi, prod.y, acc.y);
     }
@@ -488,7 +762,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       e.prod = prod;
       e.w = wi * wj;
       e.pad2 = 0.0;
-      process_pairs<NCMAX>(a, W, true, e, j, Yw, wk, accq, rflops, n_rowdiff);
+      process_pairs<NCMAX>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
       n_parent += __popc(fail & pguard);
       n_child += __popc(fail & ~pguard);
     } else if (ball) {
@@ -509,15 +783,100 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       qn += __popc(ball);
       __syncwarp();
       if (qn >= 32) {
-        process_queue<NCMAX>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, wk, accq, rflops, n_rowdiff);
+        process_queue<NCMAX>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
         __syncwarp();
         if (lane < qn - 32) queue[lane] = queue[32 + lane];
         __syncwarp();
         qn -= 32;
       }
     }
+  };
+  // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
+  fx::Acc tot;
+  auto flush = [&]() {
+    double re, im;
+    int e = a.fx.fexp[W] + le;
+    if (a.fx.nf == 1) {
+      re = (double)tot.rp;
+      im = (double)tot.ih;
+      e -= fx::kSplitBits;
+    } else {
+      constexpr double k29 = 536870912.0;
+      re = fma((double)(tot.rp - tot.rn), k29, (double)(tot.lp - tot.ln));
+      im = fma((double)tot.ih, k29, (double)tot.il);
+      e += 29 - 2 * fx::kSplitBits;
+    }
+    const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
+    acc.x += v.x;
+    acc.y += v.y;
+    tot = fx::Acc();
+  };
+  const int thr1 = fx::threshold(a.kc, 1, 0), thr2 = fx::threshold(a.kc, 2, 0);
+  // members four at a time (a step that they do not fill repeats the last one)
+  constexpr int kN = 4;
+  const int step = kFx && fxm ? kN : 1;
+  for (int c = 0; c < kW; c += step) {
+    bool slow[4] = {true, true, true, true};  // this lane's pair with member c + k goes through FP64
+    if (kFx && fxm) {
+      fx::Val u[kN], t[kN];
+      int at = 0;
+      for (int f = 0; f < a.F; f++) {
+        const int n = a.n_f[f], L = a.L_f[f];
+        if (n == 0) continue;
+        const int rho = a.fam_rank[(int64_t)W * a.F + f];
+        const unsigned short* lb = fl.lab + (size_t)a.yoff[f] * T + tid;
+        const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
+        fx::Val v[kN];
+        const int4* r[kN];
+#pragma unroll
+        for (int k = 0; k < kN; k++) {
+          const int m = mem0 + min(c + k, kW - 1);
+          r[k] = at == 0 ? a.fx.ws + (size_t)m * L
+                         : a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK] * L;
+        }
+        if (NCMAX >= 10 && rho == 2) {
+#pragma unroll
+          for (int k = 0; k < kN; k++) {
+            const int m = mem0 + min(c + k, kW - 1);
+            v[k] = fx_det2(n, r[k], a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK + 1] * L, lb, Yf, T);
+          }
+        } else {
+          fx_dots<kN>(n, r, lb, Yf, T, v);
+        }
+        const int low = rho * fl.low[f * T + tid], thr = rho == 2 ? thr2 : thr1;
+#pragma unroll
+        for (int k = 0; k < kN; k++) {
+          const int tk = at == 0 ? a.fx.thr[mem0 + min(c + k, kW - 1)] : thr;
+          bool ok = fx::usable(fx::magnitude(v[k]), fx::lane_threshold(tk, low));
+          u[k] = at == 0 ? v[k] : u[k];
+          t[k] = v[k];
+          slow[k] = (at > 0 && slow[k]) || !ok;
+        }
+        at++;
+      }
+#pragma unroll
+      for (int k = 0; k < kN; k++) {
+        if (c + k >= kW) slow[k] = false;
+        const bool use = c + k < kW && !slow[k];
+        const fx::Val uz{use ? u[k].re : 0, use ? u[k].im : 0};
+        if (a.fx.nf == 1) {  // kFlush values of 2^57
+          tot.rp += (uz.re + 4) >> 3;
+          tot.ih += (uz.im + 4) >> 3;
+        } else {
+          fx::mac(tot, fx::split(uz), fx::split(t[k]));
+        }
+      }
+      if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) flush();
+    }
+    // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
+#pragma unroll 1
+    for (int k = 0; k < step; k++) {
+      const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
+      if (__any_sync(0xffffffffu, p)) member64(c + k, p);
+    }
   }
-  if (qn > 0) process_queue<NCMAX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, wk, accq, rflops, n_rowdiff);
+  __syncwarp();
+  if (qn > 0) process_queue<NCMAX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
   acc.x = fma(wj, acc.x, accq.x);
   acc.y = fma(wj, acc.y, accq.y);
 
@@ -667,8 +1026,8 @@ __device__ __forceinline__ void kfac_one(const FwdArgs& a, int64_t t, int64_t n_
   }
 #define MHC_KF(N)                                                                         \
   case N:                                                                                 \
-    g = rho == 1 ? dev::kfac_block<N, N, 1>(S, L, N, arow, scol, K, a.kp)                 \
-                 : dev::kfac_block<N, N, (N >= 2 ? 2 : 1)>(S, L, N, arow, scol, K, a.kp); \
+    g = rho == 1 ? dev::kfac_block<N, N, 1>(S, L, N, arow, scol, K, a.kp, a.fx.nf > 0)    \
+                 : dev::kfac_block<N, N, (N >= 2 ? 2 : 1)>(S, L, N, arow, scol, K, a.kp, false); \
     break;
   switch (n) {
     MHC_KF(1)
@@ -729,7 +1088,7 @@ struct KGroup {
   // so that two groups sharing an 8-lane shared-memory phase use disjoint bank groups
   static constexpr int RAW = (NCMAX - 1) * (NCMAX - 1) + (NCMAX - 1);
   static constexpr int BS = RAW + ((4 - RAW % 8) + 8) % 8;
-  static constexpr int PS = NCMAX;                             // ints per block
+  static constexpr int PS = 3 * NCMAX;                         // ints per block: row order, two exponents
   static constexpr size_t smem() { return (size_t)GPW * (BS * sizeof(double2) + PS * sizeof(int)); }
 };
 
@@ -760,11 +1119,11 @@ __device__ __forceinline__ void kfac_group_one(const FwdArgs& a, int64_t t) {
   if (rho >= 3)  // one-sided update for these blocks
     gd = true;
   else if (rho == 2 && sig == 2)  // the (n-2) x (n-2) shared block, kapply's layout (kapply22)
-    gd = dev::group_kfac_block<KG::G>(S, L, n - 1, 1, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps);
+    gd = dev::group_kfac_block<KG::G>(S, L, n - 1, 1, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps, NCMAX, false);
   else if (sig == 2)
     gd = dev::group_kfac_block12<KG::G>(S, L, n, arow, scol, K, a.kp, g, gm, Bs, Ps);
   else
-    gd = dev::group_kfac_block<KG::G>(S, L, n, rho, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps);
+    gd = dev::group_kfac_block<KG::G>(S, L, n, rho, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps, NCMAX, a.fx.nf > 0);
   if (g == 0) a.kguard[t] = gd ? 1 : 0;
 }
 

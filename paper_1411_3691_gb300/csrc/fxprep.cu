@@ -1,0 +1,154 @@
+// fxprep.cu -- the fixed-point tables of the member dots (fx.cuh), rebuilt by every call: they
+// depend on the propagators and the weights.
+//
+// One launch.  Blocks [0, sum_f L_f) convert one propagator row each: the row's largest binary
+// exponent, then its entries as limbs, and the limbs of the column of the same label at the
+// column's exponent.  The other blocks take one source family each: a member's first row
+// of the first flavour, times the member's signed weight, is stored at the family's common
+// exponent, so that the member loop sums products of all members in integers.  A member whose
+// weighted rows lie more than kMaxAlign binades below the family's largest, or whose rows or
+// weight are not finite, or zero, is left to the FP64 path.  The work is a pass over 2 F L^2 +
+// members L entries (He-4 shapes: 206 000, 3.3 MB written).
+#include "kernels.cuh"
+
+namespace mhc {
+
+namespace {
+
+constexpr int kThreads = 128;
+
+// exponent above every entry of a row or column (largest binary exponent + 1); one warp
+__device__ __forceinline__ int row_exponent(const dev::cd* row, int pitch, int L, int lane) {
+  int e = -4096;
+  for (int l = lane; l < L; l += 32) e = max(e, dev::expo(dev::ldS(row + (size_t)l * pitch)));
+  return __reduce_max_sync(0xffffffffu, e) + 1;
+}
+
+// row b and column b of flavour f
+__device__ void prep_row(const FwdArgs& a, int f, int b) {
+  const int L = a.L_f[f], lane = threadIdx.x & 31;
+  const dev::cd* row = a.S[f] + (size_t)b * L;
+  const int e = row_exponent(row, 1, L, lane);  // every warp for itself: no barrier
+  const int ec = row_exponent(a.S[f] + b, L, L, lane);
+  if (threadIdx.x == 0) const_cast<int*>(a.fx.cexp[f])[b] = ec;
+  int4* out = const_cast<int4*>(a.fx.s[f]) + (size_t)b * L;
+  int4* outc = const_cast<int4*>(a.fx.sc[f]) + b;
+  for (int l = threadIdx.x; l < L; l += kThreads) {
+    out[l] = e <= 1023 ? fx::quant(dev::ldS(row + l), e, fx::kRowBits) : make_int4(0, 0, 0, 0);
+    outc[(size_t)l * L] = ec <= 1023 ? fx::quant(dev::ldS(a.S[f] + (size_t)l * L + b), ec, fx::kABits) : make_int4(0, 0, 0, 0);
+  }
+}
+
+__device__ void prep_family(const FwdArgs& a, int W) {
+  __shared__ int e0s[64], rest[64];
+  __shared__ double ws[64];
+  const int f0 = a.fx.f0, L0 = a.L_f[f0];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int mem0 = a.fam_info[4 * W], kW = a.fam_info[4 * W + 1];  // kW <= 64
+  // per member: the exponent above w times its first row, and the sum of its other rows' ones
+  for (int c = warp; c < kW; c += kThreads / 32) {
+    const int m = mem0 + c;
+    double w = a.w_src[a.mem_term[m]];
+    if (__popc(a.mem_par[m]) & 1) w = -w;
+    const int32_t* lab = a.mem_lab + (int64_t)m * a.F * MHC_MAX_RANK;
+    int r = 0, e0 = -4096;
+    bool bad = w == 0.0 || dev::expo(w) >= 1024;
+    for (int f = 0; f < a.F; f++) {
+      if (a.n_f[f] == 0) continue;
+      for (int t = 0; t < a.fam_rank[(int64_t)W * a.F + f]; t++) {
+        const dev::cd* row = a.S[f] + (size_t)lab[f * MHC_MAX_RANK + t] * a.L_f[f];
+        const int e = row_exponent(row, 1, a.L_f[f], lane);
+        bad |= e > 1023 || e < -1000;
+        if (f == f0 && t == 0) {
+          for (int l = lane; l < L0; l += 32) {
+            const dev::cd z = dev::ldS(row + l);
+            e0 = max(e0, dev::expo(make_double2(w * z.x, w * z.y)));
+          }
+          e0 = __reduce_max_sync(0xffffffffu, e0) + 1;
+          bad |= e0 > 1023 || e0 < -1000;
+        } else {
+          r += e;
+        }
+      }
+    }
+    if (lane == 0) {
+      ws[c] = w;
+      e0s[c] = bad ? -100000 : e0;
+      rest[c] = r;
+    }
+  }
+  __syncthreads();
+  int X = -100000;
+  for (int c = 0; c < kW; c++)
+    if (e0s[c] > -100000) X = max(X, e0s[c] + rest[c]);
+  if (threadIdx.x == 0) const_cast<int*>(a.fx.fexp)[W] = X;
+  for (int c = warp; c < kW; c += kThreads / 32) {
+    const int m = mem0 + c;
+    const bool bad = e0s[c] == -100000;
+    const int d = X - e0s[c] - rest[c];  // binades below the family's largest member
+    const bool skip = bad || d > fx::kMaxAlign;
+    if (lane == 0)
+      const_cast<int*>(a.fx.thr)[m] = skip ? fx::kNever : fx::threshold(a.kc, a.fam_rank[(int64_t)W * a.F + f0], d);
+    const int32_t lab = a.mem_lab[((int64_t)m * a.F + f0) * MHC_MAX_RANK];
+    const dev::cd* row = a.S[f0] + (size_t)lab * L0;
+    int4* out = const_cast<int4*>(a.fx.ws) + (size_t)m * L0;
+    const int e = X - rest[c];
+    for (int l = lane; l < L0; l += 32) {
+      dev::cd z = make_double2(0.0, 0.0);
+      if (!skip) {
+        z = dev::ldS(row + l);
+        z = make_double2(ws[c] * z.x, ws[c] * z.y);
+      }
+      out[l] = fx::quant(z, e, fx::kRowBits);
+    }
+  }
+}
+
+__device__ void prep_block(const FwdArgs& a, int64_t b) {
+  if (a.fx.nf == 0) return;
+  for (int f = 0; f < a.F; f++) {
+    if (a.n_f[f] == 0) continue;
+    if (b < a.L_f[f]) {
+      prep_row(a, f, (int)b);
+      return;
+    }
+    b -= a.L_f[f];
+  }
+  if (b < a.n_fam) prep_family(a, (int)b);
+}
+
+__global__ void __launch_bounds__(kThreads) fxprep_kernel(const FwdArgs a) { prep_block(a, blockIdx.x); }
+
+__global__ void __launch_bounds__(kThreads) fxprep_batch_kernel(const FwdArgs* __restrict__ desc,
+                                                                const int64_t* __restrict__ pref, int count) {
+  int lo = 0, hi = count - 1;
+  while (lo < hi) {  // last k with pref[k] <= block
+    const int mid = (lo + hi + 1) >> 1;
+    if (pref[mid] <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  prep_block(desc[lo], (int64_t)blockIdx.x - pref[lo]);
+}
+
+}  // namespace
+
+int64_t fxprep_blocks(const FwdArgs& a) {
+  if (a.fx.nf == 0) return 0;
+  int64_t n = a.n_fam;
+  for (int f = 0; f < a.F; f++) n += a.n_f[f] > 0 ? a.L_f[f] : 0;
+  return n;
+}
+
+cudaError_t launch_fxprep(const FwdArgs& a, cudaStream_t s) {
+  const int64_t n = fxprep_blocks(a);
+  if (n == 0) return cudaSuccess;
+  fxprep_kernel<<<(unsigned)n, kThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fxprep_batch(const FwdArgs* desc, const int64_t* pref, int count, int64_t total, cudaStream_t s) {
+  if (total == 0) return cudaSuccess;
+  fxprep_batch_kernel<<<(unsigned)total, kThreads, 0, s>>>(desc, pref, count);
+  return cudaGetLastError();
+}
+
+}  // namespace mhc

@@ -9,6 +9,7 @@
 
 #include "../../include/mhc.h"
 #include "device.cuh"
+#include "fx.cuh"
 #include "layout.h"
 
 namespace mhc {
@@ -38,6 +39,8 @@ struct FwdArgs {
   const double* w_src;
   const double* w_snk;
   double2* partials;         // [items]
+  double2* reduce_blocks;    // reduce_kernel's sums per block, and its counter (0 between calls)
+  unsigned* reduce_done;
   unsigned long long* counters;
   // two-sided update; snk_orig == nullptr selects the one-sided update with the sinks
   // in their own order and labels from snk_lab
@@ -62,6 +65,8 @@ struct FwdArgs {
   int64_t item0;             // first work item of the launch
   int n_ranges;
   FwdRange ranges[kMaxFwdRanges];
+  int64_t n_fam;
+  fx::Tables fx;             // fixed-point rows of the member dots (fx.nf = 0: FP64 dots)
 };
 
 namespace dev {
@@ -318,29 +323,39 @@ struct BatchItem {
   int32_t corr, W, tile, pad;
 };
 
-// per-warp refactor queue of the forward kernel
+// Per-warp scratch of the forward kernel, by n class: the refactor queue; a store of the members'
+// dots with a block's first null vector (rank-2 families against one-column sink families: two
+// flavours, 32 members, two complex values); the multipliers of a grouped refactor's shared
+// elimination by step, packed (n - 1 + n - 2 + ... + 1 complex values for n <= 18).  Before the
+// member loop the whole of it holds the block factors of the warp's sinks (fwd::fx_stage).
 constexpr int kQueueCap = 64;         // entries per warp
 constexpr int kQueueEntryBytes = 48;  // sizeof(fwd::QEntry)
-// per-warp store of the members' dots with a block's first null vector (rank-2 families
-// against one-column sink families): two flavours, 32 members, two complex values
 constexpr int kZ1Flavours = 2;
-constexpr int kZ1Bytes = kZ1Flavours * 32 * 2 * 16;
-// per-warp scratch of the grouped refactors: the multipliers of the shared elimination by
-// step, packed (n - 1 + n - 2 + ... + 1 complex values for n <= 18)
-constexpr int kWalkMaxN = 18;
-constexpr int kWalkBytes = kWalkMaxN * (kWalkMaxN - 1) / 2 * 16;
+template <int NCMAX>
+struct WarpScratch {
+  static constexpr int kWalkMaxN = NCMAX <= 8 ? 8 : 18;
+  static constexpr int kQueue = kQueueCap * kQueueEntryBytes;
+  static constexpr int kZ1 = NCMAX <= 8 ? 0 : kZ1Flavours * 32 * 2 * 16;
+  static constexpr int kWalk = kWalkMaxN * (kWalkMaxN - 1) / 2 * 16;
+  static constexpr int kBytes = kQueue + kZ1 + kWalk;
+};
 
-// host-side launchers (forward.cu and fwd_nc*.cu)
+constexpr int kReduceMaxBlocks = 128;
+
+// host-side launchers (forward.cu, fxprep.cu and fwd_nc*.cu)
+cudaError_t launch_fxprep(const FwdArgs& a, cudaStream_t s);
+cudaError_t launch_fxprep_batch(const FwdArgs* desc, const int64_t* pref, int count, int64_t total, cudaStream_t s);
+int64_t fxprep_blocks(const FwdArgs& a);
 cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
                            size_t smem, double* out, cudaStream_t s);
-cudaError_t launch_reduce(const double2* partials, int64_t items, double* out, cudaStream_t s);
+cudaError_t launch_reduce(const FwdArgs& a, int64_t items, double* out, cudaStream_t s);
 cudaError_t launch_forward_cw(const FwdArgs& a0, const double* const* ws, const double* const* wk,
                               int ncmax, int tile, int64_t n_fam, int64_t items, size_t smem, double* tmp,
                               double* out, cudaStream_t s);
 cudaError_t launch_pairs(const FwdArgs& a, int ncmax, int64_t n_pairs, int64_t n_src,
                          const int64_t* ii, const int64_t* jj, const int32_t* src_member,
                          const int32_t* mem_family, double* dets, int32_t* path, cudaStream_t s);
-size_t forward_smem_bytes(int slots, int tile);
+size_t forward_smem_bytes(int slots, int tile, int ncmax);
 #define MHC_DECL_NC(NC)                                                                       \
   cudaError_t launch_fwd_nc##NC(const FwdArgs& a, int tile, int64_t items, size_t smem,       \
                                 cudaStream_t s);                                              \

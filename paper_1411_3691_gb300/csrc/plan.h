@@ -62,6 +62,9 @@ struct DevicePlan {
   size_t kinv_bytes = 0;
   int kstride = 0;
   bool two_sided = false;
+  // fixed-point tables of the member dots (fx::Tables): one allocation, or null
+  char* fx = nullptr;
+  double* reduce = nullptr;      // reduce_kernel's block sums and counter
   double* w_src = nullptr;       // [n_src] plan weights
   double* w_snk = nullptr;       // [n_snk]
   double* partials = nullptr;    // [items][2] per-work-item partial sums

@@ -46,7 +46,7 @@ void free_device(DevicePlan& d) {
                   d.snk_lab, d.src_member, d.mem_family, d.w_src, d.w_snk, d.partials,
                   d.counters, d.bwd_rows, d.bwd_wsrc, d.bwd_wsnk, d.snk_order, d.snk_lab2,
                   d.snk_par2, d.snk_q, d.q_off, d.q_two, d.q_rank, d.kbuf, d.kguard, d.kinv, d.bwd_stage,
-                  d.bwd_accs, d.bwd_r2, d.bwd_dets, d.cw_tmp};
+                  d.bwd_accs, d.bwd_r2, d.bwd_dets, d.cw_tmp, d.fx, d.reduce};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (auto& bi : d.bwd_index) {
@@ -89,6 +89,45 @@ void plan_slots(const Plan& p, int* yoff, int* total) {
   }
   *total = std::max(s, 1);
 }
+
+// Layout of a plan's fixed-point tables from `base` (null: sizes only); returns the bytes.  The
+// member dots take the fixed-point path for one or two flavours (n_f > 0): with more, the
+// products' common scale would cost accuracy (about two binades each).  n_f <= 18 keeps the
+// solves' 64-bit sums in range (2 (n - 1) cross terms of 2^57).
+size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off += (bytes + 255) & ~(size_t)255;
+    return base + o;
+  };
+  *t = fx::Tables();
+  t->f0 = -1;
+  for (int f = 0; f < p.F; f++) {
+    if (p.n_f[f] == 0) continue;
+    if (t->f0 < 0) t->f0 = f;
+    t->nf++;
+    t->s[f] = reinterpret_cast<const int4*>(take((size_t)p.L_f[f] * p.L_f[f] * sizeof(int4)));
+    t->sc[f] = reinterpret_cast<const int4*>(take((size_t)p.L_f[f] * p.L_f[f] * sizeof(int4)));
+    t->cexp[f] = reinterpret_cast<const int*>(take((size_t)p.L_f[f] * sizeof(int)));
+  }
+  if (t->nf < 1 || t->nf > 2 || p.max_n > 18) {
+    *t = fx::Tables();
+    return 0;
+  }
+  t->ws = reinterpret_cast<const int4*>(take((size_t)p.n_src * p.L_f[t->f0] * sizeof(int4)));
+  t->thr = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
+  t->fexp = reinterpret_cast<const int*>(take((size_t)p.n_fam * sizeof(int)));
+  return off;
+}
+
+// The weighted member rows are members x L entries: above this size the FP64 dots are kept.
+constexpr size_t kMaxFxBytes = (size_t)4 << 30;
+// Below two waves of the n <= 8 kernel's twelve warps per SM a call is a chain of latencies: the
+// tables' launch and the longer code cost more than the FP64 pipe (512 x 512 terms of n = 3, 1824
+// warps: 66 us with the tables, 56 us without; 1291 x 977 of n = 5, 4 in ragged families, 7200
+// warps: 160 us against 203 us).
+constexpr int64_t kMinFxWarps = 2 * 12 * 152;
 
 mhc_status ensure_device(Plan& p) {
   int cur = 0;
@@ -188,6 +227,16 @@ mhc_status ensure_device(Plan& p) {
     if ((st = upload<int32_t>(&d.kguard, nullptr, (size_t)p.n_fam * p.n_qfam * p.F)) != MHC_OK) return st;
     d.kstride = (int)kstride;
   }
+  {
+    fx::Tables t;
+    const size_t bytes = p.n_fam * ((p.n_snk + 31) / 32) >= kMinFxWarps ? fx_layout(p, nullptr, &t) : 0;
+    if (bytes > 0 && bytes <= kMaxFxBytes && cudaMalloc(&d.fx, bytes) != cudaSuccess) {
+      d.fx = nullptr;  // the FP64 dots need no tables
+      cudaGetLastError();
+    }
+  }
+  if ((st = upload<double>(&d.reduce, nullptr, 2 * kReduceMaxBlocks + 2)) != MHC_OK) return st;
+  MHC_CUDA(cudaMemset(d.reduce, 0, (2 * kReduceMaxBlocks + 2) * sizeof(double)));
   d.tile = plan_tile(p);
   d.n_tiles = (int32_t)((p.n_snk + d.tile - 1) / d.tile);
   d.n_items = p.n_fam * d.n_tiles;
@@ -234,6 +283,10 @@ mhc_status fill_fwd_args(Plan& p, const double* const* S_f, const double* w_src,
   a.fam_order = p.dev.fam_order;
   a.n_ranges = p.dev.fam_order ? p.dev.n_ranges : 0;
   for (int r = 0; r < a.n_ranges; r++) a.ranges[r] = p.dev.ranges[r];
+  a.n_fam = p.n_fam;
+  if (p.dev.fx) fx_layout(p, p.dev.fx, &a.fx);
+  a.reduce_blocks = reinterpret_cast<double2*>(p.dev.reduce);
+  a.reduce_done = reinterpret_cast<unsigned*>(p.dev.reduce + 2 * kReduceMaxBlocks);
   if (p.dev.two_sided) {
     a.snk_pos = p.dev.snk_lab2;
     a.snk_orig = p.dev.snk_order;
@@ -291,7 +344,7 @@ mhc_status mhc_correlator(mhc_plan_t plan, const double* const* S_f, const doubl
   FwdArgs a;
   if ((st = fill_fwd_args(p, S_f, w_src_dev, w_snk_dev, a)) != MHC_OK) return st;
   const int tile = p.dev.tile;
-  const size_t smem = forward_smem_bytes(a.slots, tile);
+  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p));
   MHC_CUDA(launch_forward(a, plan_ncmax(p), tile, p.n_fam, p.dev.n_items, smem, out_dev,
                           reinterpret_cast<cudaStream_t>(stream)));
   return MHC_OK;
@@ -316,7 +369,7 @@ mhc_status mhc_correlator_cw(mhc_plan_t plan, const double* const* S_f, const do
   const double* ws[2] = {w_src_re, w_src_im};
   const double* wk[2] = {w_snk_re, w_snk_im};
   const int tile = p.dev.tile;
-  const size_t smem = forward_smem_bytes(a.slots, tile);
+  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p));
   MHC_CUDA(launch_forward_cw(a, ws, wk, plan_ncmax(p), tile, p.n_fam, p.dev.n_items, smem, p.dev.cw_tmp,
                              out_dev, reinterpret_cast<cudaStream_t>(stream)));
   return MHC_OK;

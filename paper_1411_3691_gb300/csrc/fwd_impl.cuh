@@ -921,7 +921,11 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) 
   fwd_item<NCMAX>(a, W, (int)(item % a.n_tiles), smem, &a.partials[item]);
 }
 
-// Per-pair determinants through the same update path (one thread per pair).
+// Flavours of a pair that pair_group_kernel takes: blocks that do not fit in a thread's registers.
+__device__ __forceinline__ bool pair_grouped(int n, int rho) { return n > 6 && rho <= 2; }
+
+// Per-pair determinants through the same update path (one thread per pair): the flavours with
+// n <= 6 or more than two changed rows.
 template <int NCMAX>
 __global__ void __launch_bounds__(64) pair_kernel(const FwdArgs a, int64_t n_pairs, int64_t n_src,
                                                   const int64_t* __restrict__ ii,
@@ -945,6 +949,7 @@ __global__ void __launch_bounds__(64) pair_kernel(const FwdArgs a, int64_t n_pai
   int32_t bits = 0;
   for (int f = 0; f < a.F; f++) {
     const int n = a.n_f[f];
+    if (pair_grouped(n, a.fam_rank[(int64_t)W * a.F + f])) continue;
     double2 d = make_double2(1.0, 0.0);
     if (n > 0) {
       const int rho = a.fam_rank[(int64_t)W * a.F + f];
@@ -1091,6 +1096,147 @@ struct KGroup {
   static constexpr int PS = 3 * NCMAX;                         // ints per block: row order, two exponents
   static constexpr size_t smem() { return (size_t)GPW * (BS * sizeof(double2) + PS * sizeof(int)); }
 };
+
+// Per-pair determinants of the other flavours: G lanes per (pair, flavour), the shared rows in shared
+// memory (group_lu), the null vectors by a back substitution over the lanes, the member's dots and a
+// guarded pair's fresh factorisation likewise.  A thread's own (n - 1) x n matrix lived in local
+// memory: 100 000 pairs of n = 18 took 26.4 ms; here 5.4 ms, of which the factorisations' FP64 work is
+// 2.5 ms.
+template <int NCMAX>
+struct PairGroup {
+  static constexpr int G = KGroup<NCMAX>::G, GPW = KGroup<NCMAX>::GPW;
+  static constexpr int RAW = NCMAX * (NCMAX | 1) + 2 * NCMAX + 1;
+  static constexpr int BS = RAW + ((4 - RAW % 8) + 8) % 8;  // as KGroup
+  static constexpr size_t smem() { return (size_t)GPW * (BS * sizeof(double2) + NCMAX * sizeof(int)); }
+};
+template <int NCMAX>
+__global__ void __launch_bounds__(32) pair_group_kernel(const FwdArgs a, int64_t n_pairs, int64_t n_src,
+                                                        const int64_t* __restrict__ ii,
+                                                        const int64_t* __restrict__ jj,
+                                                        const int32_t* __restrict__ src_member,
+                                                        const int32_t* __restrict__ mem_family,
+                                                        double2* __restrict__ dets, int32_t* path) {
+  using PG = PairGroup<NCMAX>;
+  constexpr int G = PG::G;
+  extern __shared__ double2 smem[];
+  const int lane = threadIdx.x, grp = lane / G, g = lane % G;
+  const unsigned gm = ((1u << G) - 1u) << (grp * G);
+  const int64_t u = (int64_t)blockIdx.x * PG::GPW + grp;
+  const int f = (int)(u / n_pairs);  // the flavour varies slowest
+  if (f >= a.F) return;
+  const int64_t p = u % n_pairs, i = ii[p], j = jj[p];
+  if (i < 0 || i >= n_src || j < 0 || j >= a.n_snk) return;  // reported by pair_kernel
+  const int m = src_member[i], W = mem_family[m];
+  const int n = a.n_f[f], rho = a.fam_rank[(int64_t)W * a.F + f], M = n - rho;
+  if (!pair_grouped(n, rho)) return;
+  dev::cd* B = smem + (size_t)grp * PG::BS;
+  dev::cd* Y = B + NCMAX * (NCMAX | 1);
+  int* perm = reinterpret_cast<int*>(smem + (size_t)PG::GPW * PG::BS) + grp * NCMAX;
+  const int L = a.L_f[f], P = n | 1;
+  const dev::cd* S = a.S[f];
+  const int32_t* arow = a.fam_arow + (int64_t)W * a.Tn + a.off_f[f];
+  const int32_t* col = a.snk_lab + j * a.Tn + a.off_f[f];
+  const int32_t* mlab = a.mem_lab + ((int64_t)m * a.F + f) * MHC_MAX_RANK;
+  auto load = [&](int rows) {  // the shared rows, then the member's
+    for (int e = g; e < rows * n; e += G) {
+      const int r = e / n, q = e - r * n;
+      B[r * P + q] = dev::ldS(S + (size_t)(r < M ? arow[r] : mlab[r - M]) * L + col[q]);
+    }
+    __syncwarp(gm);
+  };
+  auto sum = [&](dev::cd v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+      v.x += __shfl_xor_sync(gm, v.x, o);
+      v.y += __shfl_xor_sync(gm, v.y, o);
+    }
+    return v;
+  };
+  auto most = [&](int v) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) v = max(v, __shfl_xor_sync(gm, v, o));
+    return v;
+  };
+  load(M);
+  dev::cd det, d = make_double2(0.0, 0.0);
+  int parity, bits = 0;
+  bool fail = dev::group_lu<G>(B, P, perm, M, n, M, g, gm, a.kp, &det, &parity);
+  if (!fail) {
+    const dev::cd sd = parity ? dev::cneg(det) : det;
+    // null vectors z_t = [-U1^{-1} u_t ; e_t] (Y + t n); rank 1: y = sd z; rank 2: sd at Y + 2 n
+    for (int t = 0; t < rho; t++) {
+      dev::cd* z = Y + t * n;
+      for (int k = M - 1; k >= 0; k--) {
+        dev::cd s = make_double2(0.0, 0.0);
+        for (int q = k + 1 + g; q < M; q += G) s = dev::cfma(B[k * P + q], z[q], s);
+        s = sum(s);
+        if (g == 0) z[k] = dev::cmul(dev::cadd(s, B[k * P + M + t]), dev::cneg(B[k * P + k]));
+        __syncwarp(gm);
+      }
+      for (int v = g; v < rho; v += G) z[M + v] = make_double2(v == t ? 1.0 : 0.0, 0.0);
+      __syncwarp(gm);
+      if (rho == 1)
+        for (int q = g; q < n; q += G) z[q] = dev::cmul(sd, z[q]);
+    }
+    if (rho == 2 && g == 0) Y[2 * n] = sd;
+    __syncwarp(gm);
+    int ez = rho == 1 ? -4096 : 0, e1 = -4096, e2 = -4096;
+    for (int q = g; q < rho * n; q += G) ez = max(ez, dev::expo(Y[q]));
+    ez = most(ez);
+    const int ey = rho == 1 ? ez : dev::expo(sd) + 2 * ez;
+    if (rho == 1) {
+      for (int q = g; q < n; q += G) {
+        const dev::cd b = dev::ldS(S + (size_t)mlab[0] * L + col[q]);
+        e1 = max(e1, dev::expo(b));
+        d = dev::cfma(b, Y[q], d);
+      }
+      d = sum(d);
+      e2 = 0;
+    } else {
+      dev::cd d11 = d, d12 = d, d21 = d, d22 = d;
+      for (int q = g; q < n; q += G) {
+        const dev::cd b1 = dev::ldS(S + (size_t)mlab[0] * L + col[q]), b2 = dev::ldS(S + (size_t)mlab[1] * L + col[q]);
+        e1 = max(e1, dev::expo(b1));
+        e2 = max(e2, dev::expo(b2));
+        d11 = dev::cfma(b1, Y[q], d11);
+        d12 = dev::cfma(b1, Y[n + q], d12);
+        d21 = dev::cfma(b2, Y[q], d21);
+        d22 = dev::cfma(b2, Y[n + q], d22);
+      }
+      d11 = sum(d11);
+      d12 = sum(d12);
+      d21 = sum(d21);
+      d22 = sum(d22);
+      d = dev::cmul(sd, dev::cfms(d12, d21, dev::cmul(d11, d22)));
+      e2 = most(e2);
+    }
+    fail = dev::expo(d) < most(e1) + e2 + ey - a.kc;
+    if (fail && a.rowdiff) {  // one lane; the others take its result
+      bool f2 = true;
+      dev::cd d2 = d;
+      if (g == 0)
+        d2 = rho == 1 ? dev::rowdiff_det(S, L, n, mlab[0], arow, col, Y, 1, ey, a.kc, &f2)
+                      : dev::rowdiff2_det(S, L, n, mlab, arow, col, Y, 1, ey, a.kc, &f2);
+      f2 = __shfl_sync(gm, (int)f2, grp * G);
+      if (!f2) {
+        d = make_double2(__shfl_sync(gm, d2.x, grp * G), __shfl_sync(gm, d2.y, grp * G));
+        fail = false;
+        bits = 1 << (8 + f);
+      }
+    }
+  }
+  if (fail) {
+    __syncwarp(gm);
+    load(n);
+    const bool zero = dev::group_lu<G>(B, P, perm, n, n, n, g, gm, 1 << 20, &det, &parity);
+    d = zero ? make_double2(0.0, 0.0) : parity ? dev::cneg(det) : det;
+    bits = 1 << f;
+  }
+  if (g == 0) {
+    dets[p * a.F + f] = (a.mem_par[m] >> f) & 1 ? dev::cneg(d) : d;
+    if (path && bits) atomicOr(&path[p], bits);
+  }
+}
 
 template <int NCMAX>
 __device__ __forceinline__ void kfac_group_one(const FwdArgs& a, int64_t t) {
@@ -1249,6 +1395,18 @@ cudaError_t launch_pairs_nc(const FwdArgs& a, int64_t n_pairs, int64_t n_src, co
   const unsigned grid = (unsigned)((n_pairs + T - 1) / T);
   fwd::pair_kernel<NCMAX><<<grid, T, smem, s>>>(a, n_pairs, n_src, ii, jj, src_member, mem_family,
                                                 reinterpret_cast<double2*>(dets), path);
+  bool big = false;
+  for (int f = 0; f < a.F; f++) big |= a.n_f[f] > 6;
+  if (big) {  // after pair_kernel, which writes every pair's path word
+    using PG = fwd::PairGroup<NCMAX>;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(fwd::pair_group_kernel<NCMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)PG::smem())) != cudaSuccess)
+      return e;
+    const int64_t units = n_pairs * a.F;
+    fwd::pair_group_kernel<NCMAX><<<(unsigned)((units + PG::GPW - 1) / PG::GPW), 32, PG::smem(), s>>>(
+        a, n_pairs, n_src, ii, jj, src_member, mem_family, reinterpret_cast<double2*>(dets), path);
+  }
   return cudaGetLastError();
 }
 

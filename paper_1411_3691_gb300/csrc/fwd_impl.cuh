@@ -27,8 +27,7 @@ struct QEntry {
   int32_t fail;    // flavours to refactor (bit f)
   int32_t pguard;  // of those, the flavours whose shared rows failed the pivot guard
   double2 prod;    // product of the flavours that did not fail
-  double w;        // signed w_i w_j of the pair
-  double pad2;
+  double2 w;       // signed w_i w_j of the pair
 };
 
 // Algorithmic flops of the refactor path, counted with the planner's rule (real add/mul 1,
@@ -356,10 +355,7 @@ __device__ __noinline__ void process_pairs(const FwdArgs& a, int W, bool have, c
       rflops += fresh_flops(n);
     }
   }
-  if (have) {
-    acc.x = fma(e.w, prod.x, acc.x);
-    acc.y = fma(e.w, prod.y, acc.y);
-  }
+  if (have) acc = dev::add_weighted(a, e.w, prod, acc);
 }
 
 // Refactor the first count queued pairs (one per lane).  Called by the whole warp.
@@ -697,8 +693,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   }
 
   // ---- per member: one dot product per flavour --------------------------------------
-  double wj = valid ? a.w_snk[a.snk_orig ? a.snk_orig[j] : j] : 0.0;
-  if (a.snk_orig && (__popc(a.snk_par[j]) & 1)) wj = -wj;
+  const double2 wj = valid ? dev::sink_weight(a, j) : make_double2(0.0, 0.0);
   // acc: sum over the members of w_i prod_f det (this lane's sink; times w_j once, at the
   // end); accq: the refactored pairs, w_i w_j included (a queue lane holds other sinks' pairs)
   double2 acc = make_double2(0.0, 0.0), accq = make_double2(0.0, 0.0);
@@ -743,12 +738,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       }
     }
     const bool need = valid && part && fail != 0;
-    double wi = a.w_src[a.mem_term[m]];
-    if (__popc(a.mem_par[m]) & 1) wi = -wi;
-    if (part && !fail) {
-      acc.x = fma(wi, prod.x, acc.x);
-      acc.y = fma(wi, prod.y, acc.y);
-    }
+    const double2 wi = dev::source_weight(a, m);
+    if (part && !fail) acc = dev::add_weighted(a, wi, prod, acc);
     const unsigned ball = __ballot_sync(0xffffffffu, need);
     if (ball == 0xffffffffu) {
       // every lane refactors this member (a member near-singular against its family): the
@@ -760,8 +751,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       e.fail = (int32_t)fail;
       e.pguard = (int32_t)pguard;
       e.prod = prod;
-      e.w = wi * wj;
-      e.pad2 = 0.0;
+      e.w = dev::add_weighted(a, wi, wj, make_double2(0.0, 0.0));
       process_pairs<NCMAX>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
       n_parent += __popc(fail & pguard);
       n_child += __popc(fail & ~pguard);
@@ -774,8 +764,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         e.fail = (int32_t)fail;
         e.pguard = (int32_t)pguard;
         e.prod = prod;
-        e.w = wi * wj;
-        e.pad2 = 0.0;
+        e.w = dev::add_weighted(a, wi, wj, make_double2(0.0, 0.0));
         queue[pos] = e;
         n_parent += __popc(fail & pguard);
         n_child += __popc(fail & ~pguard);
@@ -877,8 +866,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   }
   __syncwarp();
   if (qn > 0) process_queue<NCMAX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
-  acc.x = fma(wj, acc.x, accq.x);
-  acc.y = fma(wj, acc.y, accq.y);
+  acc = dev::add_weighted(a, wj, acc, accq);
 
   // ---- fixed-order reduction: lanes, then warps --------------------------------------
   acc = dev::warp_sum(acc);

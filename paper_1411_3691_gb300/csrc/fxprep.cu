@@ -39,20 +39,23 @@ __device__ void prep_row(const FwdArgs& a, int f, int b) {
   }
 }
 
+__device__ __forceinline__ dev::cd weighted(const FwdArgs& a, dev::cd w, dev::cd z) {
+  return a.w_src_im ? dev::cmul(w, z) : make_double2(w.x * z.x, w.x * z.y);
+}
+
 __device__ void prep_family(const FwdArgs& a, int W) {
   __shared__ int e0s[64], rest[64];
-  __shared__ double ws[64];
+  __shared__ dev::cd ws[64];
   const int f0 = a.fx.f0, L0 = a.L_f[f0];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int mem0 = a.fam_info[4 * W], kW = a.fam_info[4 * W + 1];  // kW <= 64
   // per member: the exponent above w times its first row, and the sum of its other rows' ones
   for (int c = warp; c < kW; c += kThreads / 32) {
     const int m = mem0 + c;
-    double w = a.w_src[a.mem_term[m]];
-    if (__popc(a.mem_par[m]) & 1) w = -w;
+    const dev::cd w = dev::source_weight(a, m);
     const int32_t* lab = a.mem_lab + (int64_t)m * a.F * MHC_MAX_RANK;
     int r = 0, e0 = -4096;
-    bool bad = w == 0.0 || dev::expo(w) >= 1024;
+    bool bad = (w.x == 0.0 && w.y == 0.0) || dev::expo(w) >= 1024;
     for (int f = 0; f < a.F; f++) {
       if (a.n_f[f] == 0) continue;
       for (int t = 0; t < a.fam_rank[(int64_t)W * a.F + f]; t++) {
@@ -61,8 +64,7 @@ __device__ void prep_family(const FwdArgs& a, int W) {
         bad |= e > 1023 || e < -1000;
         if (f == f0 && t == 0) {
           for (int l = lane; l < L0; l += 32) {
-            const dev::cd z = dev::ldS(row + l);
-            e0 = max(e0, dev::expo(make_double2(w * z.x, w * z.y)));
+            e0 = max(e0, dev::expo(weighted(a, w, dev::ldS(row + l))));
           }
           e0 = __reduce_max_sync(0xffffffffu, e0) + 1;
           bad |= e0 > 1023 || e0 < -1000;
@@ -95,10 +97,7 @@ __device__ void prep_family(const FwdArgs& a, int W) {
     const int e = X - rest[c];
     for (int l = lane; l < L0; l += 32) {
       dev::cd z = make_double2(0.0, 0.0);
-      if (!skip) {
-        z = dev::ldS(row + l);
-        z = make_double2(ws[c] * z.x, ws[c] * z.y);
-      }
+      if (!skip) z = weighted(a, ws[c], dev::ldS(row + l));
       out[l] = fx::quant(z, e, fx::kRowBits);
     }
   }

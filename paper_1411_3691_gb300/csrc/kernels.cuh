@@ -38,6 +38,8 @@ struct FwdArgs {
   const int32_t* snk_lab;    // [n_snk][Tn]
   const double* w_src;
   const double* w_snk;
+  const double* w_src_im;    // imaginary parts of complex weights, both or neither null
+  const double* w_snk_im;
   double2* partials;         // [items]
   double2* reduce_blocks;    // reduce_kernel's sums per block, and its counter (0 between calls)
   unsigned* reduce_done;
@@ -267,6 +269,22 @@ __device__ __forceinline__ const int32_t* sink_cols(const FwdArgs& a, int64_t j)
   return (a.snk_orig ? a.snk_pos : a.snk_lab) + j * a.Tn;
 }
 
+// weight of member m with its sign, and of the sink at position j
+__device__ __forceinline__ cd source_weight(const FwdArgs& a, int m) {
+  const int i = a.mem_term[m];
+  const cd w = make_double2(a.w_src[i], a.w_src_im ? a.w_src_im[i] : 0.0);
+  return __popc(a.mem_par[m]) & 1 ? cneg(w) : w;
+}
+__device__ __forceinline__ cd sink_weight(const FwdArgs& a, int64_t j) {
+  const int64_t i = a.snk_orig ? a.snk_orig[j] : j;
+  const cd w = make_double2(a.w_snk[i], a.w_snk_im ? a.w_snk_im[i] : 0.0);
+  return a.snk_orig && (__popc(a.snk_par[j]) & 1) ? cneg(w) : w;
+}
+// acc + w z, w real unless the call's weights are complex
+__device__ __forceinline__ cd add_weighted(const FwdArgs& a, cd w, cd z, cd acc) {
+  return a.w_src_im ? cfma(w, z, acc) : make_double2(fma(w.x, z.x, acc.x), fma(w.x, z.y, acc.y));
+}
+
 // Rows of member m in flavour f for a fresh factorisation: the shared rows, then the
 // member's labels at the changed rows (the same order as the cached path).
 __device__ __forceinline__ void member_rows(const FwdArgs& a, int W, int m, int f, int rho,
@@ -349,9 +367,6 @@ int64_t fxprep_blocks(const FwdArgs& a);
 cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
                            size_t smem, double* out, cudaStream_t s);
 cudaError_t launch_reduce(const FwdArgs& a, int64_t items, double* out, cudaStream_t s);
-cudaError_t launch_forward_cw(const FwdArgs& a0, const double* const* ws, const double* const* wk,
-                              int ncmax, int tile, int64_t n_fam, int64_t items, size_t smem, double* tmp,
-                              double* out, cudaStream_t s);
 cudaError_t launch_pairs(const FwdArgs& a, int ncmax, int64_t n_pairs, int64_t n_src,
                          const int64_t* ii, const int64_t* jj, const int32_t* src_member,
                          const int32_t* mem_family, double* dets, int32_t* path, cudaStream_t s);

@@ -73,6 +73,27 @@ def test_weights_of_very_different_sizes(M, spread):
     check(M, w)
 
 
+def test_complex_weights(M):
+    """Complex weights in one pass: the four real-weight oracle sums of the bilinear form."""
+    w = big([6, 4], [48, 36], [4, 5, 6, 1] * 16, SINKS, seed=12, forced_frac=0.05, twins=8)
+    rng = np.random.default_rng(18)
+    ws = w.w_src + 1j * rng.normal(size=w.w_src.shape)
+    wk = w.w_snk + 1j * rng.normal(size=w.w_snk.shape)
+    ws[3], ws[4], ws[5] = 1j, 2.0, 0.0
+    plan = M.Plan.from_workload(w)
+    S = [torch.from_numpy(s).cuda() for s in w.S]
+    out = M.mhc_correlator_cw(plan.handle, S, torch.from_numpy(ws).cuda(), torch.from_numpy(wk).cuda())
+    ref, scale = 0.0, 0.0
+    for x, fx in ((ws.real, 1.0), (ws.imag, 1j)):
+        for y, fy in ((wk.real, 1.0), (wk.imag, 1j)):
+            c, s = oracle.correlator(w.S, w.n_f, w.labels_src, np.ascontiguousarray(x), w.labels_snk,
+                                     np.ascontiguousarray(y), threads=8)
+            ref, scale = ref + fx * fy * c, scale + s
+    assert abs(complex(*out.cpu().numpy()) - ref) <= 1e-11 * scale
+    assert M.mhc_get_status_code(plan.handle) == M.MHC_OK
+    plan.close()
+
+
 def test_structured_propagators(M):
     """Zeros, exactly repeated rows and labels, real entries: determinants that vanish exactly."""
     w = big([4, 3], [24, 24], [4, 5, 6, 1] * 16, SINKS, seed=10)

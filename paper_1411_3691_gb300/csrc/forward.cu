@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const double2* _
 size_t forward_smem_bytes(int slots, int tile, int ncmax) {
   const size_t cache = (size_t)slots * tile * sizeof(double2);
   const size_t scratch = ncmax <= 8 ? WarpScratch<8>::kBytes : ncmax <= 18 ? WarpScratch<18>::kBytes : WarpScratch<32>::kBytes;
-  const size_t labels = (size_t)(slots + 2 * MHC_FMAX) * tile * sizeof(short);  // fwd::FxLane
+  const size_t labels = (size_t)(slots + MHC_FMAX) * tile * sizeof(short);  // fwd::FxLane
   return cache + (size_t)(tile / 32) * scratch + labels;
 }
 

@@ -372,26 +372,24 @@ __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int
 
 // ---- solves and member dots in fixed point (fx.cuh) -------------------------------------
 // The warp's cached solves are fixed-point vectors in the y cache (rank 1: the n entries of y up
-// to a complex factor; rank 2: the 2 n entries of z1 and z2, sd stays FP64), with two shorts per
-// flavour and lane beside the column labels: the vector's exponent and how many binades its
-// largest entry lies below it.
+// to a complex factor; rank 2: the 2 n entries of z1 and z2, sd stays FP64), with the vector's
+// exponent per flavour and lane beside the column labels.
 struct FxLane {
   unsigned short* lab;  // [slot][T] column labels, at the lane
   short* ey;            // [F][T] 2 e_y (an entry of 2^56 stands for 2^e_y), + 1 when the block's det B is a factor
-  short* low;           // [F][T] binades of the largest entry below 2^56
 };
 template <int NCMAX>
 __device__ __forceinline__ FxLane fx_lane(const FwdArgs& a, double2* smem, int T) {
   char* base = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)(T >> 5) * WarpScratch<NCMAX>::kBytes;
   unsigned short* lab = reinterpret_cast<unsigned short*>(base);
   short* ey = reinterpret_cast<short*>(lab + (size_t)a.slots * T);
-  return FxLane{lab, ey, ey + MHC_FMAX * T};
+  return FxLane{lab, ey};
 }
 
 // Solve of one flavour in fixed point; false: the lane takes the FP64 factorisation.  Ks: the
 // block's factors staged in shared memory, or null.
 __device__ __forceinline__ bool fx_solve(const FwdArgs& a, int W, int Q, int f, const int32_t* col, const int4* Ks,
-                                         double2* Yf, int T, short* ey, short* low) {
+                                         double2* Yf, int T, short* ey) {
   const int n = a.n_f[f], rho = a.fam_rank[(int64_t)W * a.F + f], M = n - rho;
   const double2* K = a.kbuf + ((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f];
   const int4* Kg = reinterpret_cast<const int4*>(K);
@@ -425,19 +423,14 @@ __device__ __forceinline__ bool fx_solve(const FwdArgs& a, int W, int Q, int f, 
   } else {
     z[M * T] = one;
   }
-  int top = 64 - __clz(mag);  // bits of the largest entry (32 when below 2^32)
-  if (top > fx::kFracBits) {
-    const int sh = top - fx::kFracBits;
-    for (int q = 0; q < rho * n; q++) {
-      int4& v = reinterpret_cast<int4*>(Yf)[q * T];
-      const fx::Val x = fx::joined(v);
-      v = fx::limbs(x.re >> sh, x.im >> sh);
-    }
-    u += sh;
-    top = fx::kFracBits;
+  // the largest entry just below 2^56 (its bits by the high word: 32 when below 2^32)
+  const int sh = 64 - __clz(mag) - fx::kFracBits;
+  for (int q = 0; q < rho * n; q++) {
+    int4& v = reinterpret_cast<int4*>(Yf)[q * T];
+    const fx::Val x = fx::joined(v);
+    v = fx::limbs(fx::shift(x.re, sh), fx::shift(x.im, sh));
   }
-  *ey = (short)(2 * (u + fx::kFracBits) + 1);
-  *low = (short)(fx::kFracBits - top);
+  *ey = (short)(2 * (u + sh + fx::kFracBits) + 1);
   return true;
 }
 
@@ -463,7 +456,7 @@ __device__ __forceinline__ const int4* fx_stage(const FwdArgs& a, int W, int Q, 
 
 // A flavour's FP64 solve to fixed point, in place; ey: the member guard's scale exponent as the
 // FP64 producers define it.  false (and nothing changed): not finite, or without a normal exponent.
-__device__ __forceinline__ bool fx_from_fp64(int n, int rho, double2* Yf, int T, int ey, short* out_e, short* low) {
+__device__ __forceinline__ bool fx_from_fp64(int n, int rho, double2* Yf, int T, int ey, short* out_e) {
   if (rho == 2) {
     const double2 sd = Yf[2 * n * T];
     if (!dev::finite2(sd) || dev::expo(sd) < -900) return false;
@@ -472,7 +465,6 @@ __device__ __forceinline__ bool fx_from_fp64(int n, int rho, double2* Yf, int T,
   if (ey >= 900 || ey <= -900) return false;
   for (int q = 0; q < rho * n; q++) reinterpret_cast<int4*>(Yf)[q * T] = fx::quant(Yf[q * T], ey + 1, fx::kFracBits);
   *out_e = (short)(2 * (ey + 1));
-  *low = 0;
   return true;
 }
 
@@ -563,7 +555,7 @@ static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S
 
 // One work item (family W x sink tile) by the whole thread block; the block's sum goes
 // to *partial.  Shared by the per-plan launch and the persistent batched launch. 
-template <int NCMAX>
+template <int NCMAX, bool FX>
 __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, double2* smem,
                                          double2* partial) {
   const int T = blockDim.x;
@@ -582,9 +574,9 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   const double2* Yw = smem + (tid & ~31);  // the warp's cached solves (lane l: Yw + l)
 
   // ---- per flavour: solve, or factorise the shared rows, for this sink ----------------
-  constexpr bool kFx = NCMAX <= 18;
+  constexpr bool kFx = FX;
   const FxLane fl = fx_lane<NCMAX>(a, smem, T);
-  bool fxm = kFx && a.fx.nf > 0 && kW <= 2 * fx::kFlush, bad = false;
+  bool fxm = kFx && a.fx.nf > 0 && kW <= fx::kMaxMembers, bad = false;
   for (int f = 0; f < a.F; f++) fxm &= a.fam_rank[(int64_t)W * a.F + f] <= 2;
   const short* eyw = fl.ey + (tid & ~31);
   // flavours solved in fixed point; left to the FP64 factorisation; FP64 solves converted
@@ -604,7 +596,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       const bool blk = fx_block(a, W, Q, f, qtwo);
       const int4* Ks = __any_sync(0xffffffffu, blk) ? fx_stage<NCMAX>(a, W, Q, f, lane, scratch) : nullptr;
       if (blk) {
-        done = fx_solve(a, W, Q, f, cols + a.off_f[f], Ks, Yf, T, fl.ey + f * T + tid, fl.low + f * T + tid);
+        done = fx_solve(a, W, Q, f, cols + a.off_f[f], Ks, Yf, T, fl.ey + f * T + tid);
         if (done) infx |= 1u << f; else solo |= 1u << f;
       }
     }
@@ -625,7 +617,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         pguard |= (unsigned)g << f;
       }
       if constexpr (kFx) {
-        if (fxm && fx_from_fp64(n, rho, Yf, T, ey, fl.ey + f * T + tid, fl.low + f * T + tid)) made |= 1u << f;
+        if (fxm && fx_from_fp64(n, rho, Yf, T, ey, fl.ey + f * T + tid)) made |= 1u << f;
         bad |= fxm && !((made >> f) & 1);
       }
     }
@@ -781,24 +773,24 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
     }
   };
   // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
-  fx::Acc tot;
+  fx::Acc2 tot;
   auto flush = [&]() {
     double re, im;
     int e = a.fx.fexp[W] + le;
     if (a.fx.nf == 1) {
       re = (double)tot.rp;
       im = (double)tot.ih;
-      e -= fx::kSplitBits;
+      e -= fx::kDotBits;
     } else {
-      constexpr double k29 = 536870912.0;
-      re = fma((double)(tot.rp - tot.rn), k29, (double)(tot.lp - tot.ln));
-      im = fma((double)tot.ih, k29, (double)tot.il);
-      e += 29 - 2 * fx::kSplitBits;
+      constexpr double k30 = 1073741824.0;
+      re = fma((double)tot.hi_re(), k30, (double)tot.lo_re());
+      im = fma((double)tot.hi_im(), k30, (double)tot.lo_im());
+      e += 30 - 2 * fx::kSplitBits;
     }
     const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
     acc.x += v.x;
     acc.y += v.y;
-    tot = fx::Acc();
+    tot = fx::Acc2();
   };
   const int thr1 = fx::threshold(a.kc, 1, 0), thr2 = fx::threshold(a.kc, 2, 0);
   // members four at a time (a step that they do not fill repeats the last one)
@@ -832,11 +824,11 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         } else {
           fx_dots<kN>(n, r, lb, Yf, T, v);
         }
-        const int low = rho * fl.low[f * T + tid], thr = rho == 2 ? thr2 : thr1;
+        const int thr = rho == 2 ? thr2 : thr1;
 #pragma unroll
         for (int k = 0; k < kN; k++) {
           const int tk = at == 0 ? a.fx.thr[mem0 + min(c + k, kW - 1)] : thr;
-          bool ok = fx::usable(fx::magnitude(v[k]), fx::lane_threshold(tk, low));
+          const bool ok = fx::usable(fx::magnitude(v[k]), tk);
           u[k] = at == 0 ? v[k] : u[k];
           t[k] = v[k];
           slow[k] = (at > 0 && slow[k]) || !ok;
@@ -848,9 +840,9 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         if (c + k >= kW) slow[k] = false;
         const bool use = c + k < kW && !slow[k];
         const fx::Val uz{use ? u[k].re : 0, use ? u[k].im : 0};
-        if (a.fx.nf == 1) {  // kFlush values of 2^57
-          tot.rp += (uz.re + 4) >> 3;
-          tot.ih += (uz.im + 4) >> 3;
+        if (a.fx.nf == 1) {  // kFlush values below 2^60
+          tot.rp += uz.re;
+          tot.ih += uz.im;
         } else {
           fx::mac(tot, fx::split(uz), fx::split(t[k]));
         }
@@ -900,13 +892,15 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
 // Registers: the n <= 8 class keeps 168 (12 one-warp blocks per SM, or 3 blocks of its
 // 128-thread tile); the larger classes may use all 255, measured fastest for n = 18 (8 blocks
 // per SM against 9 at 216 and 10 at 200, whose spills cost more than the warps gain).
-template <int NCMAX>
+// FX: the plan has fixed-point tables; without them the kernel holds the FP64 path alone (half the
+// code, and 53 instead of 66 us for 512 x 512 terms of n = 3).
+template <int NCMAX, bool FX>
 __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) {
   extern __shared__ double2 smem[];
   const int64_t item = a.item0 + blockIdx.x;
   const int64_t pos = item / a.n_tiles;
   const int W = a.fam_order ? a.fam_order[pos] : (int)pos;
-  fwd_item<NCMAX>(a, W, (int)(item % a.n_tiles), smem, &a.partials[item]);
+  fwd_item<NCMAX, FX>(a, W, (int)(item % a.n_tiles), smem, &a.partials[item]);
 }
 
 // Flavours of a pair that pair_group_kernel takes: blocks that do not fit in a thread's registers.
@@ -1333,7 +1327,7 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) batch_kernel(const FwdArgs* 
     if (it >= n_items) break;
     const BatchItem bi = items[it];
     const FwdArgs& a = desc[bi.corr];
-    fwd::fwd_item<NCMAX>(a, bi.W, bi.tile, smem,
+    fwd::fwd_item<NCMAX, NCMAX <= 18>(a, bi.W, bi.tile, smem,
                     &partials[part_off[bi.corr] + (int64_t)bi.W * a.n_tiles + bi.tile]);
     __syncthreads();
   }
@@ -1361,12 +1355,12 @@ int batch_occupancy_nc(int T, size_t smem) {
   return nb > 0 ? nb : 1;
 }
 
-template <int NCMAX>
+template <int NCMAX, bool FX>
 cudaError_t launch_fwd_nc(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(fwd::fwd_kernel<NCMAX>,
+  cudaError_t e = cudaFuncSetAttribute(fwd::fwd_kernel<NCMAX, FX>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fwd::fwd_kernel<NCMAX><<<(unsigned)items, tile, smem, s>>>(a);
+  fwd::fwd_kernel<NCMAX, FX><<<(unsigned)items, tile, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -35,7 +35,8 @@ constexpr int kMaxHi = 1 << 28;         // high word of 2^60: a larger dot is no
 constexpr int kMulHi = 1 << 27;         // high word of 2^59: the largest factor of mul
 constexpr int kNever = 0x7fffffff;      // threshold of a member that the FP64 path evaluates
 constexpr int kMaxAlign = 10;           // most bits a family's common exponent may cost a member
-constexpr int kFlush = 32;              // products per 64-bit sum (see mac of split values)
+constexpr int kFlush = 8;              // members per 64-bit sum of products (Acc2)
+constexpr int kMaxMembers = 64;
 
 // round(x 2^(b - e)) for |x| < 2^e, b <= 56
 __device__ __forceinline__ long long quant(double x, int e, int b) {
@@ -125,22 +126,38 @@ __device__ __forceinline__ int threshold(int kc, int rank, int d) {
   return t >= 28 ? kNever : t <= 0 ? 1 : 1 << t;
 }
 
-// the threshold of a lane whose vector's largest entry is `s` binades below 2^56
-__device__ __forceinline__ int lane_threshold(int thr, int s) { return thr > kMaxHi ? kNever : max(thr >> s, 1); }
-
-// limbs in base 2^29 of value / 8, |value| < 2^60: |hi| <= 2^28, lo in [-2^28, 2^28), so a
-// product's four cross terms stay below 2^58 and kFlush products below 2^63.  The three bits
-// dropped are 2^-55 of the dot's scale.
-constexpr int kSplitBits = kDotBits - 3;  // 2^54 stands for the scale then
+// Products of two dots.  A dot's scale is an upper bound that it stays a few binades below, and a
+// member's weight and rows may put it another few below its family's exponent: the product keeps
+// 57 bits of the scale of each factor, and its lo lo terms.  (With 54 bits and without them the
+// correlator of 1291 x 977 terms of n = 5, 4 was off by 8e-14, against 1.8e-15 in FP64.)
+// Limbs in base 2^30 of value / 2, |value| < 2^60: |hi| <= 2^29, lo in [-2^29, 2^29); kFlush products
+// of four cross terms each stay below 2^63.
+constexpr int kSplitBits = kDotBits - 1;  // 2^56 stands for the scale then
 __device__ __forceinline__ int4 split(Val v) {
-  const int rh = (int)((v.re + (1ll << 31)) >> 32), ih = (int)((v.im + (1ll << 31)) >> 32);
-  return make_int4(rh, (int)(v.re >> 3) - (rh << 29), ih, (int)(v.im >> 3) - (ih << 29));
+  const int rh = (int)((v.re + (1ll << 30)) >> 31), ih = (int)((v.im + (1ll << 30)) >> 31);
+  return make_int4(rh, (int)(v.re >> 1) - (rh << 30), ih, (int)(v.im >> 1) - (ih << 30));
+}
+struct Acc2 : Acc {
+  long long qp = 0, qn = 0, qi = 0;  // lo lo
+  // the sums in units of 2^60 and 2^30
+  __device__ __forceinline__ long long hi_re() const { return rp - rn; }
+  __device__ __forceinline__ long long lo_re() const { return lp - ln + ((qp - qn) >> 30); }
+  __device__ __forceinline__ long long hi_im() const { return ih; }
+  __device__ __forceinline__ long long lo_im() const { return il + (qi >> 30); }
+};
+__device__ __forceinline__ void mac(Acc2& s, int4 a, int4 b) {
+  mac(static_cast<Acc&>(s), a, b);
+  s.qp = madw(a.y, b.y, s.qp);
+  s.qn = madw(a.w, b.w, s.qn);
+  s.qi = madw(a.y, b.w, s.qi);
+  s.qi = madw(a.w, b.y, s.qi);
 }
 // a b / 2 with 2^56 for the product of the scales (a, b: limbs of values below 2^59)
 __device__ __forceinline__ Val mul(int4 a, int4 b) {
-  Acc s;
+  Acc2 s;
   mac(s, a, b);
-  return Val{((s.rp - s.rn) << 6) + ((s.lp - s.ln + (1ll << 22)) >> 23), (s.ih << 6) + ((s.il + (1ll << 22)) >> 23)};
+  constexpr long long half = 1ll << 25;
+  return Val{(s.hi_re() << 4) + ((s.lo_re() + half) >> 26), (s.hi_im() << 4) + ((s.lo_im() + half) >> 26)};
 }
 
 // ---- triangular solves ------------------------------------------------------------------

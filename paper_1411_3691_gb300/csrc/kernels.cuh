@@ -360,7 +360,7 @@ struct WarpScratch {
 
 constexpr int kReduceMaxBlocks = 128;
 
-// host-side launchers (forward.cu, fxprep.cu and fwd_nc*.cu)
+// host-side launchers (forward.cu, fxprep.cu and the translation units per n class)
 cudaError_t launch_fxprep(const FwdArgs& a, cudaStream_t s);
 cudaError_t launch_fxprep_batch(const FwdArgs* desc, const int64_t* pref, int count, int64_t total, cudaStream_t s);
 int64_t fxprep_blocks(const FwdArgs& a);
@@ -387,6 +387,8 @@ size_t forward_smem_bytes(int slots, int tile, int ncmax);
   cudaError_t launch_kfac_batch_nc##NC(const FwdArgs* desc, const int64_t* kpref,            \
                                        const int64_t* nfam, int count, int64_t total,         \
                                        int big, cudaStream_t s);
+cudaError_t launch_fwd_fx_nc8(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
+cudaError_t launch_fwd_fx_nc18(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
 MHC_DECL_NC(8)
 MHC_DECL_NC(18)
 MHC_DECL_NC(32)

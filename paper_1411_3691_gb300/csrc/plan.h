@@ -143,4 +143,13 @@ double flops_rank2_block(int n);            // LU factors and -U1^{-1}u of one t
 double flops_block12(int n);                // LU factors of one (one-row, two-column) block
 double flops_kapply12(int n);               // y for one sink of a two-column sink family
 
+// The weighted member rows are members x L entries: above this size the FP64 dots are kept.
+constexpr size_t kMaxFxBytes = (size_t)4 << 30;
+// Below two waves of the n <= 8 kernel's twelve warps per SM a call is a chain of latencies: the
+// tables' launch and the longer code cost more than the FP64 pipe (512 x 512 terms of n = 3, 1824
+// warps: 66 us with the tables, 56 us without; 1291 x 977 of n = 5, 4 in ragged families, 7200
+// warps: 160 us against 203 us).  A batch counts the warps of all its plans.
+constexpr int64_t kMinFxWarps = 2 * 12 * 152;
+inline int64_t fx_warps(const Plan& p) { return p.n_fam * ((p.n_snk + 31) / 32); }
+
 }  // namespace mhc

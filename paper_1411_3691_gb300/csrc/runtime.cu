@@ -121,14 +121,6 @@ size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
   return off;
 }
 
-// The weighted member rows are members x L entries: above this size the FP64 dots are kept.
-constexpr size_t kMaxFxBytes = (size_t)4 << 30;
-// Below two waves of the n <= 8 kernel's twelve warps per SM a call is a chain of latencies: the
-// tables' launch and the longer code cost more than the FP64 pipe (512 x 512 terms of n = 3, 1824
-// warps: 66 us with the tables, 56 us without; 1291 x 977 of n = 5, 4 in ragged families, 7200
-// warps: 160 us against 203 us).
-constexpr int64_t kMinFxWarps = 2 * 12 * 152;
-
 mhc_status ensure_device(Plan& p) {
   int cur = 0;
   MHC_CUDA(cudaGetDevice(&cur));
@@ -229,7 +221,7 @@ mhc_status ensure_device(Plan& p) {
   }
   {
     fx::Tables t;
-    const size_t bytes = p.n_fam * ((p.n_snk + 31) / 32) >= kMinFxWarps ? fx_layout(p, nullptr, &t) : 0;
+    const size_t bytes = fx_warps(p) >= kMinFxWarps ? fx_layout(p, nullptr, &t) : 0;
     if (bytes > 0 && bytes <= kMaxFxBytes && cudaMalloc(&d.fx, bytes) != cudaSuccess) {
       d.fx = nullptr;  // the FP64 dots need no tables
       cudaGetLastError();

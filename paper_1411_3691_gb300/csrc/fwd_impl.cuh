@@ -265,6 +265,11 @@ __device__ __forceinline__ dev::cd fx_factor(const FwdArgs& a, int W, int Q, int
   return a.kbuf[((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f] + (n - 1) * (n - 1) + n];
 }
 
+// The kernel without tables takes real weights only (complex ones go to the kernel with tables,
+// which runs plans without them too); the n <= 32 class has the one kernel.
+template <int NCMAX, bool FX>
+constexpr bool kComplexWeights = FX || NCMAX > 18;
+
 // Refactor one pair per lane (the lanes with have; e: the pair, j: its sink position):
 // the product of the flavours that passed, times fresh determinants of the flavours that
 // failed, accumulated into acc.  With a.rowdiff the row-difference update is tried first
@@ -272,12 +277,12 @@ __device__ __forceinline__ dev::cd fx_factor(const FwdArgs& a, int W, int Q, int
 // family with one or two changed columns (n <= 18) are factorised together (group_fresh);
 // the others one per lane.  Yw: the warp's cached solves (lane l at Yw + l, stride
 // blockDim.x), in fixed point with exponents eyw when fxm; wk: the warp's scratch for group_fresh.
-// Called by the whole warp; a call, not inlined: the member loop keeps its registers and the
-// instruction cache its lines.
-template <int NCMAX>
-__device__ __noinline__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
-                              const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc, unsigned long long& rflops,
-                              unsigned long long& nrd) {
+// Called by the whole warp.
+template <int NCMAX, bool FX>
+__device__ __forceinline__ void refactor_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
+                                               const double2* Yw, bool fxm, const short* eyw, double2* wk,
+                                               double2& acc, unsigned long long& rflops, unsigned long long& nrd) {
+  constexpr bool kCw = kComplexWeights<NCMAX, FX>;
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int T = blockDim.x;
@@ -295,28 +300,32 @@ __device__ __noinline__ void process_pairs(const FwdArgs& a, int W, bool have, c
       const int rho = a.fam_rank[(int64_t)W * a.F + f];
       if (!((cand >> f) & 1) || rho > 2 || n < rho + 1) continue;
       const double2* Yf = Yw + (size_t)a.yoff[f] * T + e.lane;
-      double2 yl[2 * NCMAX + 1];  // the solve of the pair's sink
-      if (fxm) {
-        const int e2 = eyw[f * T + e.lane], eq = e2 >> 1;
-        const double2 fac = fx_factor(a, W, Q, f, e2 & 1, Yf, T);
-        for (int q = 0; q < rho * n; q++) {
-          yl[q] = fx::value(reinterpret_cast<const int4*>(Yf)[q * T], eq);
-          if (rho == 1) yl[q] = dev::cmul(yl[q], fac);
+      double2 yl[FX ? 2 * NCMAX + 1 : 1];  // the solve of the pair's sink, when it is not FP64
+      const double2* y = Yf;
+      int ys = T;
+      if constexpr (FX) {
+        if (fxm) {
+          const int e2 = eyw[f * T + e.lane], eq = e2 >> 1;
+          const double2 fac = fx_factor(a, W, Q, f, e2 & 1, Yf, T);
+          for (int q = 0; q < rho * n; q++) {
+            yl[q] = fx::value(reinterpret_cast<const int4*>(Yf)[q * T], eq);
+            if (rho == 1) yl[q] = dev::cmul(yl[q], fac);
+          }
+          if (rho == 2) yl[2 * n] = fac;
+          y = yl;
+          ys = 1;
         }
-        if (rho == 2) yl[2 * n] = fac;
-      } else {
-        for (int q = 0; q < rho * n + (rho == 2); q++) yl[q] = Yf[q * T];
       }
-      const int ey = dev::cached_scale(yl, 1, n, rho);
+      const int ey = dev::cached_scale(y, ys, n, rho);
       bool f2 = true;
       const int32_t* mlab = a.mem_lab + ((int64_t)e.member * a.F + f) * MHC_MAX_RANK;
       const int32_t* arow = a.fam_arow + (int64_t)W * a.Tn + a.off_f[f];
       double2 d;
       if constexpr (NCMAX >= 10)  // two-row families need n_f >= 10
-        d = rho == 1 ? dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2)
-                     : dev::rowdiff2_det(a.S[f], a.L_f[f], n, mlab, arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2);
+        d = rho == 1 ? dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], y, ys, ey, a.kc, &f2)
+                     : dev::rowdiff2_det(a.S[f], a.L_f[f], n, mlab, arow, cols + a.off_f[f], y, ys, ey, a.kc, &f2);
       else
-        d = dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], yl, 1, ey, a.kc, &f2);
+        d = dev::rowdiff_det(a.S[f], a.L_f[f], n, mlab[0], arow, cols + a.off_f[f], y, ys, ey, a.kc, &f2);
       rflops += rho == 1 ? dev::rowdiff_flops(n) : dev::rowdiff2_flops(n);
       if (!f2) {
         prod = dev::cmul(prod, d);
@@ -355,11 +364,30 @@ __device__ __noinline__ void process_pairs(const FwdArgs& a, int W, bool have, c
       rflops += fresh_flops(n);
     }
   }
-  if (have) acc = dev::add_weighted(a, e.w, prod, acc);
+  if (have) acc = dev::add_weighted<kCw>(a, e.w, prod, acc);
+}
+
+// With the fixed-point member loop a call, not inlined: that loop keeps its registers and the
+// instruction cache its lines.
+template <int NCMAX>
+__device__ __noinline__ void refactor_call(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
+                                           const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc,
+                                           unsigned long long& rflops, unsigned long long& nrd) {
+  refactor_pairs<NCMAX, true>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
+}
+
+template <int NCMAX, bool FX>
+__device__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j, const double2* Yw,
+                              bool fxm, const short* eyw, double2* wk, double2& acc, unsigned long long& rflops,
+                              unsigned long long& nrd) {
+  if constexpr (FX)
+    refactor_call<NCMAX>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
+  else
+    refactor_pairs<NCMAX, false>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
 }
 
 // Refactor the first count queued pairs (one per lane).  Called by the whole warp.
-template <int NCMAX>
+template <int NCMAX, bool FX>
 __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int64_t jbase,
                               const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc,
                               unsigned long long& rflops, unsigned long long& nrd) {
@@ -367,7 +395,7 @@ __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int
   const bool have = lane < count;
   QEntry e = {};
   if (have) e = q[lane];
-  process_pairs<NCMAX>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, fxm, eyw, wk, acc, rflops, nrd);
+  process_pairs<NCMAX, FX>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, fxm, eyw, wk, acc, rflops, nrd);
 }
 
 // ---- solves and member dots in fixed point (fx.cuh) -------------------------------------
@@ -574,7 +602,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   const double2* Yw = smem + (tid & ~31);  // the warp's cached solves (lane l: Yw + l)
 
   // ---- per flavour: solve, or factorise the shared rows, for this sink ----------------
-  constexpr bool kFx = FX;
+  constexpr bool kFx = FX, kCw = kComplexWeights<NCMAX, FX>;
   const FxLane fl = fx_lane<NCMAX>(a, smem, T);
   bool fxm = kFx && a.fx.nf > 0 && kW <= fx::kMaxMembers, bad = false;
   for (int f = 0; f < a.F; f++) fxm &= a.fam_rank[(int64_t)W * a.F + f] <= 2;
@@ -685,7 +713,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   }
 
   // ---- per member: one dot product per flavour --------------------------------------
-  const double2 wj = valid ? dev::sink_weight(a, j) : make_double2(0.0, 0.0);
+  const double2 wj = valid ? dev::sink_weight<kCw>(a, j) : make_double2(0.0, 0.0);
   // acc: sum over the members of w_i prod_f det (this lane's sink; times w_j once, at the
   // end); accq: the refactored pairs, w_i w_j included (a queue lane holds other sinks' pairs)
   double2 acc = make_double2(0.0, 0.0), accq = make_double2(0.0, 0.0);
@@ -730,8 +758,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       }
     }
     const bool need = valid && part && fail != 0;
-    const double2 wi = dev::source_weight(a, m);
-    if (part && !fail) acc = dev::add_weighted(a, wi, prod, acc);
+    const double2 wi = dev::source_weight<kCw>(a, m);
+    if (part && !fail) acc = dev::add_weighted<kCw>(a, wi, prod, acc);
     const unsigned ball = __ballot_sync(0xffffffffu, need);
     if (ball == 0xffffffffu) {
       // every lane refactors this member (a member near-singular against its family): the
@@ -743,8 +771,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       e.fail = (int32_t)fail;
       e.pguard = (int32_t)pguard;
       e.prod = prod;
-      e.w = dev::add_weighted(a, wi, wj, make_double2(0.0, 0.0));
-      process_pairs<NCMAX>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+      e.w = dev::add_weighted<kCw>(a, wi, wj, make_double2(0.0, 0.0));
+      process_pairs<NCMAX, FX>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
       n_parent += __popc(fail & pguard);
       n_child += __popc(fail & ~pguard);
     } else if (ball) {
@@ -756,7 +784,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         e.fail = (int32_t)fail;
         e.pguard = (int32_t)pguard;
         e.prod = prod;
-        e.w = dev::add_weighted(a, wi, wj, make_double2(0.0, 0.0));
+        e.w = dev::add_weighted<kCw>(a, wi, wj, make_double2(0.0, 0.0));
         queue[pos] = e;
         n_parent += __popc(fail & pguard);
         n_child += __popc(fail & ~pguard);
@@ -764,7 +792,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       qn += __popc(ball);
       __syncwarp();
       if (qn >= 32) {
-        process_queue<NCMAX>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+        process_queue<NCMAX, FX>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
         __syncwarp();
         if (lane < qn - 32) queue[lane] = queue[32 + lane];
         __syncwarp();
@@ -772,93 +800,97 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       }
     }
   };
-  // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
-  fx::Acc2 tot;
-  auto flush = [&]() {
-    double re, im;
-    int e = a.fx.fexp[W] + le;
-    if (a.fx.nf == 1) {
-      re = (double)tot.rp;
-      im = (double)tot.ih;
-      e -= fx::kDotBits;
-    } else {
-      constexpr double k30 = 1073741824.0;
-      re = fma((double)tot.hi_re(), k30, (double)tot.lo_re());
-      im = fma((double)tot.hi_im(), k30, (double)tot.lo_im());
-      e += 30 - 2 * fx::kSplitBits;
-    }
-    const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
-    acc.x += v.x;
-    acc.y += v.y;
-    tot = fx::Acc2();
-  };
-  const int thr1 = fx::threshold(a.kc, 1, 0), thr2 = fx::threshold(a.kc, 2, 0);
-  // members four at a time (a step that they do not fill repeats the last one)
-  constexpr int kN = 4;
-  const int step = kFx && fxm ? kN : 1;
-  for (int c = 0; c < kW; c += step) {
-    bool slow[4] = {true, true, true, true};  // this lane's pair with member c + k goes through FP64
-    if (kFx && fxm) {
-      fx::Val u[kN], t[kN];
-      int at = 0;
-      for (int f = 0; f < a.F; f++) {
-        const int n = a.n_f[f], L = a.L_f[f];
-        if (n == 0) continue;
-        const int rho = a.fam_rank[(int64_t)W * a.F + f];
-        const unsigned short* lb = fl.lab + (size_t)a.yoff[f] * T + tid;
-        const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
-        fx::Val v[kN];
-        const int4* r[kN];
-#pragma unroll
-        for (int k = 0; k < kN; k++) {
-          const int m = mem0 + min(c + k, kW - 1);
-          r[k] = at == 0 ? a.fx.ws + (size_t)m * L
-                         : a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK] * L;
-        }
-        if (NCMAX >= 10 && rho == 2) {
-#pragma unroll
+  if constexpr (!kFx) {
+    for (int c = 0; c < kW; c++) member64(c, true);
+  } else {
+    // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
+    fx::Acc2 tot;
+    auto flush = [&]() {
+      double re, im;
+      int e = a.fx.fexp[W] + le;
+      if (a.fx.nf == 1) {
+        re = (double)tot.rp;
+        im = (double)tot.ih;
+        e -= fx::kDotBits;
+      } else {
+        constexpr double k30 = 1073741824.0;
+        re = fma((double)tot.hi_re(), k30, (double)tot.lo_re());
+        im = fma((double)tot.hi_im(), k30, (double)tot.lo_im());
+        e += 30 - 2 * fx::kSplitBits;
+      }
+      const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
+      acc.x += v.x;
+      acc.y += v.y;
+      tot = fx::Acc2();
+    };
+    const int thr1 = fx::threshold(a.kc, 1, 0), thr2 = fx::threshold(a.kc, 2, 0);
+    // members four at a time (a step that they do not fill repeats the last one)
+    constexpr int kN = 4;
+    const int step = fxm ? kN : 1;
+    for (int c = 0; c < kW; c += step) {
+      bool slow[4] = {true, true, true, true};  // this lane's pair with member c + k goes through FP64
+      if (fxm) {
+        fx::Val u[kN], t[kN];
+        int at = 0;
+        for (int f = 0; f < a.F; f++) {
+          const int n = a.n_f[f], L = a.L_f[f];
+          if (n == 0) continue;
+          const int rho = a.fam_rank[(int64_t)W * a.F + f];
+          const unsigned short* lb = fl.lab + (size_t)a.yoff[f] * T + tid;
+          const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
+          fx::Val v[kN];
+          const int4* r[kN];
+  #pragma unroll
           for (int k = 0; k < kN; k++) {
             const int m = mem0 + min(c + k, kW - 1);
-            v[k] = fx_det2(n, r[k], a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK + 1] * L, lb, Yf, T);
+            r[k] = at == 0 ? a.fx.ws + (size_t)m * L
+                           : a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK] * L;
           }
-        } else {
-          fx_dots<kN>(n, r, lb, Yf, T, v);
+          if (NCMAX >= 10 && rho == 2) {
+  #pragma unroll
+            for (int k = 0; k < kN; k++) {
+              const int m = mem0 + min(c + k, kW - 1);
+              v[k] = fx_det2(n, r[k], a.fx.s[f] + (size_t)a.mem_lab[((int64_t)m * a.F + f) * MHC_MAX_RANK + 1] * L, lb, Yf, T);
+            }
+          } else {
+            fx_dots<kN>(n, r, lb, Yf, T, v);
+          }
+          const int thr = rho == 2 ? thr2 : thr1;
+  #pragma unroll
+          for (int k = 0; k < kN; k++) {
+            const int tk = at == 0 ? a.fx.thr[mem0 + min(c + k, kW - 1)] : thr;
+            const bool ok = fx::usable(fx::magnitude(v[k]), tk);
+            u[k] = at == 0 ? v[k] : u[k];
+            t[k] = v[k];
+            slow[k] = (at > 0 && slow[k]) || !ok;
+          }
+          at++;
         }
-        const int thr = rho == 2 ? thr2 : thr1;
-#pragma unroll
+  #pragma unroll
         for (int k = 0; k < kN; k++) {
-          const int tk = at == 0 ? a.fx.thr[mem0 + min(c + k, kW - 1)] : thr;
-          const bool ok = fx::usable(fx::magnitude(v[k]), tk);
-          u[k] = at == 0 ? v[k] : u[k];
-          t[k] = v[k];
-          slow[k] = (at > 0 && slow[k]) || !ok;
+          if (c + k >= kW) slow[k] = false;
+          const bool use = c + k < kW && !slow[k];
+          const fx::Val uz{use ? u[k].re : 0, use ? u[k].im : 0};
+          if (a.fx.nf == 1) {  // kFlush values below 2^60
+            tot.rp += uz.re;
+            tot.ih += uz.im;
+          } else {
+            fx::mac(tot, fx::split(uz), fx::split(t[k]));
+          }
         }
-        at++;
+        if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) flush();
       }
-#pragma unroll
-      for (int k = 0; k < kN; k++) {
-        if (c + k >= kW) slow[k] = false;
-        const bool use = c + k < kW && !slow[k];
-        const fx::Val uz{use ? u[k].re : 0, use ? u[k].im : 0};
-        if (a.fx.nf == 1) {  // kFlush values below 2^60
-          tot.rp += uz.re;
-          tot.ih += uz.im;
-        } else {
-          fx::mac(tot, fx::split(uz), fx::split(t[k]));
-        }
+      // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
+  #pragma unroll 1
+      for (int k = 0; k < step; k++) {
+        const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
+        if (__any_sync(0xffffffffu, p)) member64(c + k, p);
       }
-      if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) flush();
-    }
-    // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
-#pragma unroll 1
-    for (int k = 0; k < step; k++) {
-      const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
-      if (__any_sync(0xffffffffu, p)) member64(c + k, p);
     }
   }
   __syncwarp();
-  if (qn > 0) process_queue<NCMAX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
-  acc = dev::add_weighted(a, wj, acc, accq);
+  if (qn > 0) process_queue<NCMAX, FX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+  acc = dev::add_weighted<kCw>(a, wj, acc, accq);
 
   // ---- fixed-order reduction: lanes, then warps --------------------------------------
   acc = dev::warp_sum(acc);
@@ -889,11 +921,39 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   }
 }
 
+// The last block of a call to finish sums the items' partials in a fixed order (smem: past the
+// entries that fwd_item's own sum uses).
+__device__ __forceinline__ void fold_partials(const FwdArgs& a, double2* smem) {
+  const int T = blockDim.x, tid = threadIdx.x;
+  double2* red = smem + 8;
+  int* last = reinterpret_cast<int*>(smem + 16);
+  if (tid == 0) {
+    __threadfence();
+    const unsigned n1 = (unsigned)a.fold_items - 1;
+    *last = atomicInc(a.reduce_done, n1) == n1;  // the last one wraps it to 0
+  }
+  __syncthreads();
+  if (!*last) return;
+  __threadfence();
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int64_t i = tid; i < a.fold_items; i += T) s = dev::cadd(s, __ldcg(a.partials + i));
+  s = dev::warp_sum(s);
+  if ((tid & 31) == 0) red[tid >> 5] = s;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < (T >> 5); w++) s = dev::cadd(s, red[w]);
+    a.out[0] = s.x;
+    a.out[1] = s.y;
+  }
+}
+
 // Registers: the n <= 8 class keeps 168 (12 one-warp blocks per SM, or 3 blocks of its
 // 128-thread tile); the larger classes may use all 255, measured fastest for n = 18 (8 blocks
 // per SM against 9 at 216 and 10 at 200, whose spills cost more than the warps gain).
-// FX: the plan has fixed-point tables; without them the kernel holds the FP64 path alone (half the
-// code, and 53 instead of 66 us for 512 x 512 terms of n = 3).
+// FX: the plan has fixed-point tables, or complex weights; else the kernel holds the FP64 path for
+// real weights alone.  512 x 512 terms of n = 3: 55 us per call, and 64 us when it also carried the
+// complex weights, converted solves for the refactors and a launch for the partials' sum.
 template <int NCMAX, bool FX>
 __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) {
   extern __shared__ double2 smem[];
@@ -901,6 +961,7 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) 
   const int64_t pos = item / a.n_tiles;
   const int W = a.fam_order ? a.fam_order[pos] : (int)pos;
   fwd_item<NCMAX, FX>(a, W, (int)(item % a.n_tiles), smem, &a.partials[item]);
+  if (a.fold_items > 0) fold_partials(a, smem);
 }
 
 // Flavours of a pair that pair_group_kernel takes: blocks that do not fit in a thread's registers.

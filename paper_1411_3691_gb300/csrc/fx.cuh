@@ -35,7 +35,7 @@ constexpr int kMaxHi = 1 << 28;         // high word of 2^60: a larger dot is no
 constexpr int kMulHi = 1 << 27;         // high word of 2^59: the largest factor of mul
 constexpr int kNever = 0x7fffffff;      // threshold of a member that the FP64 path evaluates
 constexpr int kMaxAlign = 10;           // most bits a family's common exponent may cost a member
-constexpr int kFlush = 8;              // members per 64-bit sum of products (Acc2)
+constexpr int kFlush = 8;               // members per 64-bit sum of products (Acc2)
 constexpr int kMaxMembers = 64;
 
 // round(x 2^(b - e)) for |x| < 2^e, b <= 56
@@ -75,8 +75,8 @@ struct Acc {
   long long rp = 0, rn = 0, lp = 0, ln = 0, ih = 0, il = 0;
 };
 // a b + c.  As inline PTX it comes out as a multiplication and an addition on two pipes; the one
-// instruction that the compiler makes of the C expression has half the rate and a longer latency:
-// He-4 shapes 1.04 ms with this, 1.26 ms with that.
+// instruction that the compiler makes of the C expression has half the rate and a longer latency
+// (forward of 512 x 512 terms of n = 3 with these dots: 58 us with this, 64 us with that).
 __device__ __forceinline__ long long madw(int a, int b, long long c) {
 #ifdef __CUDA_ARCH__
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));

@@ -52,7 +52,7 @@ __device__ void prep_family(const FwdArgs& a, int W) {
   // per member: the exponent above w times its first row, and the sum of its other rows' ones
   for (int c = warp; c < kW; c += kThreads / 32) {
     const int m = mem0 + c;
-    const dev::cd w = dev::source_weight(a, m);
+    const dev::cd w = dev::source_weight<true>(a, m);
     const int32_t* lab = a.mem_lab + (int64_t)m * a.F * MHC_MAX_RANK;
     int r = 0, e0 = -4096;
     bool bad = (w.x == 0.0 && w.y == 0.0) || dev::expo(w) >= 1024;

@@ -43,6 +43,9 @@ struct FwdArgs {
   double2* partials;         // [items]
   double2* reduce_blocks;    // reduce_kernel's sums per block, and its counter (0 between calls)
   unsigned* reduce_done;
+  // > 0: that many work items of fwd_kernel, whose last block sums the partials into out
+  int64_t fold_items;
+  double* out;
   unsigned long long* counters;
   // two-sided update; snk_orig == nullptr selects the one-sided update with the sinks
   // in their own order and labels from snk_lab
@@ -269,20 +272,23 @@ __device__ __forceinline__ const int32_t* sink_cols(const FwdArgs& a, int64_t j)
   return (a.snk_orig ? a.snk_pos : a.snk_lab) + j * a.Tn;
 }
 
-// weight of member m with its sign, and of the sink at position j
+// weight of member m with its sign, and of the sink at position j (CW: they may be complex)
+template <bool CW>
 __device__ __forceinline__ cd source_weight(const FwdArgs& a, int m) {
   const int i = a.mem_term[m];
-  const cd w = make_double2(a.w_src[i], a.w_src_im ? a.w_src_im[i] : 0.0);
+  const cd w = make_double2(a.w_src[i], CW && a.w_src_im ? a.w_src_im[i] : 0.0);
   return __popc(a.mem_par[m]) & 1 ? cneg(w) : w;
 }
+template <bool CW>
 __device__ __forceinline__ cd sink_weight(const FwdArgs& a, int64_t j) {
   const int64_t i = a.snk_orig ? a.snk_orig[j] : j;
-  const cd w = make_double2(a.w_snk[i], a.w_snk_im ? a.w_snk_im[i] : 0.0);
+  const cd w = make_double2(a.w_snk[i], CW && a.w_snk_im ? a.w_snk_im[i] : 0.0);
   return a.snk_orig && (__popc(a.snk_par[j]) & 1) ? cneg(w) : w;
 }
 // acc + w z, w real unless the call's weights are complex
+template <bool CW>
 __device__ __forceinline__ cd add_weighted(const FwdArgs& a, cd w, cd z, cd acc) {
-  return a.w_src_im ? cfma(w, z, acc) : make_double2(fma(w.x, z.x, acc.x), fma(w.x, z.y, acc.y));
+  return CW && a.w_src_im ? cfma(w, z, acc) : make_double2(fma(w.x, z.x, acc.x), fma(w.x, z.y, acc.y));
 }
 
 // Rows of member m in flavour f for a fresh factorisation: the shared rows, then the

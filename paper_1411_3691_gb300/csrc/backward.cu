@@ -88,17 +88,29 @@ __global__ void fin_dwsrc_kernel(int64_t n_src, const int32_t* __restrict__ src_
   dw[i] = g[0] * s.x + g[1] * s.y;
 }
 
-// dw_snk[j] = Re(conj(g) sum_W part[W][j])
-__global__ void fin_dwsnk_kernel(int64_t n_snk, int64_t n_fam, const double2* __restrict__ part,
-                                 const double* __restrict__ g, double* __restrict__ dw) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_snk) return;
+// dw_snk[j] = Re(conj(g) sum_W part[W][j]).  One block per 32 sinks, its eight warps the families
+// round-robin, then the warps in order (a thread per sink, 16 blocks for the He-4 shapes, took 54 us
+// for one chain of 256 loads each).
+__global__ void __launch_bounds__(256) fin_dwsnk_kernel(int64_t n_snk, int64_t n_fam, const double2* __restrict__ part,
+                                                        const double* __restrict__ g, double* __restrict__ dw) {
+  __shared__ double2 red[8][32];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int64_t j = (int64_t)blockIdx.x * 32 + lane, jc = j < n_snk ? j : n_snk - 1;
   double2 s = make_double2(0.0, 0.0);
-  for (int64_t W = 0; W < n_fam; W++) {
-    s.x += part[W * n_snk + j].x;
-    s.y += part[W * n_snk + j].y;
+  for (int64_t W = wp; W < n_fam; W += 8) {
+    const double2 v = part[W * n_snk + jc];
+    s.x += v.x;
+    s.y += v.y;
   }
-  dw[j] = g[0] * s.x + g[1] * s.y;
+  red[wp][lane] = s;
+  __syncthreads();
+  if (wp == 0 && j < n_snk) {
+    for (int w = 1; w < 8; w++) {
+      s.x += red[w][lane].x;
+      s.y += red[w][lane].y;
+    }
+    dw[j] = g[0] * s.x + g[1] * s.y;
+  }
 }
 
 template <typename T>
@@ -162,7 +174,7 @@ extern "C" mhc_status mhc_correlator_backward(mhc_plan_t plan, const double* con
               "plan with a smaller opts.max_family");
     return MHC_EUNSUPPORTED;
   }
-  const size_t smem = smem_of(T);
+  const size_t smem = smem_of(T) + (size_t)p.max_n * kLabStride * sizeof(int);  // and the column labels
   const int warps = T / 32;
   const int n_tiles = (int)((p.n_snk + T - 1) / T);
   const int slots_max = Mmax + max_rank * kmax;
@@ -288,7 +300,7 @@ extern "C" mhc_status mhc_correlator_backward(mhc_plan_t plan, const double* con
     fin_dwsrc_kernel<<<(unsigned)((p.n_src + 255) / 256), 256, 0, s>>>(p.n_src, d.src_member, b.dwsrc_part,
                                                                         n_chunks, g_out_dev, dw_src_dev);
   if (dw_snk_dev)
-    fin_dwsnk_kernel<<<(unsigned)((p.n_snk + 255) / 256), 256, 0, s>>>(p.n_snk, p.n_fam, b.dwsnk_part,
+    fin_dwsnk_kernel<<<(unsigned)((p.n_snk + 31) / 32), 256, 0, s>>>(p.n_snk, p.n_fam, b.dwsnk_part,
                                                                         g_out_dev, dw_snk_dev);
   e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -152,20 +152,43 @@ __device__ __forceinline__ bool lu_block(const cd* __restrict__ S, int L, int n_
 #pragma unroll UNR
   for (int k = 0; k < M; k++) {
     double best = dev::abs1(A[k][k]);
+    if constexpr (NFIX > 0) {  // in registers: rows change places as the search goes
 #pragma unroll UNR
-    for (int i = k + 1; i < M; i++) {
-      const double m = dev::abs1(A[i][k]);
-      const bool sw = dev::gt_nonneg(m, best);
-      best = sw ? m : best;
-      parity ^= (int)sw;
-      const int pk = perm[k], pi = perm[i];
-      perm[k] = sw ? pi : pk;
-      perm[i] = sw ? pk : pi;
+      for (int i = k + 1; i < M; i++) {
+        const double m = dev::abs1(A[i][k]);
+        const bool sw = dev::gt_nonneg(m, best);
+        best = sw ? m : best;
+        parity ^= (int)sw;
+        const int pk = perm[k], pi = perm[i];
+        perm[k] = sw ? pi : pk;
+        perm[i] = sw ? pk : pi;
 #pragma unroll UNR
-      for (int q = 0; q < n; q++) {  // whole rows: the multipliers travel with them
-        const cd t = A[k][q];
-        A[k][q] = sw ? A[i][q] : t;
-        A[i][q] = sw ? t : A[i][q];
+        for (int q = 0; q < n; q++) {  // whole rows: the multipliers travel with them
+          const cd t = A[k][q];
+          A[k][q] = sw ? A[i][q] : t;
+          A[i][q] = sw ? t : A[i][q];
+        }
+      }
+    } else {  // in local memory: the search first, then one exchange of rows
+      // (with the scatter's labels: 6.78 -> 5.48 ms for 640 x 768 ragged terms of n = 9, 12)
+      int p = k;
+      for (int i = k + 1; i < M; i++) {
+        const double m = dev::abs1(A[i][k]);
+        if (dev::gt_nonneg(m, best)) {
+          best = m;
+          p = i;
+        }
+      }
+      if (p != k) {
+        parity ^= 1;
+        const int pk = perm[k];
+        perm[k] = perm[p];
+        perm[p] = pk;
+        for (int q = 0; q < n; q++) {
+          const cd t = A[k][q];
+          A[k][q] = A[p][q];
+          A[p][q] = t;
+        }
       }
     }
     const int e = dev::expo(best);
@@ -864,28 +887,33 @@ __device__ __forceinline__ void dispatch_cof_pass(const FwdArgs& a, const BwdArg
 // repeats a label, whose cells are added one column at a time; a __syncwarp after every
 // sink orders the additions to one accumulator entry by sink, so the order is fixed.  Each
 // sink's metadata (sink family, number of shared columns, column labels, weight) sits in
-// the registers of the sink's own lane and reaches the other lanes by shuffles.
+// the registers of the sink's own lane and reaches the other lanes by shuffles, but for the column
+// labels (labs: shared memory, [q][kLabStride]).  Latency bounds it: for n > 6 the labels were an
+// array in local memory, read n times per sink behind as many shuffles, and the cell's value was
+// loaded where it is added; now it is loaded one sink ahead (n > 6 only: with n <= 6 the registers
+// cost more, 8.94 against 8.89 ms on the He-4 shapes).
 template <int NC, int NFIX>
 __device__ __forceinline__ void scatter_rows(const FwdArgs& a, const BwdArgs& B, int f, int n_rt,
                                              int kW, int mem0, int nlive, int T, int warp, int lane,
                                              const int32_t* __restrict__ mycol, int myQ, int mynsh,
                                              const cd* Stage, const cd* Ysm,
-                                             const cd* Dets, cd* Df) {
+                                             const cd* Dets, cd* Df, int* labs) {
   constexpr int UNR = NFIX ? NC : 1;
   constexpr unsigned FULL = 0xffffffffu;
   const int n = NFIX ? NFIX : n_rt;
   const int M = n - 1;
+  constexpr bool kAhead = NFIX == 0;
   const int nslots = M + kW;
   const int ncells = nslots * n;
-  int cl[NC];
 #pragma unroll UNR
-  for (int q = 0; q < n; q++) cl[q] = mycol[q];
+  for (int q = 0; q < n; q++) labs[q * kLabStride + lane] = mycol[q];
   // does this lane's sink repeat a label in flavour f
   int myrep = 0;
 #pragma unroll UNR
   for (int q = 1; q < n; q++)
 #pragma unroll UNR
-    for (int p = 0; p < q; p++) myrep |= cl[q] == cl[p];
+    for (int p = 0; p < q; p++) myrep |= labs[q * kLabStride + lane] == labs[p * kLabStride + lane];
+  __syncwarp();
   for (int e0 = 0; e0 < ncells; e0 += 32) {
     const int e = e0 + lane;
     const bool act = e < ncells;
@@ -899,22 +927,24 @@ __device__ __forceinline__ void scatter_rows(const FwdArgs& a, const BwdArgs& B,
     const int c = mem ? s - M : 0;
     cd* Drow = Df + (size_t)s * B.Lmax;
     const cd* Ycol = Ysm + (size_t)(a.yoff[f] + q) * T;
+    const int* collab = labs + q * kLabStride;  // the label of this cell's column in each sink
+    auto cell = [&](int jl) {
+      const int ts = warp * 32 + jl;
+      return mem ? Ycol[ts] : Stage[(size_t)ts * B.mn_max + s * n + q];
+    };
     // the sweep over the sinks, compiled apart for the steps of shared rows only
     auto sweep = [&](auto sh) {
       cd acc = make_double2(0.0, 0.0);
       int curlab = 0, curQ = -2, nsh = 0;
+      cd next = make_double2(0.0, 0.0);  // the next sink's value, loaded a step ahead
+      if (kAhead) next = cell(0);
       for (int jl = 0; jl <= nlive; jl++) {
         const bool live = jl < nlive;
         const int src = jl & 31;
         const int Qj = __shfl_sync(FULL, myQ, src);
         const int nsj = __shfl_sync(FULL, mynsh, src);
         const int rep = __shfl_sync(FULL, myrep, src);
-        int lab = 0;  // the label of this cell's column in sink jl
-#pragma unroll UNR
-        for (int p = 0; p < n; p++) {
-          const int t = __shfl_sync(FULL, cl[p], src);
-          lab = p == q ? t : lab;
-        }
+        const int lab = collab[src];
         if (!live || Qj != curQ || Qj < 0) {  // flush the summed shared columns of the previous family
           // one column at a time: the family's shared labels may repeat
           for (int p = 0; p < nsh; p++) {
@@ -933,7 +963,8 @@ __device__ __forceinline__ void scatter_rows(const FwdArgs& a, const BwdArgs& B,
         }
         const int ts = warp * 32 + jl;
         const cd g = (mem && !decltype(sh)::value) ? Dets[dix(c, f, B.kmax, T, ts)] : make_double2(1.0, 0.0);
-        const cd v = mem ? Ycol[ts] : Stage[(size_t)ts * B.mn_max + s * n + q];
+        const cd v = kAhead ? next : cell(jl);
+        if (kAhead && jl + 1 < nlive) next = cell(jl + 1);
         const bool shcol = q < nsh;
         if (!rep) {
           // one complex FMA (an addition in a step of shared rows) per lane, on the register
@@ -969,9 +1000,10 @@ template <int NCMAX>
 __device__ __forceinline__ void dispatch_scatter(const FwdArgs& a, const BwdArgs& B, int f, int n,
                                                  int kW, int mem0, int nlive, int T, int warp, int lane,
                                                  const int32_t* mycol, int myQ, int mynsh,
-                                                 const cd* Stage, const cd* Ysm, const cd* Dets, cd* Df) {
+                                                 const cd* Stage, const cd* Ysm, const cd* Dets, cd* Df,
+                                                 int* labs) {
 #define MHC_SC(NN) scatter_rows<NN, NN>(a, B, f, NN, kW, mem0, nlive, T, warp, lane, mycol, myQ, mynsh, \
-                                        Stage, Ysm, Dets, Df)
+                                        Stage, Ysm, Dets, Df, labs)
   switch (n) {
     case 1: MHC_SC(1); return;
     case 2: MHC_SC(2); return;
@@ -981,7 +1013,7 @@ __device__ __forceinline__ void dispatch_scatter(const FwdArgs& a, const BwdArgs
     case 6: MHC_SC(6); return;
     default:
       scatter_rows<NCMAX, 0>(a, B, f, n, kW, mem0, nlive, T, warp, lane, mycol, myQ, mynsh, Stage, Ysm,
-                             Dets, Df);
+                             Dets, Df, labs);
   }
 #undef MHC_SC
 }
@@ -1002,6 +1034,7 @@ __global__ void __launch_bounds__(32, NCMAX <= 8 ? 14 : 9) bwd_kernel(const BwdA
   // global scratch of the block (L1-resident), which leaves the shared memory small enough
   // for the registers to set the occupancy
   cd* Ysm = smem;
+  int* labs = reinterpret_cast<int*>(smem + (size_t)B.ysl * T);  // [q][kLabStride]: scatter_rows
   cd* Dets = B.dets + (size_t)cta * a.F * B.kmax * (T + 1);
   // dw_src accumulators: global scratch of this block (L1/L2-resident), which leaves the
   // shared memory to the data the scatter shares across lanes
@@ -1181,7 +1214,7 @@ __global__ void __launch_bounds__(32, NCMAX <= 8 ? 14 : 9) bwd_kernel(const BwdA
       const int64_t rem = a.n_snk - ((int64_t)tile * T + warp * 32);
       const int nlive = rem < 32 ? (int)rem : 32;
       dispatch_scatter<NCMAX>(a, B, f, n, kW, mem0, nlive, T, warp, lane, col, qtwo ? Q : -1, mynsh,
-                              Stage, Ysm, Dets, Dw + (size_t)f * B.slots_max * B.Lmax);
+                              Stage, Ysm, Dets, Dw + (size_t)f * B.slots_max * B.Lmax, labs);
       __syncwarp();
     }
   }

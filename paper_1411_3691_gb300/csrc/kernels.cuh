@@ -365,6 +365,7 @@ struct WarpScratch {
 };
 
 constexpr int kReduceMaxBlocks = 128;
+constexpr int kLabStride = 33;  // scatter_rows' column labels in shared memory: 32 sinks, padded
 
 // host-side launchers (forward.cu, fxprep.cu and the translation units per n class)
 cudaError_t launch_fxprep(const FwdArgs& a, cudaStream_t s);

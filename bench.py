@@ -135,7 +135,8 @@ def call_launches(plan, w, st) -> int:
     forward kernel's last block sums the partials itself (up to 16 per thread of a block)."""
     n_fam, n_max = len(plan.families()["rank"]), max(w.n_f)
     warps = n_fam * ((len(w.w_snk) + 31) // 32)
-    tables = sum(n > 0 for n in w.n_f) in (1, 2) and n_max <= 18 and warps >= 2 * 12 * 152
+    tables = (sum(n > 0 for n in w.n_f) in (1, 2) and n_max <= 18 and warps >= 2 * 12 * 152
+              and st["two_sided_blocks"] > 0 and (n_max > 8 or len(w.w_src) >= 4 * n_fam))
     tile = 128 if n_max <= 8 else 64 if n_max <= 12 else 32
     folded = n_fam * ((len(w.w_snk) + tile - 1) // tile) <= 16 * tile
     return forward_launches(plan, w, st) + tables - folded

@@ -466,7 +466,7 @@ mhc_status mhc_batch_create(mhc_batch_t* out, int32_t count, const mhc_plan_t* p
   for (int k = 0; k < count && warps >= kMinFxWarps; k++) {
     const Plan& p = *b->plans[k];
     fx::Tables t;
-    const size_t bytes = p.dev.fx ? 0 : fx_layout(p, nullptr, &t);
+    const size_t bytes = p.dev.fx || !fx_pays(p) ? 0 : fx_layout(p, nullptr, &t);
     if (bytes == 0 || fx_own + bytes > kMaxFxBytes) continue;
     if (cudaMalloc(&b->own_fx[k], bytes) != cudaSuccess) {
       b->own_fx[k] = nullptr;

@@ -151,5 +151,17 @@ constexpr size_t kMaxFxBytes = (size_t)4 << 30;
 // warps: 160 us against 203 us).  A batch counts the warps of all its plans.
 constexpr int64_t kMinFxWarps = 2 * 12 * 152;
 inline int64_t fx_warps(const Plan& p) { return p.n_fam * ((p.n_snk + 31) / 32); }
+// The tables pay by the dots, and the sinks' own factorisations stay FP64 work, slower beside the longer
+// code.  For n <= 8, where those and the solves are short and in registers, they take four members
+// per family and few sinks outside families: 2365 x 2081 terms of n = 4, 3 with 18 % of the sinks
+// alone 758 us with the tables and 665 without, 746 x 3136 of n = 5, 6 with 2.2 members per family
+// 1380 and 1151, 870 x 2820 of n = 3, 4 with one member 1341 and 940; 1291 x 977 with 8.4 members and few
+// such sinks 167 and 206.  Above, they paid from one member on (1172 x 415 of n = 10: 1189 and 1299).
+inline bool fx_pays(const Plan& p) {
+  if (!p.dev.two_sided || (p.max_n <= 8 && p.n_src < 4 * p.n_fam)) return false;
+  int64_t alone = 0;
+  for (const int32_t q : p.snk_q) alone += q < 0 || !p.q_two[q];
+  return alone * (p.max_n <= 8 ? 8 : 2) <= p.n_snk;
+}
 
 }  // namespace mhc

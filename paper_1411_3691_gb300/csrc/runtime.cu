@@ -221,7 +221,7 @@ mhc_status ensure_device(Plan& p) {
   }
   {
     fx::Tables t;
-    const size_t bytes = fx_warps(p) >= kMinFxWarps ? fx_layout(p, nullptr, &t) : 0;
+    const size_t bytes = fx_warps(p) >= kMinFxWarps && fx_pays(p) ? fx_layout(p, nullptr, &t) : 0;
     if (bytes > 0 && bytes <= kMaxFxBytes && cudaMalloc(&d.fx, bytes) != cudaSuccess) {
       d.fx = nullptr;  // the FP64 dots need no tables
       cudaGetLastError();

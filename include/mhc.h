@@ -139,6 +139,16 @@ typedef struct {
                                     (mhc_plan_opts.row_difference = 1)                 */
 } mhc_stats;
 
+/* How one mhc_correlator call of a plan runs (mhc_forward_info). */
+typedef struct {
+  int32_t tables;       /* 1: the plan holds fixed-point tables of the propagators      */
+  int32_t tables_used;  /* 1: and the last call's solves and dots ran on them           */
+  int32_t folded_sum;   /* 1: the forward kernel's last block sums the partials, no
+                           launch of its own                                           */
+  int32_t launches;     /* kernel launches of one call                                 */
+  int64_t table_bytes;  /* device memory of the tables (0 without)                      */
+} mhc_forward_path;
+
 /* Thread-local message describing the last failure of this thread's last call. */
 const char* mhc_last_error(void);
 
@@ -176,6 +186,13 @@ void mhc_plan_destroy(mhc_plan_t plan);
 /* Copy the plan's statistics (including the last run's device counters, as of the
  * last mhc_get_status). */
 mhc_status mhc_plan_stats(mhc_plan_t plan, mhc_stats* out);
+
+/*
+ * How the plan's correlator calls run on the current device, for inspection, launch counts
+ * and tests.  The plan's device tables must be there (any device call uploads them), else
+ * MHC_EINVAL.  Waits for the stream.
+ */
+mhc_status mhc_forward_info(mhc_plan_t plan, mhc_forward_path* out, mhc_stream_t stream);
 
 /*
  * Export the work families (host; for inspection and tests).  Pass NULL for the

@@ -85,6 +85,8 @@ static cudaError_t launch_fwd_items(const FwdArgs& a, int ncmax, int tile, int64
 constexpr int kFoldPerThread = 16;
 cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
                            size_t smem, double* out, cudaStream_t s) {
+bool forward_folds(int64_t items, int tile) { return items <= (int64_t)kFoldPerThread * tile; }
+
   cudaError_t e = launch_fxprep(a, s);
   if (e != cudaSuccess) return e;
   if (a.snk_orig) {  // two-sided update: the LU factors of every (family, sink family) block first
@@ -98,7 +100,7 @@ cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam,
     if (e != cudaSuccess) return e;
   }
   FwdArgs fa = a;
-  fa.fold_items = items <= (int64_t)kFoldPerThread * tile ? items : 0;
+  fa.fold_items = forward_folds(items, tile) ? items : 0;
   fa.out = out;
   {
     TraceRange trace("forward kernel");

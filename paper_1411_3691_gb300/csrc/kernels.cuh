@@ -377,6 +377,7 @@ cudaError_t launch_reduce(const FwdArgs& a, int64_t items, double* out, cudaStre
 cudaError_t launch_pairs(const FwdArgs& a, int ncmax, int64_t n_pairs, int64_t n_src,
                          const int64_t* ii, const int64_t* jj, const int32_t* src_member,
                          const int32_t* mem_family, double* dets, int32_t* path, cudaStream_t s);
+bool forward_folds(int64_t items, int tile);
 size_t forward_smem_bytes(int slots, int tile, int ncmax);
 #define MHC_DECL_NC(NC)                                                                       \
   cudaError_t launch_fwd_nc##NC(const FwdArgs& a, int tile, int64_t items, size_t smem,       \

@@ -342,6 +342,32 @@ mhc_status mhc_correlator(mhc_plan_t plan, const double* const* S_f, const doubl
   return MHC_OK;
 }
 
+mhc_status mhc_forward_info(mhc_plan_t plan, mhc_forward_path* out, mhc_stream_t stream) {
+  if (!plan || !out) {
+    set_error("mhc_forward_info: NULL plan or output");
+    return MHC_EINVAL;
+  }
+  Plan& p = *reinterpret_cast<Plan*>(plan);
+  int cur = 0;
+  MHC_CUDA(cudaGetDevice(&cur));
+  if (p.dev.device != cur) {
+    set_error("mhc_forward_info: the plan's tables are not on the current device yet; call "
+              "mhc_correlator with it first");
+    return MHC_EINVAL;
+  }
+  MHC_CUDA(cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(stream)));
+  fx::Tables t;
+  *out = mhc_forward_path();
+  out->tables = p.dev.fx ? 1 : 0;
+  out->tables_used = out->tables;
+  out->table_bytes = p.dev.fx ? (int64_t)fx_layout(p, nullptr, &t) : 0;
+  out->folded_sum = forward_folds(p.dev.n_items, p.dev.tile) ? 1 : 0;
+  const int kfac = p.dev.two_sided ? 1 + (p.max_n > 6 ? 1 : 0) : 0;
+  const int fwd = p.dev.fam_order ? p.dev.n_ranges : 1;
+  out->launches = out->tables + kfac + fwd + 1 - out->folded_sum;
+  return MHC_OK;
+}
+
 mhc_status mhc_correlator_cw(mhc_plan_t plan, const double* const* S_f, const double* w_src_re,
                              const double* w_src_im, const double* w_snk_re, const double* w_snk_im,
                              double* out_dev, mhc_stream_t stream) {

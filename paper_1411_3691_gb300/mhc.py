@@ -27,7 +27,7 @@ MHC_NMAX = 32
 MHC_FMAX = 8
 
 EXPORTED = ["mhc_last_error", "mhc_plan_opts_default", "mhc_plan", "mhc_plan_destroy",
-            "mhc_plan_stats", "mhc_plan_families", "mhc_plan_sinks", "mhc_correlator", "mhc_correlator_noalloc",
+            "mhc_plan_stats", "mhc_forward_info", "mhc_plan_families", "mhc_plan_sinks", "mhc_correlator", "mhc_correlator_noalloc",
             "mhc_correlator_cw",
             "mhc_correlator_backward",
             "mhc_pair_dets", "mhc_get_status", "mhc_batch_create", "mhc_batch_destroy",
@@ -65,6 +65,11 @@ class Stats(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_ if k != "reserved"}
 
 
+class ForwardPath(ctypes.Structure):
+    _fields_ = [("tables", ctypes.c_int32), ("tables_used", ctypes.c_int32), ("folded_sum", ctypes.c_int32),
+                ("launches", ctypes.c_int32), ("table_bytes", ctypes.c_int64)]
+
+
 _lib = None
 _vp = ctypes.c_void_p
 _i32p = ctypes.POINTER(ctypes.c_int32)
@@ -87,6 +92,7 @@ def lib():
         L.mhc_plan_destroy.argtypes = [_vp]
         L.mhc_plan_destroy.restype = None
         L.mhc_plan_stats.argtypes = [_vp, ctypes.POINTER(Stats)]
+        L.mhc_forward_info.argtypes = [_vp, ctypes.POINTER(ForwardPath), _vp]
         L.mhc_plan_families.argtypes = [_vp, _i64p, _i64p, _i32p, _i32p, _i32p, _i64p, _i32p, _i32p]
         L.mhc_plan_sinks.argtypes = [_vp, _i64p, _i32p, _i32p, _i32p, _i32p, _i32p]
         L.mhc_correlator.argtypes = [_vp, ctypes.POINTER(_vp), _vp, _vp, _vp, _vp]
@@ -180,6 +186,14 @@ def mhc_plan_stats(plan) -> dict:
     s = Stats()
     _check(lib().mhc_plan_stats(_vp(plan), ctypes.byref(s)))
     return s.as_dict()
+
+
+def mhc_forward_info(plan, stream=None) -> dict:
+    """How the plan's correlator calls run (after a first one): tables, tables_used, folded_sum,
+    launches, table_bytes."""
+    s = ForwardPath()
+    _check(lib().mhc_forward_info(_vp(plan), ctypes.byref(s), _stream(stream)))
+    return {k: getattr(s, k) for k, _ in s._fields_}
 
 
 def mhc_plan_families(plan, F: int, Tn: int, n_src: int) -> dict:
@@ -363,6 +377,9 @@ class Plan:
 
     def stats(self):
         return mhc_plan_stats(self.handle)
+
+    def forward_info(self, stream=None):
+        return mhc_forward_info(self.handle, stream)
 
     def families(self):
         return mhc_plan_families(self.handle, self.F, self.Tn, self.n_src)

@@ -155,7 +155,6 @@ BatchShape make_shape(const mhc_batch_s& b, const int (&Tc)[kClasses]) {
   };
   std::vector<Cost> all[kClasses];
   sh.part_off.push_back(0);
-  int max_slots[kClasses] = {1, 1, 1};
   for (int k = 0; k < b.count; k++) {
     const Plan& p = *b.plans[k];
     const int cl = class_of(p);
@@ -165,7 +164,7 @@ BatchShape make_shape(const mhc_batch_s& b, const int (&Tc)[kClasses]) {
     sh.ncmax = std::max(sh.ncmax, plan_ncmax(p));
     int yoff[MHC_FMAX], slots = 0;
     plan_slots(p, yoff, &slots);
-    max_slots[cl] = std::max(max_slots[cl], slots);
+    sh.cls_smem[cl] = std::max(sh.cls_smem[cl], forward_smem_bytes(slots, T, kClassNc[cl], p.dev.fx || b.own_fx[k]));
     for (int64_t W = 0; W < p.n_fam; W++) {
       double c = 0.0;
       const double kW = (double)(p.fam_off[W + 1] - p.fam_off[W]);
@@ -188,7 +187,6 @@ BatchShape make_shape(const mhc_batch_s& b, const int (&Tc)[kClasses]) {
     for (auto& x : all[c]) sh.items.push_back(x.it);
     const int64_t n = (int64_t)all[c].size();
     if (n == 0) continue;
-    sh.cls_smem[c] = forward_smem_bytes(max_slots[c], Tc[c], kClassNc[c]);
     const int occ = c == 0 ? batch_occupancy_nc8(Tc[c], sh.cls_smem[c])
                            : (c == 1 ? batch_occupancy_nc18(Tc[c], sh.cls_smem[c])
                                      : batch_occupancy_nc32(Tc[c], sh.cls_smem[c]));

@@ -48,11 +48,13 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const double2* _
 
 }  // namespace
 
-size_t forward_smem_bytes(int slots, int tile, int ncmax) {
+// tables: the launch's work items may use fixed-point tables (their warps' scratch is larger)
+size_t forward_smem_bytes(int slots, int tile, int ncmax, bool tables) {
   const size_t cache = (size_t)slots * tile * sizeof(double2);
-  const size_t scratch = ncmax <= 8 ? WarpScratch<8>::kBytes : ncmax <= 18 ? WarpScratch<18>::kBytes : WarpScratch<32>::kBytes;
-  const size_t labels = (size_t)(slots + MHC_FMAX) * tile * sizeof(short);  // fwd::FxLane
-  return cache + (size_t)(tile / 32) * scratch + labels;
+  const size_t scratch = ncmax <= 8    ? WarpScratch<8>::bytes(slots, tables)
+                         : ncmax <= 18 ? WarpScratch<18>::bytes(slots, tables)
+                                       : WarpScratch<32>::bytes(slots, tables);
+  return cache + (size_t)(tile / 32) * scratch;
 }
 
 // fwd_kernel over items [0, items): one launch per layout range, each with its own y
@@ -72,7 +74,7 @@ static cudaError_t launch_fwd_items(const FwdArgs& a, int ncmax, int tile, int64
     ar.slots = g.slots;
     for (int f = 0; f < MHC_FMAX; f++) ar.yoff[f] = g.yoff[f];
     ar.item0 = g.first * a.n_tiles;
-    const cudaError_t e = one(ar, g.count * a.n_tiles, forward_smem_bytes(g.slots, tile, ncmax));
+    const cudaError_t e = one(ar, g.count * a.n_tiles, forward_smem_bytes(g.slots, tile, ncmax, a.fx.nf > 0));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -83,10 +85,10 @@ static cudaError_t launch_fwd_items(const FwdArgs& a, int ncmax, int tile, int64
 // blocks: 512 x 512 terms (444 blocks of 128 threads, one wave) 8 us faster, 1291 x 977 (1600) 1 us
 // faster, 1944 x 1944 10 us and 4096 x 4096 terms (8192 blocks) 23 us slower.
 constexpr int kFoldPerThread = 16;
-cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
-                           size_t smem, double* out, cudaStream_t s) {
 bool forward_folds(int64_t items, int tile) { return items <= (int64_t)kFoldPerThread * tile; }
 
+cudaError_t launch_forward(const FwdArgs& a, int ncmax, int tile, int64_t n_fam, int64_t items,
+                           size_t smem, double* out, cudaStream_t s) {
   cudaError_t e = launch_fxprep(a, s);
   if (e != cudaSuccess) return e;
   if (a.snk_orig) {  // two-sided update: the LU factors of every (family, sink family) block first

@@ -256,6 +256,9 @@ __device__ __forceinline__ bool fx_block(const FwdArgs& a, int W, int Q, int f, 
          !a.kguard[((int64_t)W * a.n_q + Q) * a.F + f];
 }
 
+// where the solves' exponents of flavour f start (WarpScratch)
+__device__ __forceinline__ int fx_at(const FwdArgs& a, int f) { return f == a.fx.f0 ? 0 : 32; }
+
 // complex factor of a flavour's fixed-point solve: det B of a block solved in fixed point, sd of
 // a two-row family, else 1
 __device__ __forceinline__ dev::cd fx_factor(const FwdArgs& a, int W, int Q, int f, bool blk, const double2* Yf, int T) {
@@ -305,7 +308,7 @@ __device__ __forceinline__ void refactor_pairs(const FwdArgs& a, int W, bool hav
       int ys = T;
       if constexpr (FX) {
         if (fxm) {
-          const int e2 = eyw[f * T + e.lane], eq = e2 >> 1;
+          const int e2 = eyw[fx_at(a, f) + e.lane], eq = e2 >> 1;
           const double2 fac = fx_factor(a, W, Q, f, e2 & 1, Yf, T);
           for (int q = 0; q < rho * n; q++) {
             yl[q] = fx::value(reinterpret_cast<const int4*>(Yf)[q * T], eq);
@@ -400,19 +403,10 @@ __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int
 
 // ---- solves and member dots in fixed point (fx.cuh) -------------------------------------
 // The warp's cached solves are fixed-point vectors in the y cache (rank 1: the n entries of y up
-// to a complex factor; rank 2: the 2 n entries of z1 and z2, sd stays FP64), with the vector's
-// exponent per flavour and lane beside the column labels.
-struct FxLane {
-  unsigned short* lab;  // [slot][T] column labels, at the lane
-  short* ey;            // [F][T] 2 e_y (an entry of 2^56 stands for 2^e_y), + 1 when the block's det B is a factor
-};
-template <int NCMAX>
-__device__ __forceinline__ FxLane fx_lane(const FwdArgs& a, double2* smem, int T) {
-  char* base = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)(T >> 5) * WarpScratch<NCMAX>::kBytes;
-  unsigned short* lab = reinterpret_cast<unsigned short*>(base);
-  short* ey = reinterpret_cast<short*>(lab + (size_t)a.slots * T);
-  return FxLane{lab, ey};
-}
+// to a complex factor; rank 2: the 2 n entries of z1 and z2, sd stays FP64).  In its scratch
+// (WarpScratch): the column labels, [slot][lane], from the start of the member loop; the solves'
+// exponents (fx_at), [flavour][lane]: 2 e_y (an entry of 2^56 stands for 2^e_y), + 1 when the block's
+// det B is a factor.
 
 // Solve of one flavour in fixed point; false: the lane takes the FP64 factorisation.  Ks: the
 // block's factors staged in shared memory, or null.
@@ -513,7 +507,7 @@ __device__ __forceinline__ void fx_dots(int n, const int4* const (&r)[kN], const
   fx::Acc s[kN];
 #pragma unroll 1
   for (int q = 0; q < n; q++) {
-    const int o = lab[q * T];
+    const int o = lab[q * 32];
     const int4 y = Y[q * T];
 #pragma unroll
     for (int k = 0; k < kN; k++) fx::mac(s[k], __ldg(r[k] + o), y);
@@ -529,7 +523,7 @@ __device__ __forceinline__ fx::Val fx_det2(int n, const int4* __restrict__ r1, c
   fx::Acc s11, s12, s21, s22;
 #pragma unroll 1
   for (int q = 0; q < n; q++) {
-    const int o = lab[q * T];
+    const int o = lab[q * 32];
     const int4 z1 = Y[q * T], z2 = Y[(n + q) * T];
     const int4 a = __ldg(r1 + o), b = __ldg(r2 + o);
     fx::mac(s11, a, z1);
@@ -596,17 +590,17 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   const bool qtwo = Q >= 0 && a.q_two[Q];
   const int mem0 = a.fam_info[4 * W], kW = a.fam_info[4 * W + 1];
   using WS = WarpScratch<NCMAX>;
-  char* scratch = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)warp * WS::kBytes;
+  char* scratch = reinterpret_cast<char*>(smem + (size_t)a.slots * T) + (size_t)warp * WS::bytes(a.slots, a.fx.nf > 0);
   QEntry* queue = reinterpret_cast<QEntry*>(scratch);
   double2* Y = smem + tid;
   const double2* Yw = smem + (tid & ~31);  // the warp's cached solves (lane l: Yw + l)
 
   // ---- per flavour: solve, or factorise the shared rows, for this sink ----------------
   constexpr bool kFx = FX, kCw = kComplexWeights<NCMAX, FX>;
-  const FxLane fl = fx_lane<NCMAX>(a, smem, T);
+  unsigned short* lab = reinterpret_cast<unsigned short*>(scratch + WS::kQueue + WS::kWalk) + lane;
+  short* eyw = reinterpret_cast<short*>(scratch + WS::exponents(a.slots));
   bool fxm = kFx && a.fx.nf > 0 && kW <= fx::kMaxMembers, bad = false;
   for (int f = 0; f < a.F; f++) fxm &= a.fam_rank[(int64_t)W * a.F + f] <= 2;
-  const short* eyw = fl.ey + (tid & ~31);
   // flavours solved in fixed point; left to the FP64 factorisation; FP64 solves converted
   unsigned infx = 0, solo = 0, made = 0;
   unsigned pguard = 0;
@@ -624,7 +618,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       const bool blk = fx_block(a, W, Q, f, qtwo);
       const int4* Ks = __any_sync(0xffffffffu, blk) ? fx_stage<NCMAX>(a, W, Q, f, lane, scratch) : nullptr;
       if (blk) {
-        done = fx_solve(a, W, Q, f, cols + a.off_f[f], Ks, Yf, T, fl.ey + f * T + tid);
+        done = fx_solve(a, W, Q, f, cols + a.off_f[f], Ks, Yf, T, eyw + fx_at(a, f) + lane);
         if (done) infx |= 1u << f; else solo |= 1u << f;
       }
     }
@@ -645,7 +639,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         pguard |= (unsigned)g << f;
       }
       if constexpr (kFx) {
-        if (fxm && fx_from_fp64(n, rho, Yf, T, ey, fl.ey + f * T + tid)) made |= 1u << f;
+        if (fxm && fx_from_fp64(n, rho, Yf, T, ey, eyw + fx_at(a, f) + lane)) made |= 1u << f;
         bad |= fxm && !((made >> f) & 1);
       }
     }
@@ -658,19 +652,19 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   double2 lf = make_double2(1.0, 0.0);  // their factors
   if constexpr (kFx) {
     const bool keep = fxm && !__any_sync(0xffffffffu, bad || pguard != 0);
+    __syncwarp();  // the labels lie where the solves read the staged block factors
     for (int f = 0; f < a.F; f++) {
       const int n = a.n_f[f];
       if (n == 0) continue;
       const int rho = a.fam_rank[(int64_t)W * a.F + f];
       double2* Yf = Y + (size_t)a.yoff[f] * T;
-      const int e = fl.ey[f * T + tid] >> 1;
       const bool blk = (infx >> f) & 1;
       if (keep) {
         lf = dev::cmul(lf, fx_factor(a, W, Q, f, blk, Yf, T));
-        le += rho * e + (rho == 2);  // fx::mul halves
-        for (int q = 0; q < n; q++) fl.lab[(size_t)(a.yoff[f] + q) * T + tid] = (unsigned short)cols[a.off_f[f] + q];
+        le += rho * (eyw[fx_at(a, f) + lane] >> 1) + (rho == 2);  // fx::mul halves
+        for (int q = 0; q < n; q++) lab[(a.yoff[f] + q) * 32] = (unsigned short)cols[a.off_f[f] + q];
       } else if (blk || ((made >> f) & 1)) {
-        fx_to_fp64(n, rho, Yf, T, e, fx_factor(a, W, Q, f, blk, Yf, T));
+        fx_to_fp64(n, rho, Yf, T, eyw[fx_at(a, f) + lane] >> 1, fx_factor(a, W, Q, f, blk, Yf, T));
         eys.set(f, dev::cached_scale(Yf, T, n, rho));
       }
     }
@@ -683,9 +677,9 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   // (two-row families need n_f >= 10: the classes below compile none of this)
   constexpr bool kZ1 = NCMAX >= 10;
   int zf0 = -1, zf1 = -1;
-  double2* z1d = reinterpret_cast<double2*>(scratch + WS::kQueue);
+  double2* z1d = reinterpret_cast<double2*>(scratch + WS::kQueue + WS::kWalk);
   // the warp's scratch for the grouped refactors' multipliers (group_fresh)
-  double2* wk = reinterpret_cast<double2*>(scratch + WS::kQueue + WS::kZ1);
+  double2* wk = reinterpret_cast<double2*>(scratch + WS::kQueue);
   // (the shuffle and the vote run on every lane: qtwo differs between lanes whose sinks
   // belong to a two-sided family and lanes whose sinks stand alone)
   const int Q0 = kZ1 ? __shfl_sync(0xffffffffu, Q, 0) : 0;
@@ -737,7 +731,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       if constexpr (kFx) {
         if (fxm) {
           d = fx_member64(a.S[f], a.L_f[f], n, rho, mlab, cols + a.off_f[f], reinterpret_cast<const int4*>(Yf), T,
-                          fl.ey[f * T + tid] >> 1, fx_factor(a, W, Q, f, (infx >> f) & 1, Yf, T), a.kc, &cf);
+                          eyw[fx_at(a, f) + lane] >> 1, fx_factor(a, W, Q, f, (infx >> f) & 1, Yf, T), a.kc, &cf);
           fixed = true;
         }
       }
@@ -836,7 +830,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           const int n = a.n_f[f], L = a.L_f[f];
           if (n == 0) continue;
           const int rho = a.fam_rank[(int64_t)W * a.F + f];
-          const unsigned short* lb = fl.lab + (size_t)a.yoff[f] * T + tid;
+          const unsigned short* lb = lab + a.yoff[f] * 32;
           const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
           fx::Val v[kN];
           const int4* r[kN];

@@ -347,11 +347,14 @@ struct BatchItem {
   int32_t corr, W, tile, pad;
 };
 
-// Per-warp scratch of the forward kernel, by n class: the refactor queue; a store of the members'
-// dots with a block's first null vector (rank-2 families against one-column sink families: two
-// flavours, 32 members, two complex values); the multipliers of a grouped refactor's shared
-// elimination by step, packed (n - 1 + n - 2 + ... + 1 complex values for n <= 18).  Before the
-// member loop the whole of it holds the block factors of the warp's sinks (fwd::fx_stage).
+// Per-warp scratch of the forward kernel, by n class: the refactor queue; the multipliers of a grouped
+// refactor's shared elimination by step, packed (n - 1 + n - 2 + ... + 1 complex values for n <= 18); a
+// store of the members' dots with a block's first null vector (rank-2 families against one-column sink
+// families: two flavours, 32 members, two complex values).  With fixed-point tables the sinks' column
+// labels (2 bytes per slot and lane) lie over that store, which only FP64 dots use, and the solves'
+// exponents of two flavours behind it: 384 bytes more per warp for two flavours of n = 18, and none
+// for a launch without tables.  Before the member loop the first kBytes hold the block factors of the
+// warp's sinks (fwd::fx_stage).
 constexpr int kQueueCap = 64;         // entries per warp
 constexpr int kQueueEntryBytes = 48;  // sizeof(fwd::QEntry)
 constexpr int kZ1Flavours = 2;
@@ -361,7 +364,14 @@ struct WarpScratch {
   static constexpr int kQueue = kQueueCap * kQueueEntryBytes;
   static constexpr int kZ1 = NCMAX <= 8 ? 0 : kZ1Flavours * 32 * 2 * 16;
   static constexpr int kWalk = kWalkMaxN * (kWalkMaxN - 1) / 2 * 16;
-  static constexpr int kBytes = kQueue + kZ1 + kWalk;
+  static constexpr int kBytes = kQueue + kWalk + kZ1;
+  // offset of the exponents behind the labels of `slots` y-cache slots
+  __host__ __device__ static constexpr int exponents(int slots) {
+    return kQueue + kWalk + (slots * 64 > kZ1 ? slots * 64 : kZ1);
+  }
+  __host__ __device__ static constexpr int bytes(int slots, bool tables) {
+    return tables ? exponents(slots) + 2 * 32 * (int)sizeof(short) : kBytes;
+  }
 };
 
 constexpr int kReduceMaxBlocks = 128;
@@ -378,7 +388,7 @@ cudaError_t launch_pairs(const FwdArgs& a, int ncmax, int64_t n_pairs, int64_t n
                          const int64_t* ii, const int64_t* jj, const int32_t* src_member,
                          const int32_t* mem_family, double* dets, int32_t* path, cudaStream_t s);
 bool forward_folds(int64_t items, int tile);
-size_t forward_smem_bytes(int slots, int tile, int ncmax);
+size_t forward_smem_bytes(int slots, int tile, int ncmax, bool tables);
 #define MHC_DECL_NC(NC)                                                                       \
   cudaError_t launch_fwd_nc##NC(const FwdArgs& a, int tile, int64_t items, size_t smem,       \
                                 cudaStream_t s);                                              \

@@ -101,7 +101,7 @@ extern "C" mhc_status mhc_correlator_noalloc(mhc_plan_t plan, const double* cons
   // Every work item writes its own slot before the reduction reads it, so the array
   // needs no clearing between calls.
   a.partials = scratch;
-  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p));
+  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p), a.fx.nf > 0);
   cudaError_t e = launch_forward(a, plan_ncmax(p), tile, p.n_fam, items, smem, out_dev,
                                  reinterpret_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) {

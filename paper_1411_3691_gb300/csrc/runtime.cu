@@ -336,7 +336,7 @@ mhc_status mhc_correlator(mhc_plan_t plan, const double* const* S_f, const doubl
   FwdArgs a;
   if ((st = fill_fwd_args(p, S_f, w_src_dev, w_snk_dev, a)) != MHC_OK) return st;
   const int tile = p.dev.tile;
-  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p));
+  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p), a.fx.nf > 0);
   MHC_CUDA(launch_forward(a, plan_ncmax(p), tile, p.n_fam, p.dev.n_items, smem, out_dev,
                           reinterpret_cast<cudaStream_t>(stream)));
   return MHC_OK;
@@ -383,7 +383,7 @@ mhc_status mhc_correlator_cw(mhc_plan_t plan, const double* const* S_f, const do
   a.w_src_im = w_src_im;
   a.w_snk_im = w_snk_im;
   const int tile = p.dev.tile;
-  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p));
+  const size_t smem = forward_smem_bytes(a.slots, tile, plan_ncmax(p), a.fx.nf > 0);
   MHC_CUDA(launch_forward(a, plan_ncmax(p), tile, p.n_fam, p.dev.n_items, smem, out_dev,
                           reinterpret_cast<cudaStream_t>(stream)));
   return MHC_OK;

@@ -48,7 +48,11 @@ __device__ __forceinline__ int expo(cd z) { return max(expo(z.x), expo(z.y)); }
 // with the PTX approximate reciprocal; two steps reach full double precision.
 __device__ __forceinline__ double rcp_nr(double d) {
   double r;
+#ifdef __CUDA_ARCH__
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+#else
+  r = 1.0 / d;  // the host tests of this arithmetic
+#endif
   double e = fma(-d, r, 1.0);
   r = fma(r, e, r);
   e = fma(-d, r, 1.0);
@@ -69,6 +73,7 @@ __device__ __forceinline__ cd ldS(const cd* __restrict__ p) { return __ldg(p); }
 namespace fx {
 __device__ __forceinline__ int4 factor_limbs(dev::cd z, int e);
 __device__ __forceinline__ bool exponents_ok(int eu, int er);
+__device__ __forceinline__ bool block_fits(int lo, int hi);
 }  // namespace fx
 
 namespace dev {
@@ -667,12 +672,23 @@ __device__ __forceinline__ bool kfac_block(const cd* __restrict__ S, int L, int 
   const int C = RHO == 2 ? M + 1 : M;  // columns kept
   cd B[MC][MC + 1];
   int perm[MC];
+  int rlo = 4096, rhi = -4096;  // exponents of the rows
+  int ce[MC + 1];               // and of the columns
+#pragma unroll UNR
+  for (int u = 0; u < C; u++) ce[u] = -4096;
 #pragma unroll UNR
   for (int i = 0; i < M; i++) {
     perm[i] = i;
     const cd* row = S + (size_t)arow[i] * L;
+    int e = -4096;
 #pragma unroll UNR
-    for (int u = 0; u < C; u++) B[i][u] = ldS(row + scol[u]);
+    for (int u = 0; u < C; u++) {
+      B[i][u] = ldS(row + scol[u]);
+      e = max(e, expo(B[i][u]));
+      ce[u] = max(ce[u], expo(B[i][u]));
+    }
+    rlo = min(rlo, e);
+    rhi = max(rhi, e);
   }
   int parity = 0, emin = 4096, emax = -4096;
   bool zero = false;
@@ -715,6 +731,13 @@ __device__ __forceinline__ bool kfac_block(const cd* __restrict__ S, int L, int 
   if (M > 0 && (zero || emax - emin > kp)) return true;
   const cd sd = parity ? cneg(det) : det;
   if (fxf && RHO == 1) {  // the same factors as limbs (fx.cuh, solve)
+    int clo = 4096, chi = -4096;
+#pragma unroll UNR
+    for (int u = 0; u < C; u++) {
+      clo = min(clo, ce[u]);
+      chi = max(chi, ce[u]);
+    }
+    if (!fx::block_fits(rlo, rhi) || !fx::block_fits(clo, chi)) return true;
     int4* X = reinterpret_cast<int4*>(K);
 #pragma unroll UNR
     for (int i = 0; i < M; i++) {
@@ -984,6 +1007,25 @@ __device__ __forceinline__ bool group_kfac_block(const cd* __restrict__ S, int L
     Bs[i * P + u] = ldS(S + (size_t)arow[i] * L + scol[u]);
   }
   __syncwarp(gm);
+  if (fxf) {  // exponents of the rows, then of the columns
+    for (int t = 0; t < 2; t++) {
+      const int outer = t ? C : M, inner = t ? M : C, so = t ? 1 : P, si = t ? P : 1;
+      int lo = 4096, hi = -4096;
+      for (int i = g; i < outer; i += G) {
+        int e = -4096;
+        for (int u = 0; u < inner; u++) e = max(e, expo(Bs[i * so + u * si]));
+        lo = min(lo, e);
+        hi = max(hi, e);
+      }
+#pragma unroll
+      for (int off = 1; off < G; off <<= 1) {
+        lo = min(lo, __shfl_xor_sync(gm, lo, off));
+        hi = max(hi, __shfl_xor_sync(gm, hi, off));
+      }
+      if (!fx::block_fits(lo, hi)) return true;
+    }
+    __syncwarp(gm);
+  }
   cd det;
   int parity;
   if (group_lu<G>(Bs, P, Ps, M, C, M, g, gm, kp, &det, &parity)) return true;

@@ -412,47 +412,17 @@ __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int
 // block's factors staged in shared memory, or null.
 __device__ __forceinline__ bool fx_solve(const FwdArgs& a, int W, int Q, int f, const int32_t* col, const int4* Ks,
                                          double2* Yf, int T, short* ey) {
-  const int n = a.n_f[f], rho = a.fam_rank[(int64_t)W * a.F + f], M = n - rho;
+  const int n = a.n_f[f], rho = a.fam_rank[(int64_t)W * a.F + f];
   const double2* K = a.kbuf + ((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f];
-  const int4* Kg = reinterpret_cast<const int4*>(K);
-  int4* z = reinterpret_cast<int4*>(Yf) + (rho == 2 ? n * T : 0);
   const int c = col[n - 1], ea = a.fx.cexp[f][c];
-  if (ea > 900 || ea < -900) return false;
-  const int zlo = rho == 2 ? max(0, __ldg(Kg + M * M).w) : 0;
-  int u = zlo - 55, mag = 0;
-  if (M > 0) {
-    const int4* ac = a.fx.sc[f] + c;
-    const bool ok = Ks ? fx::solve<true>(M, ac, ea, zlo, Ks, z, T, &u, &mag)
-                       : fx::solve<false>(M, ac, ea, zlo, Kg, z, T, &u, &mag);
-    if (!ok) return false;
-  }
-  // the unit entries; u >= -55, and an entry 1 below the unit is lost against the others
-  const fx::Val unit{u <= 0 ? 1ll << -u : 0ll, 0ll};
-  const int4 one = fx::limbs(unit), zero = make_int4(0, 0, 0, 0);
-  mag = max(mag, fx::magnitude(unit));
-  if (rho == 2) {
-    z[M * T] = zero;
-    z[(M + 1) * T] = one;
-    int4* z1 = reinterpret_cast<int4*>(Yf);
-    for (int q = 0; q < M; q++) {
-      const int4 v = fx::quant(__ldg(K + M * M + M + q), u + fx::kFracBits, fx::kFracBits);
-      z1[q * T] = v;
-      mag = max(mag, fx::magnitude(fx::joined(v)));
-    }
-    z1[M * T] = one;
-    z1[(M + 1) * T] = zero;
-    Yf[2 * n * T] = __ldg(K + M * M + 2 * M);
-  } else {
-    z[M * T] = one;
-  }
-  // the largest entry just below 2^56 (its bits by the high word: 32 when below 2^32)
-  const int sh = 64 - __clz(mag) - fx::kFracBits;
-  for (int q = 0; q < rho * n; q++) {
-    int4& v = reinterpret_cast<int4*>(Yf)[q * T];
-    const fx::Val x = fx::joined(v);
-    v = fx::limbs(fx::shift(x.re, sh), fx::shift(x.im, sh));
-  }
-  *ey = (short)(2 * (u + sh + fx::kFracBits) + 1);
+  int4* Yx = reinterpret_cast<int4*>(Yf);
+  int e2 = 0;
+  double2 sd;
+  const bool ok = Ks ? fx::solve_sink<true>(n, rho, a.fx.sc[f] + c, ea, Ks, K, Yx, T, &e2, &sd)
+                     : fx::solve_sink<false>(n, rho, a.fx.sc[f] + c, ea, reinterpret_cast<const int4*>(K), K, Yx, T, &e2, &sd);
+  if (!ok) return false;
+  if (rho == 2) Yf[2 * n * T] = sd;
+  *ey = (short)e2;
   return true;
 }
 

@@ -167,24 +167,38 @@ __device__ __forceinline__ Val mul(int4 a, int4 b) {
 // pivoting: |l| <= sqrt 2), row i of U with its own exponent eU_i, the pivot's reciprocal r_i
 // with er_i.  w keeps the unit of a, 2^(ea - 55).  z's unit is chosen per sink so that the largest
 // |r_i w_i| is at 2^54; entries may grow to 2^58 (on random blocks of n = 3 to 18 w grew by at most
-// 2^2 and z by 2^3.5).  Every sum is exact but for the dropped lo lo products, below one unit.  A
-// value above its limit, or a column so far below its exponent that w would keep fewer than 45
-// bits, is reported and the sink takes the one-sided FP64 factorisation, ten times the work: the
-// limits are far from what occurs.  The error against the exact solve is the FP64 one's (both are
-// the factors': mean 1.8e-15 at n = 18, 1.0e-15 at n = 12, of the largest entry).
+// 2^2 and z by 2^3.5).  Every sum is exact but for the dropped lo lo products, below one unit.
+// What one unit for all of a vector costs is bounded by checks; a sink or block that fails one is
+// reported and takes the one-sided FP64 factorisation, ten times the work, so the limits lie where
+// random blocks hardly ever come:
+//   - the rows of a block have exponents within kBlockSpread, and its columns too (block_fits, by the
+//     kfac routines): a row far below the others has its part of a, w and L in that many bits less, and
+//     a column its part of U, against larger entries of z;
+//   - w keeps kMinBits bits (a column far below its exponent), one less where it is a single entry;
+//   - the largest r_i w_i is at least 2^kLeadBits units of w times the largest r_i: one unit of any w_i
+//     moves z by at most 2^-kLeadBits of its largest entry.  product_exponent reads high limbs only;
+//     with this a w_i without one is below 2^-20 of the largest product, and no T overflows;
+//   - nothing grows above its limit.
+// The error against the exact solve is the FP64 one's (both are the factors': mean 1.8e-15 at n = 18,
+// 1.0e-15 at n = 12, of the largest entry).
 //   layout: LU[M][M] limbs (diagonal: r_i) | (S row offset of the row's label, eU_i, er_i, e of
 //           -U1^{-1} u) [M] | ... | -det B | det B (FP64)
 constexpr int kFactBits = 54;
 constexpr int kABits = 55;   // |a| <= 2^55
 constexpr int kZBits = 54;   // the largest |r_i w_i|, within a factor of two
 constexpr int kTopBits = 58;
-constexpr int kMinBits = 45;
+constexpr int kMinBits = 52;
+constexpr int kLeadBits = 47;
+constexpr int kBlockSpread = 3;
 
 __device__ __forceinline__ int4 factor_limbs(dev::cd z, int e) { return quant(z, e, kFactBits); }
 // row i's exponents: normal, and |U_i| / |pivot| within the shifts of sum_shifted
 __device__ __forceinline__ bool exponents_ok(int eu, int er) {
   return eu > -900 && eu < 900 && er > -900 && er < 900 && eu + er <= 20;
 }
+
+// lowest and highest exponent of a block's rows, or columns (each its largest entry's)
+__device__ __forceinline__ bool block_fits(int lo, int hi) { return hi - lo <= kBlockSpread; }
 
 __device__ __forceinline__ int bits(long long x) { return 64 - __clzll(x ^ (x >> 63)); }
 __device__ __forceinline__ Val joined(int4 l) {
@@ -218,7 +232,7 @@ template <bool SM>
 __device__ __forceinline__ bool solve(int M, const int4* __restrict__ a, int ea, int zlo, const int4* __restrict__ K,
                                       int4* Y, int ys, int* unit, int* mag) {
   auto ld = [](const int4* q) { return SM ? *q : __ldg(q); };
-  int mx = -100000, top = 0;
+  int mx = -100000, top = 0, lead = -100000;
   for (int i = 0; i < M; i += 2) {
     const bool two = i + 1 < M;
     const int i1 = two ? i + 1 : i;
@@ -237,6 +251,7 @@ __device__ __forceinline__ bool solve(int M, const int4* __restrict__ a, int ea,
     Y[i * ys] = l0;
     top = max(top, magnitude(w0));
     mx = max(mx, product_exponent(l0, ld(k0 + i), t0.z));
+    lead = max(lead, max(t0.z, t1.z));
     if (two) {
       mac(s1, ld(k1 + i), l0);
       const Val q1 = sum_shifted(s1, 1), w1{a1.re - q1.re, a1.im - q1.im};
@@ -246,7 +261,7 @@ __device__ __forceinline__ bool solve(int M, const int4* __restrict__ a, int ea,
       mx = max(mx, product_exponent(l1, ld(k1 + i1), t1.z));
     }
   }
-  bool ok = top < kFits && top >= 1 << (kMinBits - 33);
+  bool ok = top < kFits && top >= 1 << (kMinBits - (M > 1 ? 33 : 34)) && mx >= lead + kLeadBits;
   // unit exponent u of z: largest r_i w_i (2^(mx + ea - 55)) at 2^54
   const int u = max(mx + ea - kABits - kZBits, zlo - 55);
   *unit = u;
@@ -290,6 +305,47 @@ __device__ __forceinline__ bool solve(int M, const int4* __restrict__ a, int ea,
   }
   *mag = top;
   return ok && max(over, top) < kFits;
+}
+
+// One sink's solve from its block's factors: z in Y (rank 1: n entries, the last 1; rank 2: z1 and z2),
+// scaled so that the largest entry just fills 2^56.  F: the block's limbs (staged when SM), K: the same
+// block in global memory, for its FP64 entries.  *e2: 2 e_y + 1 (an entry of 2^56 stands for 2^e_y; det
+// B is a factor); *sd: rank 2, the FP64 factor.
+template <bool SM>
+__device__ __forceinline__ bool solve_sink(int n, int rho, const int4* __restrict__ a, int ea, const int4* __restrict__ F,
+                                           const dev::cd* __restrict__ K, int4* Y, int ys, int* e2, dev::cd* sd) {
+  const int M = n - rho;
+  if (ea > 900 || ea < -900) return false;
+  int4* z = Y + (rho == 2 ? n * ys : 0);
+  const int zlo = rho == 2 ? max(0, __ldg(reinterpret_cast<const int4*>(K) + M * M).w) : 0;
+  int u = zlo - 55, mag = 0;
+  if (M > 0 && !solve<SM>(M, a, ea, zlo, F, z, ys, &u, &mag)) return false;
+  // the unit entries; u >= -55, and an entry 1 below the unit is lost against the others
+  const Val unit{u <= 0 ? 1ll << -u : 0ll, 0ll};
+  const int4 one = limbs(unit), zero = make_int4(0, 0, 0, 0);
+  mag = max(mag, magnitude(unit));
+  if (rho == 2) {
+    z[M * ys] = zero;
+    z[(M + 1) * ys] = one;
+    for (int q = 0; q < M; q++) {
+      const int4 v = quant(__ldg(K + M * M + M + q), u + kFracBits, kFracBits);
+      Y[q * ys] = v;
+      mag = max(mag, magnitude(joined(v)));
+    }
+    Y[M * ys] = one;
+    Y[(M + 1) * ys] = zero;
+    *sd = __ldg(K + M * M + 2 * M);
+  } else {
+    z[M * ys] = one;
+  }
+  // the largest entry just below 2^56 (its bits by the high word: 32 when below 2^32)
+  const int sh = 64 - __clz(mag) - kFracBits;
+  for (int q = 0; q < rho * n; q++) {
+    const Val x = joined(Y[q * ys]);
+    Y[q * ys] = limbs(shift(x.re, sh), shift(x.im, sh));
+  }
+  *e2 = 2 * (u + sh + kFracBits) + 1;
+  return true;
 }
 
 // Tables of one plan for one set of propagators and weights, rebuilt by every call.

@@ -1,0 +1,37 @@
+"""The arithmetic of csrc/fx.cuh on the host (tests/fixed_point_host.cpp compiles it with a C++ compiler),
+against long double and beside the FP64 path, over propagators whose rows and columns differ in size and
+tolerances that let every pivot pass."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no host C++ compiler")
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("fx") / "fixed_point_host")
+    subprocess.run(["g++", "-O2", "-w", "-std=c++17", "-I", os.path.join(HERE, "host_stub"), "-o", exe,
+                    os.path.join(HERE, "fixed_point_host.cpp")], check=True)
+
+    def run(*args):
+        out = subprocess.run([exe, *map(str, args)], check=True, capture_output=True, text=True).stdout
+        return [float(x) for x in out.split()]
+
+    return run
+
+
+@pytest.mark.parametrize("pivots", [13, 4096])  # the default pivot guard, and none
+@pytest.mark.parametrize("pattern, spread", [("rows", 0), ("rows", 4), ("rows", 10), ("rows", 30), ("cols", 4),
+                                             ("cols", 20), ("both", 4), ("onerow", 8), ("onecol", 8), ("onecol", 30)])
+@pytest.mark.parametrize("n", [2, 3, 6, 12, 18])
+def test_solves(host, n, pattern, spread, pivots):
+    """An accepted solve has a unit in 2^55 times a spread of 2^3 at every place where FP64 has one in
+    2^53: four times the error, and sixteen in the extremes, where a small w meets a large pivot (2^-47)."""
+    blocks, refused, sinks, left, med, worst, med64, worst64 = host(n, pattern, spread, pivots)
+    assert med <= 4 * med64 + 2.0 ** -53 and worst <= 16 * worst64 + 2.0 ** -47
+    if spread == 0:
+        assert refused <= 0.01 * blocks and left <= 0.05 * sinks

@@ -769,25 +769,32 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   } else {
     // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
     fx::Acc2 tot;
-    auto flush = [&]() {
+    auto add = [&](const fx::Acc2& s, int d) {  // acc += s, d binades below that exponent
       double re, im;
-      int e = a.fx.fexp[W] + le;
+      int e = a.fx.fexp[W] + le - d;
       if (a.fx.nf == 1) {
-        re = (double)tot.rp;
-        im = (double)tot.ih;
+        re = (double)s.rp;
+        im = (double)s.ih;
         e -= fx::kDotBits;
       } else {
         constexpr double k30 = 1073741824.0;
-        re = fma((double)tot.hi_re(), k30, (double)tot.lo_re());
-        im = fma((double)tot.hi_im(), k30, (double)tot.lo_im());
+        re = fma((double)s.hi_re(), k30, (double)s.lo_re());
+        im = fma((double)s.hi_im(), k30, (double)s.lo_im());
         e += 30 - 2 * fx::kSplitBits;
       }
       const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
       acc.x += v.x;
       acc.y += v.y;
-      tot = fx::Acc2();
     };
-    const int thr1 = fx::threshold(a.kc, 1, 0), thr2 = fx::threshold(a.kc, 2, 0);
+    auto term = [&](fx::Acc2& s, fx::Val u, fx::Val t) {  // s += u t; u alone with one flavour
+      if (a.fx.nf == 1) {  // kFlush values below 2^60
+        s.rp += u.re;
+        s.ih += u.im;
+      } else {
+        fx::mac(s, fx::split(u), fx::split(t));
+      }
+    };
+    const int thr1 = fx::threshold(a.kc, 1), thr2 = fx::threshold(a.kc, 2);
     // members four at a time (a step that they do not fill repeats the last one)
     constexpr int kN = 4;
     const int step = fxm ? kN : 1;
@@ -822,27 +829,36 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           const int thr = rho == 2 ? thr2 : thr1;
   #pragma unroll
           for (int k = 0; k < kN; k++) {
-            const int tk = at == 0 ? a.fx.thr[mem0 + min(c + k, kW - 1)] : thr;
-            const bool ok = fx::usable(fx::magnitude(v[k]), tk);
+            const bool ok = fx::usable(fx::magnitude(v[k]), thr);
             u[k] = at == 0 ? v[k] : u[k];
             t[k] = v[k];
             slow[k] = (at > 0 && slow[k]) || !ok;
           }
           at++;
         }
+        unsigned far = 0;  // members that their family's exponent would cost too many bits
   #pragma unroll
         for (int k = 0; k < kN; k++) {
-          if (c + k >= kW) slow[k] = false;
-          const bool use = c + k < kW && !slow[k];
-          const fx::Val uz{use ? u[k].re : 0, use ? u[k].im : 0};
-          if (a.fx.nf == 1) {  // kFlush values below 2^60
-            tot.rp += uz.re;
-            tot.ih += uz.im;
-          } else {
-            fx::mac(tot, fx::split(uz), fx::split(t[k]));
-          }
+          const int d = __ldg(a.fx.shift + mem0 + min(c + k, kW - 1));
+          slow[k] = c + k < kW && (slow[k] || d == fx::kNever);
+          const bool use = c + k < kW && !slow[k] && fx::aligns(d, a.fx.nf);
+          far |= (unsigned)(c + k < kW && !fx::aligns(d, a.fx.nf) && d < fx::kMute) << k;
+          const int du = !use ? 0 : a.fx.nf == 1 ? d : d >> 1, dt = use ? d - du : 0;
+          term(tot, use ? fx::aligned(u[k], du) : fx::Val{0, 0}, fx::aligned(t[k], dt));
         }
-        if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) flush();
+        if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) {
+          add(tot, 0);
+          tot = fx::Acc2();
+        }
+        while (far) {
+          const int k = __ffs(far) - 1;
+          far &= far - 1;
+          const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
+          const fx::Val uk = k == 0 ? u[0] : k == 1 ? u[1] : k == 2 ? u[2] : u[3];
+          fx::Acc2 one;
+          term(one, p ? fx::Val{0, 0} : uk, k == 0 ? t[0] : k == 1 ? t[1] : k == 2 ? t[2] : t[3]);
+          add(one, __ldg(a.fx.shift + mem0 + c + k));
+        }
       }
       // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
   #pragma unroll 1

@@ -33,8 +33,10 @@ constexpr int kRowBits = 55;            // a propagator row: |entry| <= 2^55
 constexpr int kDotBits = 57;            // a dot: 2^57 stands for the product of the scales
 constexpr int kMaxHi = 1 << 28;         // high word of 2^60: a larger dot is not used
 constexpr int kMulHi = 1 << 27;         // high word of 2^59: the largest factor of mul
-constexpr int kNever = 0x7fffffff;      // threshold of a member that the FP64 path evaluates
-constexpr int kMaxAlign = 10;           // most bits a family's common exponent may cost a member
+constexpr int kNever = 0x7fffffff;      // a threshold that no value reaches; Tables::shift: the FP64
+                                        // path evaluates the member
+constexpr int kMute = 0x7ffffffe;       // Tables::shift: the member's weight is zero
+constexpr int kMaxAlign = 4;            // most bits of a dot that its family's common exponent may cost
 constexpr int kFlush = 8;               // members per 64-bit sum of products (Acc2)
 constexpr int kMaxMembers = 64;
 
@@ -61,6 +63,7 @@ __device__ __forceinline__ double pow2(int e) {  // 2^e for normal e, else satur
   return e < -1022 ? 0.0 : __longlong_as_double((long long)min(e + 1023, 2047) << 52);
 }
 __device__ __forceinline__ double scale2(double x, int e) {  // x 2^e without intermediate overflow
+  e = min(e, 2046);  // more is infinite as well, and 0 stays 0
   const int h = e >> 1;
   return x * pow2(h) * pow2(e - h);
 }
@@ -119,16 +122,15 @@ __device__ __forceinline__ bool usable(int mag, int thr, int top = kMaxHi) { ret
 // can fire: |det| < 2^(e(row) + e(y) - kc) with floor exponents, here against exponents above the
 // entries.  Rank 1: e(row) + e(y) <= r + e_y - 2, and a complex factor det B taken out of y moves
 // either side by up to sqrt 2: 2^(57 - 1 - kc) covers both, and one binade more is kept.  Rank 2:
-// two rows and two null vectors, e <= r_1 + r_2 + 2 e_z - 4, with 2^56 for the scales: 2^(53 - kc).  `d`: binades by which a
-// member lies below its family's common exponent.  At least 1: below 2^32 the FP64 path decides.
-__device__ __forceinline__ int threshold(int kc, int rank, int d) {
-  const int t = (rank == 1 ? kDotBits : 53) - 32 - kc - d;
+// two rows and two null vectors, e <= r_1 + r_2 + 2 e_z - 4, with 2^56 for the scales: 2^(53 - kc).
+// At least 1: below 2^32 the FP64 path decides.
+__device__ __forceinline__ int threshold(int kc, int rank) {
+  const int t = (rank == 1 ? kDotBits : 53) - 32 - kc;
   return t >= 28 ? kNever : t <= 0 ? 1 : 1 << t;
 }
 
-// Products of two dots.  A dot's scale is an upper bound that it stays a few binades below, and a
-// member's weight and rows may put it another few below its family's exponent: the product keeps
-// 57 bits of the scale of each factor, and its lo lo terms.  (With 54 bits and without them the
+// Products of two dots.  A dot's scale is an upper bound that it stays a few binades below: the product
+// keeps 57 bits of the scale of each factor, and its lo lo terms.  (With 54 bits and without them the
 // correlator of 1291 x 977 terms of n = 5, 4 was off by 8e-14, against 1.8e-15 in FP64.)
 // Limbs in base 2^30 of value / 2, |value| < 2^60: |hi| <= 2^29, lo in [-2^29, 2^29); kFlush products
 // of four cross terms each stay below 2^63.
@@ -136,6 +138,14 @@ constexpr int kSplitBits = kDotBits - 1;  // 2^56 stands for the scale then
 __device__ __forceinline__ int4 split(Val v) {
   const int rh = (int)((v.re + (1ll << 30)) >> 31), ih = (int)((v.im + (1ll << 30)) >> 31);
   return make_int4(rh, (int)(v.re >> 1) - (rh << 30), ih, (int)(v.im >> 1) - (ih << 30));
+}
+// A member whose product lies d binades below its family's exponent: its two dots shifted by half of d
+// each, a single one by d.  Up to kMaxAlign a dot stays as accurate as FP64 would form it (2^-57 2^4 of the
+// scale, half a unit of it on average); a member further down is summed in FP64 by itself.
+__device__ __forceinline__ bool aligns(int d, int flavours) { return d <= flavours * kMaxAlign; }
+__device__ __forceinline__ Val aligned(Val v, int d) {
+  const long long half = (1ll << d) >> 1;
+  return Val{(v.re + half) >> d, (v.im + half) >> d};
 }
 struct Acc2 : Acc {
   long long qp = 0, qn = 0, qi = 0;  // lo lo
@@ -353,10 +363,11 @@ struct Tables {
   const int4* s[MHC_FMAX];      // [L_f][L_f] propagator rows, each with its own exponent
   const int4* sc[MHC_FMAX];     // [L_f][L_f] the same entries with one exponent per column
   const int* cexp[MHC_FMAX];    // [L_f] that exponent (above every entry of the column)
-  const int4* ws;               // [members][L_f0] first flavour's first member row times the weight
-  const int* thr;               // [members] threshold of the first flavour's value (kNever: the FP64
-                                // path evaluates the member)
-  const int* fexp;              // [W] common exponent of the family's products
+  const int4* ws;               // [members][L_f0] first flavour's first member row times the weight (as
+                                // it is where that is zero), with an exponent of its own
+  const int* shift;             // [members] binades by which the member's product scale lies below its
+                                // family's, or kMute, or kNever
+  const int* fexp;              // [W] exponent of the family's products: its largest member's
   int f0, nf;                   // first flavour with n_f > 0; flavours with n_f > 0 (0: no tables)
 };
 

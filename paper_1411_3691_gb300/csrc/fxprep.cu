@@ -4,10 +4,12 @@
 // One launch.  Blocks [0, sum_f L_f) convert one propagator row each: the row's largest binary
 // exponent, then its entries as limbs, and the limbs of the column of the same label at the
 // column's exponent.  The other blocks take one source family each: a member's first row
-// of the first flavour, times the member's signed weight, is stored at the family's common
-// exponent, so that the member loop sums products of all members in integers.  A member whose
-// weighted rows lie more than kMaxAlign binades below the family's largest, or whose rows or
-// weight are not finite, or zero, is left to the FP64 path.  The work is a pass over 2 F L^2 +
+// of the first flavour, times the member's signed weight, is stored at its own exponent, beside the
+// binades by which the member's product scale lies below its family's largest: by that many the member
+// loop shifts the product before it sums the members in integers (aligning the rows instead would round
+// every entry of a small member, not its product).  A row with a weight of zero is stored as it is: its
+// pairs pass the guards as the others, and count nothing.  A member whose rows or weight are not finite,
+// or whose rows are zero, is left to the FP64 path.  The work is a pass over 2 F L^2 +
 // members L entries (He-4 shapes: 206 000, 3.3 MB written).
 #include "kernels.cuh"
 
@@ -39,7 +41,9 @@ __device__ void prep_row(const FwdArgs& a, int f, int b) {
   }
 }
 
+__device__ __forceinline__ bool is_zero(dev::cd w) { return w.x == 0.0 && w.y == 0.0; }
 __device__ __forceinline__ dev::cd weighted(const FwdArgs& a, dev::cd w, dev::cd z) {
+  if (is_zero(w)) return z;
   return a.w_src_im ? dev::cmul(w, z) : make_double2(w.x * z.x, w.x * z.y);
 }
 
@@ -55,7 +59,7 @@ __device__ void prep_family(const FwdArgs& a, int W) {
     const dev::cd w = dev::source_weight<true>(a, m);
     const int32_t* lab = a.mem_lab + (int64_t)m * a.F * MHC_MAX_RANK;
     int r = 0, e0 = -4096;
-    bool bad = (w.x == 0.0 && w.y == 0.0) || dev::expo(w) >= 1024;
+    bool bad = dev::expo(w) >= 1024;
     for (int f = 0; f < a.F; f++) {
       if (a.n_f[f] == 0) continue;
       for (int t = 0; t < a.fam_rank[(int64_t)W * a.F + f]; t++) {
@@ -82,23 +86,20 @@ __device__ void prep_family(const FwdArgs& a, int W) {
   __syncthreads();
   int X = -100000;
   for (int c = 0; c < kW; c++)
-    if (e0s[c] > -100000) X = max(X, e0s[c] + rest[c]);
+    if (e0s[c] > -100000 && !is_zero(ws[c])) X = max(X, e0s[c] + rest[c]);
   if (threadIdx.x == 0) const_cast<int*>(a.fx.fexp)[W] = X;
   for (int c = warp; c < kW; c += kThreads / 32) {
     const int m = mem0 + c;
     const bool bad = e0s[c] == -100000;
-    const int d = X - e0s[c] - rest[c];  // binades below the family's largest member
-    const bool skip = bad || d > fx::kMaxAlign;
     if (lane == 0)
-      const_cast<int*>(a.fx.thr)[m] = skip ? fx::kNever : fx::threshold(a.kc, a.fam_rank[(int64_t)W * a.F + f0], d);
+      const_cast<int*>(a.fx.shift)[m] = bad ? fx::kNever : is_zero(ws[c]) ? fx::kMute : X - e0s[c] - rest[c];
     const int32_t lab = a.mem_lab[((int64_t)m * a.F + f0) * MHC_MAX_RANK];
     const dev::cd* row = a.S[f0] + (size_t)lab * L0;
     int4* out = const_cast<int4*>(a.fx.ws) + (size_t)m * L0;
-    const int e = X - rest[c];
     for (int l = lane; l < L0; l += 32) {
       dev::cd z = make_double2(0.0, 0.0);
-      if (!skip) z = weighted(a, ws[c], dev::ldS(row + l));
-      out[l] = fx::quant(z, e, fx::kRowBits);
+      if (!bad) z = weighted(a, ws[c], dev::ldS(row + l));
+      out[l] = fx::quant(z, bad ? 0 : e0s[c], fx::kRowBits);
     }
   }
 }

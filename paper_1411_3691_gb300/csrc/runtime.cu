@@ -116,7 +116,7 @@ size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
     return 0;
   }
   t->ws = reinterpret_cast<const int4*>(take((size_t)p.n_src * p.L_f[t->f0] * sizeof(int4)));
-  t->thr = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
+  t->shift = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
   t->fexp = reinterpret_cast<const int*>(take((size_t)p.n_fam * sizeof(int)));
   return off;
 }

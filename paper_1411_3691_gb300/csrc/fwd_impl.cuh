@@ -507,9 +507,31 @@ __device__ __forceinline__ fx::Val fx_det2(int n, const int4* __restrict__ r1, c
   return ok ? fx::Val{p.re - m.re, p.im - m.im} : fx::Val{0, 0};  // half the determinant
 }
 
+// Whether a member's products in a flavour come close to the scale (fx::accepted): rows r1 (and r2
+// against both null vectors: every one of the four dots) and this lane's solve.
+static __device__ __noinline__ bool fx_carries(int n, int rho, const int4* __restrict__ r1, const int4* __restrict__ r2,
+                                               const unsigned short* lab, const int4* Y, int T) {
+  int p11 = 0, p12 = 0, p21 = 0, p22 = 0;
+#pragma unroll 1
+  for (int q = 0; q < n; q++) {
+    const int o = lab[q * 32];
+    const int4 a = __ldg(r1 + o), z = Y[q * T];
+    p11 = max(p11, fx::product_magnitude(a, z));
+    if (rho == 2) {
+      const int4 b = __ldg(r2 + o), z2 = Y[(n + q) * T];
+      p12 = max(p12, fx::product_magnitude(a, z2));
+      p21 = max(p21, fx::product_magnitude(b, z));
+      p22 = max(p22, fx::product_magnitude(b, z2));
+    }
+  }
+  return (rho == 2 ? min(min(p11, p12), min(p21, p22)) : p11) >= fx::kCarries;
+}
+
 // One member's determinant in FP64 from a fixed-point solve, with the FP64 lemma guard: the pairs
-// whose fixed-point value is out of range or near the guard.  The solve's entries carry at least
-// the accuracy of FP64 ones at their largest entry's scale, which is the guard's scale.
+// whose fixed-point value is out of range, too small to be sure of, or near the guard.  The solve's
+// entries carry at least the accuracy of FP64 ones at their largest entry's scale, which is the guard's
+// scale; where every product is far below it and the determinant too, that is not enough, and the pair
+// is refactored (bounds as fx::accepted, with floor exponents).
 static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S, int L, int n, int rho,
                                             const int32_t* __restrict__ lab, const int32_t* __restrict__ col,
                                             const int4* Y, int T, int e, dev::cd factor, int kc, bool* fail) {
@@ -517,31 +539,42 @@ static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S
   dev::cd d = make_double2(0.0, 0.0);
   int eb = -4096, ez = -4096;
   if (rho == 1) {
+    int ep = -8192;
     for (int q = 0; q < n; q++) {
       const dev::cd y = dev::cmul(fx::value(Y[q * T], e), factor), b = dev::ldS(r1 + col[q]);
       ez = max(ez, dev::expo(y));
       eb = max(eb, dev::expo(b));
+      ep = max(ep, dev::expo(y) + dev::expo(b));
       d = dev::cfma(b, y, d);
     }
-    *fail = dev::expo(d) < eb + ez - kc;
+    const int ed = dev::expo(d), es = eb + ez;
+    *fail = ed < es - kc || (ed < es - fx::kFloorBits && ep < es - fx::kCarryBits);
     return d;
   }
   const dev::cd* r2 = S + (size_t)lab[1] * L;
   dev::cd d11 = d, d12 = d, d21 = d, d22 = d;
-  int e2 = -4096;
+  int e2 = -4096, p11 = -8192, p12 = -8192, p21 = -8192, p22 = -8192;
   for (int q = 0; q < n; q++) {
     const dev::cd z1 = fx::value(Y[q * T], e), z2 = fx::value(Y[(n + q) * T], e);
     const dev::cd b1 = dev::ldS(r1 + col[q]), b2 = dev::ldS(r2 + col[q]);
-    ez = max(ez, max(dev::expo(z1), dev::expo(z2)));
-    eb = max(eb, dev::expo(b1));
-    e2 = max(e2, dev::expo(b2));
+    const int ez1 = dev::expo(z1), ez2 = dev::expo(z2), eb1 = dev::expo(b1), eb2 = dev::expo(b2);
+    ez = max(ez, max(ez1, ez2));
+    eb = max(eb, eb1);
+    e2 = max(e2, eb2);
+    p11 = max(p11, eb1 + ez1);
+    p12 = max(p12, eb1 + ez2);
+    p21 = max(p21, eb2 + ez1);
+    p22 = max(p22, eb2 + ez2);
     d11 = dev::cfma(b1, z1, d11);
     d12 = dev::cfma(b1, z2, d12);
     d21 = dev::cfma(b2, z1, d21);
     d22 = dev::cfma(b2, z2, d22);
   }
+  ez = max(ez, 0);
   d = dev::cmul(factor, dev::cfms(d12, d21, dev::cmul(d11, d22)));
-  *fail = dev::expo(d) < eb + e2 + dev::expo(factor) + 2 * max(ez, 0) - kc;
+  const int ed = dev::expo(d), es = eb + e2 + dev::expo(factor) + 2 * ez;
+  const bool carried = min(p11, p12) >= eb + ez - fx::kCarryBits && min(p21, p22) >= e2 + ez - fx::kCarryBits;
+  *fail = ed < es - kc || (ed < es - fx::kFloorBits2 && !carried);
   return d;
 }
 
@@ -795,18 +828,21 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       }
     };
     const int thr1 = fx::threshold(a.kc, 1), thr2 = fx::threshold(a.kc, 2);
+    const int sure1 = fx::accepted(a.kc, 1), sure2 = fx::accepted(a.kc, 2);
     // members four at a time (a step that they do not fill repeats the last one)
     constexpr int kN = 4;
     const int step = fxm ? kN : 1;
     for (int c = 0; c < kW; c += step) {
-      bool slow[4] = {true, true, true, true};  // this lane's pair with member c + k goes through FP64
+      unsigned slow = 15;  // bit k: this lane's pair with member c + k goes through FP64
       if (fxm) {
         fx::Val u[kN], t[kN];
         int at = 0;
+        slow = 0;
         for (int f = 0; f < a.F; f++) {
           const int n = a.n_f[f], L = a.L_f[f];
           if (n == 0) continue;
           const int rho = a.fam_rank[(int64_t)W * a.F + f];
+          const unsigned before = slow;  // by an earlier flavour
           const unsigned short* lb = lab + a.yoff[f] * 32;
           const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
           fx::Val v[kN];
@@ -826,13 +862,24 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           } else {
             fx_dots<kN>(n, r, lb, Yf, T, v);
           }
-          const int thr = rho == 2 ? thr2 : thr1;
+          const int thr = rho == 2 ? thr2 : thr1, sure = rho == 2 ? sure2 : sure1;
+          unsigned look = 0;  // values that the guard lets pass, but small: it depends on the products
   #pragma unroll
           for (int k = 0; k < kN; k++) {
-            const bool ok = fx::usable(fx::magnitude(v[k]), thr);
+            const int mag = fx::magnitude(v[k]);
+            const bool ok = fx::usable(mag, sure);
             u[k] = at == 0 ? v[k] : u[k];
             t[k] = v[k];
-            slow[k] = (at > 0 && slow[k]) || !ok;
+            look |= (unsigned)(!ok && c + k < kW && fx::usable(mag, thr)) << k;
+            slow |= (unsigned)!ok << k;
+          }
+          for (unsigned todo = __reduce_or_sync(0xffffffffu, look); todo; todo &= todo - 1) {
+            const int k = __ffs(todo) - 1, m = mem0 + c + k;
+            const int32_t* mlab = a.mem_lab + ((int64_t)m * a.F + f) * MHC_MAX_RANK;
+            const int4* r1 = at == 0 ? a.fx.ws + (size_t)m * L : a.fx.s[f] + (size_t)mlab[0] * L;
+            const bool two = NCMAX >= 10 && rho == 2;
+            if (fx_carries(n, two ? 2 : 1, r1, a.fx.s[f] + (size_t)mlab[two ? 1 : 0] * L, lb, Yf, T))
+              slow &= ~(look & (1u << k) & ~before);
           }
           at++;
         }
@@ -840,8 +887,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   #pragma unroll
         for (int k = 0; k < kN; k++) {
           const int d = __ldg(a.fx.shift + mem0 + min(c + k, kW - 1));
-          slow[k] = c + k < kW && (slow[k] || d == fx::kNever);
-          const bool use = c + k < kW && !slow[k] && fx::aligns(d, a.fx.nf);
+          if (d == fx::kNever) slow |= 1u << k;
+          const bool use = c + k < kW && !((slow >> k) & 1) && fx::aligns(d, a.fx.nf);
           far |= (unsigned)(c + k < kW && !fx::aligns(d, a.fx.nf) && d < fx::kMute) << k;
           const int du = !use ? 0 : a.fx.nf == 1 ? d : d >> 1, dt = use ? d - du : 0;
           term(tot, use ? fx::aligned(u[k], du) : fx::Val{0, 0}, fx::aligned(t[k], dt));
@@ -853,7 +900,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         while (far) {
           const int k = __ffs(far) - 1;
           far &= far - 1;
-          const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
+          const bool p = (slow >> k) & 1;
           const fx::Val uk = k == 0 ? u[0] : k == 1 ? u[1] : k == 2 ? u[2] : u[3];
           fx::Acc2 one;
           term(one, p ? fx::Val{0, 0} : uk, k == 0 ? t[0] : k == 1 ? t[1] : k == 2 ? t[2] : t[3]);
@@ -861,10 +908,10 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         }
       }
       // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
-  #pragma unroll 1
-      for (int k = 0; k < step; k++) {
-        const bool p = k == 0 ? slow[0] : k == 1 ? slow[1] : k == 2 ? slow[2] : slow[3];
-        if (__any_sync(0xffffffffu, p)) member64(c + k, p);
+      slow &= (1u << min(step, kW - c)) - 1u;
+      for (unsigned todo = __reduce_or_sync(0xffffffffu, slow); todo; todo &= todo - 1) {
+        const int k = __ffs(todo) - 1;
+        member64(c + k, (slow >> k) & 1);
       }
     }
   }

@@ -11,11 +11,13 @@
 // integer round(x 2^(b - e)), |.| <= 2^b (b = 54 .. 57, below), split as hi 2^27 + lo with lo in
 // [-2^26, 2^26).  A sum accumulates hi hi and hi lo + lo hi in 64 bits and drops lo lo, at most
 // 2^52 per product against 2^111 for the vectors' scale in a dot.  A dot is off by less than
-// (2 n) 2^-56 |g|max |y|max then, a quarter of what the FP64 chain's n 2^-53 allows at the same
-// scale.  A dot that comes out below 2^-kc of that scale (kc: the lemma guard's exponent) or above
-// eight times it is not used: the FP64 path forms that determinant again and applies its own
-// guard, so which pairs are refactored does not depend on this arithmetic.  (Random blocks of
-// n = 6 to 18: the median dot is 2^-1.7 of the scale, one in a thousand lies above 2^0.6 to 2^1.)
+// (2 n) 2^-56 |g|max |y|max then.  That is a quarter of what an FP64 chain may be off by when its
+// largest product has that size, and more than FP64's error when all products are far smaller.  So a
+// dot well below the scale is used only after a look at the products (accepted, below), and one below
+// 2^-kc of it (kc: the lemma guard's exponent) or above eight times it never: the FP64 path forms that
+// determinant again and applies its own guard, so which pairs are refactored does not depend on this
+// arithmetic.  (Random blocks of n = 6 to 18: the median dot is 2^-1.7 of the scale, one in a thousand
+// lies above 2^0.6 to 2^1.)
 #pragma once
 
 #include <cuda_runtime.h>
@@ -127,6 +129,26 @@ __device__ __forceinline__ bool usable(int mag, int thr, int top = kMaxHi) { ret
 __device__ __forceinline__ int threshold(int kc, int rank) {
   const int t = (rank == 1 ? kDotBits : 53) - 32 - kc;
   return t >= 28 ? kNever : t <= 0 ? 1 : 1 << t;
+}
+
+// High word of the smallest |value| accepted by itself, whatever the guard allows.  A dot is off by a
+// few units of 2^57 2^-56 times the square root of n, so a value of 2^(57 - kFloorBits) by some 2^-48 of
+// itself (a two-row determinant has three bits more to give: its two dots are each off by as little).  A
+// smaller one may be a sum of large products that cancel, where FP64 is off as much: it is accepted
+// when the largest product is within kCarryBits binades of the scale.  Or every product is far below the
+// scale, as the row is large where the solve is small: then FP64 rounds each product at its own size,
+// and the FP64 path evaluates the pair.  On random blocks of n = 3 to 18 one dot in 700 lies below the
+// floor.
+constexpr int kFloorBits = 7;
+constexpr int kFloorBits2 = 10;  // of a two-row determinant, 2^56 for the scales
+constexpr int kCarryBits = 4;
+constexpr int kCarries = 1 << (kDotBits - kCarryBits - 32);
+__device__ __forceinline__ int accepted(int kc, int rank) {
+  return max(threshold(kc, rank), 1 << (rank == 1 ? kDotBits - 32 - kFloorBits : kDotBits - 1 - 32 - kFloorBits2));
+}
+// high word of the product of the larger components' high limbs, 2^57 for the scale
+__device__ __forceinline__ int product_magnitude(int4 a, int4 b) {
+  return (int)(madw(max(abs(a.x), abs(a.z)), max(abs(b.x), abs(b.z)), 0) >> 32);
 }
 
 // Products of two dots.  A dot's scale is an upper bound that it stays a few binades below: the product

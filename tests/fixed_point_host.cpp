@@ -1,11 +1,12 @@
-// Host test of csrc/fx.cuh: the solves that the fixed-point path accepts, against long double, beside
-// the FP64 path's (csrc/device.cuh: kfac_block, kapply).  Prints: blocks, those refused, sinks, those
-// refused, and the accepted solves' largest error by their largest entry, median and maximum, then the
-// same for FP64.
-// usage: fixed_point_host n pattern spread kp [seed]
+// Host test of csrc/fx.cuh: the solves and the determinants that the fixed-point path accepts, against
+// long double, beside the FP64 path's (csrc/device.cuh: kfac_block, kapply, member_det).  Prints: blocks,
+// those refused, sinks, those refused, and the accepted solves' largest error by their largest entry,
+// median and maximum, then the same for FP64; determinants accepted, left to the FP64 path, and the
+// accepted ones' relative error, median and maximum, then the same for FP64.
+// usage: fixed_point_host n pattern spread kp kc [seed]
 //   pattern: rows | cols | both: scaled by random powers of two over 2^spread; decay: by
 //   2^-spread per step between 12-label sites; onerow, onecol: one label in eight scaled by 2^-spread;
-//   flip: rows and columns alternately by 2^spread
+//   flip: rows and columns alternately by 2^spread; unused: columns that no sink has scaled by 2^spread
 #include <complex>
 #include <cstdio>
 #include <cstdlib>
@@ -20,6 +21,26 @@ typedef std::complex<long double> CL;
 typedef dev::cd cd;
 
 static CL wide(cd z) { return CL(z.x, z.y); }
+
+static CL exact_det(std::vector<std::vector<CL>> A) {
+  const int n = (int)A.size();
+  CL det = 1;
+  for (int k = 0; k < n; k++) {
+    int p = k;
+    for (int i = k; i < n; i++)
+      if (std::abs(A[i][k]) > std::abs(A[p][k])) p = i;
+    if (p != k) {
+      std::swap(A[p], A[k]);
+      det = -det;
+    }
+    det *= A[k][k];
+    for (int i = k + 1; i < n; i++) {
+      const CL l = A[i][k] / A[k][k];
+      for (int q = k; q < n; q++) A[i][q] -= l * A[k][q];
+    }
+  }
+  return det;
+}
 
 // z = -B^{-1} a in long double
 static std::vector<CL> exact_solve(std::vector<std::vector<CL>> A, std::vector<CL> x) {
@@ -45,12 +66,15 @@ static std::vector<CL> exact_solve(std::vector<std::vector<CL>> A, std::vector<C
 }
 
 int main(int argc, char** argv) {
-  const int n = atoi(argv[1]), spread = atoi(argv[3]), kp = atoi(argv[4]);
+  const int n = atoi(argv[1]), spread = atoi(argv[3]), kp = atoi(argv[4]), kc = atoi(argv[5]);
   const std::string pattern = argv[2];
-  std::mt19937_64 g(argc > 5 ? atoi(argv[5]) : 1);
+  std::mt19937_64 g(argc > 6 ? atoi(argv[6]) : 1);
   std::normal_distribution<double> N(0, std::sqrt(.5));
   const int L = n == 18 ? 96 : 12 * ((n + 2) / 3) + 12, M = n - 1;
   std::vector<cd> S((size_t)L * L);
+  std::vector<int> used(L, 1);
+  for (int l = 0; l < L; l++)
+    if (pattern == "unused" && l % 4 == 3) used[l] = 0;
   std::vector<int> re(L), ce(L);
   for (int l = 0; l < L; l++) re[l] = (int)(g() % (spread + 1)), ce[l] = (int)(g() % (spread + 1));
   for (int a = 0; a < L; a++)
@@ -61,25 +85,32 @@ int main(int argc, char** argv) {
       if (pattern == "decay") e = -spread * std::abs(a / 12 - b / 12);
       if (pattern == "onerow") e = a % 8 ? 0 : -spread;
       if (pattern == "onecol") e = b % 8 ? 0 : -spread;
+      if (pattern == "unused" && !used[b]) e = spread;
       if (pattern == "flip") e = (a ^ b) & 1 ? spread : 0;
       const double f = std::ldexp(1.0, e);
       S[(size_t)a * L + b] = {(N(g) + (a == b ? (n == 18 ? 3 : 2) : 0)) * f, N(g) * f};
     }
-  std::vector<int> cexp(L);
-  for (int c = 0; c < L; c++) {
-    int e = -4096;
-    for (int a = 0; a < L; a++) e = max(e, dev::expo(S[(size_t)a * L + c]));
-    cexp[c] = e + 1;
+  std::vector<int> rexp(L), cexp(L);
+  for (int l = 0; l < L; l++) {
+    int er = -4096, ec = -4096;
+    for (int k = 0; k < L; k++) {
+      er = max(er, dev::expo(S[(size_t)l * L + k]));
+      ec = max(ec, dev::expo(S[(size_t)k * L + l]));
+    }
+    rexp[l] = er + 1;
+    cexp[l] = ec + 1;
   }
-  std::vector<double> efx, e64;
-  long blocks = 0, brefused = 0, sinks = 0, srefused = 0;
-  for (int t = 0; t < 3000; t++) {
+  std::vector<double> efx, e64, dfx, d64;
+  long blocks = 0, brefused = 0, sinks = 0, srefused = 0, accepted = 0, left = 0;
+  for (int t = 0; t < (n > 9 ? 800 : 3000); t++) {
     std::vector<int> p(L);
     for (int i = 0; i < L; i++) p[i] = i;
     std::shuffle(p.begin(), p.end(), g);
-    std::vector<int32_t> rows(p.begin(), p.begin() + M);
+    std::vector<int32_t> rows(p.begin(), p.begin() + M), members(p.begin() + M, p.begin() + M + 4);
     std::shuffle(p.begin(), p.end(), g);
-    std::vector<int32_t> cols(p.begin(), p.begin() + n + 3);
+    std::vector<int32_t> cols;
+    for (int l : p)
+      if (used[l] && (int)cols.size() < n + 3) cols.push_back(l);
     std::vector<cd> K(M * M + M + 2), KX(M * M + M + 2), Y(n);
     const bool guard = dev::kfac_block<18, 0, 1>(S.data(), L, n, rows.data(), cols.data(), K.data(), kp, false);
     if (guard) continue;
@@ -110,16 +141,44 @@ int main(int argc, char** argv) {
         x[i] = wide(S[(size_t)rows[i] * L + c[M]]);
       }
       const std::vector<CL> z = exact_solve(B, x);
-      long double top = 1, dx = 0, d64 = 0;  // the unit entry
+      long double top = 1, dx = 0, dy = 0;  // the unit entry
       for (int i = 0; i < M; i++) {
         const fx::Val v = fx::joined(y[i]);
         top = max(top, std::abs(z[i]));
         const int u = (e2 >> 1) - fx::kFracBits;
         dx = max(dx, std::abs(CL(std::ldexp((long double)v.re, u), std::ldexp((long double)v.im, u)) - z[i]));
-        d64 = max(d64, std::abs(wide(Y[i]) / wide(Y[M]) - z[i]));  // y = det B z
+        dy = max(dy, std::abs(wide(Y[i]) / wide(Y[M]) - z[i]));  // y = det B z
       }
       efx.push_back((double)(dx / top));
-      e64.push_back((double)(d64 / top));
+      e64.push_back((double)(dy / top));
+      for (int m : members) {
+        bool fail = false;
+        const cd det64 = dev::member_det<18, 0, 1>(S.data(), L, n, &m, c.data(), Y.data(), 1, ey, kc, &fail);
+        if (fail) continue;  // refactored
+        fx::Acc s;
+        std::vector<int4> row(n);
+        int largest = 0;
+        for (int q = 0; q < n; q++) {
+          row[q] = fx::quant(S[(size_t)m * L + c[q]], rexp[m], fx::kRowBits);
+          fx::mac(s, row[q], y[q]);
+          largest = max(largest, fx::product_magnitude(row[q], y[q]));
+        }
+        const fx::Val v = fx::finish(s);
+        const int mag = fx::magnitude(v);
+        if (!fx::usable(mag, fx::accepted(kc, 1)) && !(fx::usable(mag, fx::threshold(kc, 1)) && largest >= fx::kCarries)) {
+          left++;
+          continue;
+        }
+        accepted++;
+        std::vector<std::vector<CL>> A(n, std::vector<CL>(n));
+        for (int i = 0; i < n; i++)
+          for (int q = 0; q < n; q++) A[i][q] = wide(S[(size_t)(i < M ? rows[i] : m) * L + c[q]]);
+        const CL ref = exact_det(A);
+        const int u = (e2 >> 1) + rexp[m] - fx::kDotBits;
+        const CL got = CL(std::ldexp((long double)v.re, u), std::ldexp((long double)v.im, u)) * wide(KX[M * M + M + 1]);
+        dfx.push_back((double)(std::abs(got - ref) / std::abs(ref)));
+        d64.push_back((double)(std::abs(wide(det64) - ref) / std::abs(ref)));
+      }
     }
   }
   auto stat = [](std::vector<double> v, double* med, double* mx) {
@@ -132,6 +191,9 @@ int main(int argc, char** argv) {
   double a, b, c, d;
   stat(efx, &a, &b);
   stat(e64, &c, &d);
-  printf("%ld %ld %ld %ld %.3e %.3e %.3e %.3e\n", blocks, brefused, sinks, srefused, a, b, c, d);
+  printf("%ld %ld %ld %ld %.3e %.3e %.3e %.3e ", blocks, brefused, sinks, srefused, a, b, c, d);
+  stat(dfx, &a, &b);
+  stat(d64, &c, &d);
+  printf("%ld %ld %.3e %.3e %.3e %.3e\n", accepted, left, a, b, c, d);
   return 0;
 }

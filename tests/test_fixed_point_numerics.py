@@ -31,7 +31,21 @@ def host(tmp_path_factory):
 def test_solves(host, n, pattern, spread, pivots):
     """An accepted solve has a unit in 2^55 times a spread of 2^3 at every place where FP64 has one in
     2^53: four times the error, and sixteen in the extremes, where a small w meets a large pivot (2^-47)."""
-    blocks, refused, sinks, left, med, worst, med64, worst64 = host(n, pattern, spread, pivots)
+    blocks, refused, sinks, left, med, worst, med64, worst64 = host(n, pattern, spread, pivots, 10)[:8]
     assert med <= 4 * med64 + 2.0 ** -53 and worst <= 16 * worst64 + 2.0 ** -47
     if spread == 0:
         assert refused <= 0.01 * blocks and left <= 0.05 * sinks
+
+
+@pytest.mark.parametrize("guard", [10, 30, 4096])  # the default lemma guard, a lower one, and none
+@pytest.mark.parametrize("pattern, spread", [("rows", 0), ("rows", 4), ("cols", 4), ("cols", 20), ("onecol", 8), ("onerow", 8),
+                                             ("unused", 5), ("unused", 10), ("unused", 25), ("unused", 45)])
+@pytest.mark.parametrize("n", [3, 6, 12, 18])
+def test_determinants(host, n, pattern, spread, guard):
+    """An accepted determinant: a value of 2^-7 of the scale is off by a few units of 2^-56 of it, 2^-46 at
+    the most; beyond that as the solves, four times FP64's error and sixteen in the extremes."""
+    out = host(n, pattern, spread, 13 if guard == 10 else 4096, guard)
+    accepted, left, med, worst, med64, worst64 = out[8:]
+    assert med <= 4 * med64 + 2.0 ** -49 and worst <= 16 * worst64 + 2.0 ** -46
+    if spread == 0:
+        assert left <= 0.005 * accepted

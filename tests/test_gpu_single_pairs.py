@@ -136,3 +136,16 @@ def test_zero_weights_pass_the_guards(M):
     after = run.plan.stats()
     assert after["refactor_child"] == before["refactor_child"] and after["refactor_parent"] == before["refactor_parent"]
     run.plan.close()
+
+
+@pytest.mark.parametrize("tau_child", [1e-3, 0.0])
+@pytest.mark.parametrize("n", [[6, 5], [18], [12, 10]])
+def test_smallest_values(M, n, tau_child):
+    """The smallest of a source's determinants, also with no lemma guard behind the accuracy floor."""
+    run = Runner(M, make(n, 70 + sum(n)), tau_child=tau_child)
+    assert run.tables() == 1
+    for terms in families(run)[::24]:
+        for j in np.argsort(run.all_dets(terms[0]))[:4]:
+            ref = run.exact(terms[0], j)
+            assert abs(run.C({terms[0]: 1.0}, {j: 1.0}) - ref) <= 1e-12 * abs(ref)
+    run.plan.close()

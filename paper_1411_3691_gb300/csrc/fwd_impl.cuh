@@ -268,11 +268,6 @@ __device__ __forceinline__ dev::cd fx_factor(const FwdArgs& a, int W, int Q, int
   return a.kbuf[((int64_t)W * a.n_q + Q) * a.kstride + a.koff[f] + (n - 1) * (n - 1) + n];
 }
 
-// The kernel without tables takes real weights only (complex ones go to the kernel with tables,
-// which runs plans without them too); the n <= 32 class has the one kernel.
-template <int NCMAX, bool FX>
-constexpr bool kComplexWeights = FX || NCMAX > 18;
-
 // Refactor one pair per lane (the lanes with have; e: the pair, j: its sink position):
 // the product of the flavours that passed, times fresh determinants of the flavours that
 // failed, accumulated into acc.  With a.rowdiff the row-difference update is tried first
@@ -281,11 +276,10 @@ constexpr bool kComplexWeights = FX || NCMAX > 18;
 // the others one per lane.  Yw: the warp's cached solves (lane l at Yw + l, stride
 // blockDim.x), in fixed point with exponents eyw when fxm; wk: the warp's scratch for group_fresh.
 // Called by the whole warp.
-template <int NCMAX, bool FX>
+template <int NCMAX, bool FX, bool CW>
 __device__ __forceinline__ void refactor_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
                                                const double2* Yw, bool fxm, const short* eyw, double2* wk,
                                                double2& acc, unsigned long long& rflops, unsigned long long& nrd) {
-  constexpr bool kCw = kComplexWeights<NCMAX, FX>;
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int T = blockDim.x;
@@ -367,30 +361,30 @@ __device__ __forceinline__ void refactor_pairs(const FwdArgs& a, int W, bool hav
       rflops += fresh_flops(n);
     }
   }
-  if (have) acc = dev::add_weighted<kCw>(a, e.w, prod, acc);
+  if (have) acc = dev::add_weighted<CW>(a, e.w, prod, acc);
 }
 
 // With the fixed-point member loop a call, not inlined: that loop keeps its registers and the
 // instruction cache its lines.
-template <int NCMAX>
+template <int NCMAX, bool CW>
 __device__ __noinline__ void refactor_call(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j,
                                            const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc,
                                            unsigned long long& rflops, unsigned long long& nrd) {
-  refactor_pairs<NCMAX, true>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
+  refactor_pairs<NCMAX, true, CW>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
 }
 
-template <int NCMAX, bool FX>
+template <int NCMAX, bool FX, bool CW>
 __device__ void process_pairs(const FwdArgs& a, int W, bool have, const QEntry& e, int64_t j, const double2* Yw,
                               bool fxm, const short* eyw, double2* wk, double2& acc, unsigned long long& rflops,
                               unsigned long long& nrd) {
   if constexpr (FX)
-    refactor_call<NCMAX>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
+    refactor_call<NCMAX, CW>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
   else
-    refactor_pairs<NCMAX, false>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
+    refactor_pairs<NCMAX, false, CW>(a, W, have, e, j, Yw, fxm, eyw, wk, acc, rflops, nrd);
 }
 
 // Refactor the first count queued pairs (one per lane).  Called by the whole warp.
-template <int NCMAX, bool FX>
+template <int NCMAX, bool FX, bool CW>
 __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int64_t jbase,
                               const double2* Yw, bool fxm, const short* eyw, double2* wk, double2& acc,
                               unsigned long long& rflops, unsigned long long& nrd) {
@@ -398,7 +392,7 @@ __device__ void process_queue(const FwdArgs& a, int W, QEntry* q, int count, int
   const bool have = lane < count;
   QEntry e = {};
   if (have) e = q[lane];
-  process_pairs<NCMAX, FX>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, fxm, eyw, wk, acc, rflops, nrd);
+  process_pairs<NCMAX, FX, CW>(a, W, have, e, jbase + (have ? e.lane : 0), Yw, fxm, eyw, wk, acc, rflops, nrd);
 }
 
 // ---- solves and member dots in fixed point (fx.cuh) -------------------------------------
@@ -579,8 +573,9 @@ static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S
 }
 
 // One work item (family W x sink tile) by the whole thread block; the block's sum goes
-// to *partial.  Shared by the per-plan launch and the persistent batched launch. 
-template <int NCMAX, bool FX>
+// to *partial.  Shared by the per-plan launch and the persistent batched launch.  FX: the plan has
+// fixed-point tables; else the FP64 path alone.  CW: the weights may be complex.
+template <int NCMAX, bool FX, bool CW>
 __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, double2* smem,
                                          double2* partial) {
   const int T = blockDim.x;
@@ -599,7 +594,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   const double2* Yw = smem + (tid & ~31);  // the warp's cached solves (lane l: Yw + l)
 
   // ---- per flavour: solve, or factorise the shared rows, for this sink ----------------
-  constexpr bool kFx = FX, kCw = kComplexWeights<NCMAX, FX>;
+  constexpr bool kFx = FX;
   unsigned short* lab = reinterpret_cast<unsigned short*>(scratch + WS::kQueue + WS::kWalk) + lane;
   short* eyw = reinterpret_cast<short*>(scratch + WS::exponents(a.slots));
   bool fxm = kFx && a.fx.nf > 0 && kW <= fx::kMaxMembers, bad = false;
@@ -710,7 +705,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   }
 
   // ---- per member: one dot product per flavour --------------------------------------
-  const double2 wj = valid ? dev::sink_weight<kCw>(a, j) : make_double2(0.0, 0.0);
+  const double2 wj = valid ? dev::sink_weight<CW>(a, j) : make_double2(0.0, 0.0);
   // acc: sum over the members of w_i prod_f det (this lane's sink; times w_j once, at the
   // end); accq: the refactored pairs, w_i w_j included (a queue lane holds other sinks' pairs)
   double2 acc = make_double2(0.0, 0.0), accq = make_double2(0.0, 0.0);
@@ -755,8 +750,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       }
     }
     const bool need = valid && part && fail != 0;
-    const double2 wi = dev::source_weight<kCw>(a, m);
-    if (part && !fail) acc = dev::add_weighted<kCw>(a, wi, prod, acc);
+    const double2 wi = dev::source_weight<CW>(a, m);
+    if (part && !fail) acc = dev::add_weighted<CW>(a, wi, prod, acc);
     const unsigned ball = __ballot_sync(0xffffffffu, need);
     if (ball == 0xffffffffu) {
       // every lane refactors this member (a member near-singular against its family): the
@@ -768,8 +763,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       e.fail = (int32_t)fail;
       e.pguard = (int32_t)pguard;
       e.prod = prod;
-      e.w = dev::add_weighted<kCw>(a, wi, wj, make_double2(0.0, 0.0));
-      process_pairs<NCMAX, FX>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+      e.w = dev::add_weighted<CW>(a, wi, wj, make_double2(0.0, 0.0));
+      process_pairs<NCMAX, FX, CW>(a, W, true, e, j, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
       n_parent += __popc(fail & pguard);
       n_child += __popc(fail & ~pguard);
     } else if (ball) {
@@ -781,7 +776,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
         e.fail = (int32_t)fail;
         e.pguard = (int32_t)pguard;
         e.prod = prod;
-        e.w = dev::add_weighted<kCw>(a, wi, wj, make_double2(0.0, 0.0));
+        e.w = dev::add_weighted<CW>(a, wi, wj, make_double2(0.0, 0.0));
         queue[pos] = e;
         n_parent += __popc(fail & pguard);
         n_child += __popc(fail & ~pguard);
@@ -789,7 +784,7 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
       qn += __popc(ball);
       __syncwarp();
       if (qn >= 32) {
-        process_queue<NCMAX, FX>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+        process_queue<NCMAX, FX, CW>(a, W, queue, 32, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
         __syncwarp();
         if (lane < qn - 32) queue[lane] = queue[32 + lane];
         __syncwarp();
@@ -907,7 +902,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           add(one, __ldg(a.fx.shift + mem0 + c + k));
         }
       }
-      // pairs out of the fixed-point range or near the lemma guard (every pair without tables)
+      // pairs out of the fixed-point range or near the lemma guard (every pair of a family or warp that
+      // the format does not take)
       slow &= (1u << min(step, kW - c)) - 1u;
       for (unsigned todo = __reduce_or_sync(0xffffffffu, slow); todo; todo &= todo - 1) {
         const int k = __ffs(todo) - 1;
@@ -916,8 +912,8 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
     }
   }
   __syncwarp();
-  if (qn > 0) process_queue<NCMAX, FX>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
-  acc = dev::add_weighted<kCw>(a, wj, acc, accq);
+  if (qn > 0) process_queue<NCMAX, FX, CW>(a, W, queue, qn, (int64_t)tile * T + warp * 32, Yw, fxm, eyw, wk, accq, rflops, n_rowdiff);
+  acc = dev::add_weighted<CW>(a, wj, acc, accq);
 
   // ---- fixed-order reduction: lanes, then warps --------------------------------------
   acc = dev::warp_sum(acc);
@@ -978,16 +974,25 @@ __device__ __forceinline__ void fold_partials(const FwdArgs& a, double2* smem) {
 // Registers: the n <= 8 class keeps 168 (12 one-warp blocks per SM, or 3 blocks of its
 // 128-thread tile); the larger classes may use all 255, measured fastest for n = 18 (8 blocks
 // per SM against 9 at 216 and 10 at 200, whose spills cost more than the warps gain).
-// FX: the plan has fixed-point tables, or complex weights; else the kernel holds the FP64 path for
-// real weights alone.  512 x 512 terms of n = 3: 55 us per call, and 64 us when it also carried the
-// complex weights, converted solves for the refactors and a launch for the partials' sum.
+// FX: the call has fixed-point tables, or complex weights; else the kernel holds the FP64 path for
+// real weights alone (n <= 32: for both).  512 x 512 terms of n = 3: 55 us per call, and 64 us when it
+// also carried the complex weights, converted solves for the refactors and a launch for the partials'
+// sum.  The FX kernel keeps the FP64 path apart, as a copy of its own.
 template <int NCMAX, bool FX>
 __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) {
   extern __shared__ double2 smem[];
   const int64_t item = a.item0 + blockIdx.x;
   const int64_t pos = item / a.n_tiles;
   const int W = a.fam_order ? a.fam_order[pos] : (int)pos;
-  fwd_item<NCMAX, FX>(a, W, (int)(item % a.n_tiles), smem, &a.partials[item]);
+  const int tile = (int)(item % a.n_tiles);
+  if constexpr (FX) {
+    if (a.fx.nf > 0)
+      fwd_item<NCMAX, true, true>(a, W, tile, smem, &a.partials[item]);
+    else
+      fwd_item<NCMAX, false, true>(a, W, tile, smem, &a.partials[item]);
+  } else {
+    fwd_item<NCMAX, false, (NCMAX > 18)>(a, W, tile, smem, &a.partials[item]);
+  }
   if (a.fold_items > 0) fold_partials(a, smem);
 }
 
@@ -1399,7 +1404,8 @@ cudaError_t launch_kfac_nc(const FwdArgs& a, int64_t n_fam, cudaStream_t s) {
 
 // Persistent batched launch: blocks pull (correlator, family, tile) items from a list
 // ordered by decreasing cost through one atomic counter; each item's partial goes to its
-// own slot (see batch.cu).  Registers as fwd_kernel's (at most 128 threads per block).
+// own slot (see batch.cu).  Registers as fwd_kernel's (at most 128 threads per block).  The paths with
+// and without tables are copies of their own (FP64 items ran 4 % slower through the one that has both).
 template <int NCMAX>
 __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) batch_kernel(const FwdArgs* __restrict__ desc,
                                                     const BatchItem* __restrict__ items,
@@ -1415,8 +1421,11 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) batch_kernel(const FwdArgs* 
     if (it >= n_items) break;
     const BatchItem bi = items[it];
     const FwdArgs& a = desc[bi.corr];
-    fwd::fwd_item<NCMAX, NCMAX <= 18>(a, bi.W, bi.tile, smem,
-                    &partials[part_off[bi.corr] + (int64_t)bi.W * a.n_tiles + bi.tile]);
+    double2* partial = &partials[part_off[bi.corr] + (int64_t)bi.W * a.n_tiles + bi.tile];
+    if (NCMAX <= 18 && a.fx.nf > 0)
+      fwd::fwd_item<NCMAX, (NCMAX <= 18), false>(a, bi.W, bi.tile, smem, partial);
+    else
+      fwd::fwd_item<NCMAX, false, false>(a, bi.W, bi.tile, smem, partial);
     __syncthreads();
   }
 }

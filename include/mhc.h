@@ -142,7 +142,7 @@ typedef struct {
 /* How one mhc_correlator call of a plan runs (mhc_forward_info). */
 typedef struct {
   int32_t tables;       /* 1: the plan holds fixed-point tables of the propagators      */
-  int32_t tables_used;  /* 1: and the last call's solves and dots ran on them           */
+  int32_t tables_used;  /* 1: and the last call's propagators suited them (else FP64)   */
   int32_t folded_sum;   /* 1: the forward kernel's last block sums the partials, no
                            launch of its own                                           */
   int32_t launches;     /* kernel launches of one call                                 */

@@ -39,6 +39,7 @@ mhc_status fill_fwd_args(Plan& p, const double* const* S_f, const double* w_src,
                          const double* w_snk, FwdArgs& a);
 void plan_slots(const Plan& p, int* yoff, int* total);
 size_t fx_layout(const Plan& p, char* base, fx::Tables* t);
+bool fx_alloc(const Plan& p, char** base);
 
 namespace {
 
@@ -131,7 +132,8 @@ struct mhc_batch_s {
   // a plan given more than once (one plan, several propagator sets: gauge configurations,
   // time slices) gets batch-owned block factors, guard flags and fixed-point tables for its
   // later entries; a plan too small for tables of its own gets them where the batch fills the chip
-  std::vector<void*> own_kbuf, own_kguard, own_fx;  // [count], null where the plan's own are used
+  std::vector<void*> own_kbuf, own_kguard;  // [count], null where the plan's own are used
+  std::vector<char*> own_fx;
   cudaStream_t side = nullptr;    // second branch: the class kernels run concurrently
   cudaEvent_t fork = nullptr, join = nullptr;
   std::vector<const void*> key;  // S and out pointers the graph was captured with
@@ -298,15 +300,13 @@ mhc_status fill_descs(mhc_batch_s& b, const BatchShape& sh, const double* const*
     bool repeat = false;
     for (int k2 = 0; k2 < k; k2++) repeat |= b.plans[k2] == b.plans[k];
     if (!p.dev.fx && b.own_fx[k]) {
-      fx_layout(p, reinterpret_cast<char*>(b.own_fx[k]), &desc[k].fx);
+      fx_layout(p, b.own_fx[k], &desc[k].fx);
     } else if (repeat && desc[k].fx.nf > 0) {
-      fx::Tables t;
-      const size_t bytes = fx_layout(p, nullptr, &t);
-      if (!b.own_fx[k] && cudaMalloc(&b.own_fx[k], bytes) != cudaSuccess) {
+      if (!b.own_fx[k] && !fx_alloc(p, &b.own_fx[k])) {
         set_error("mhc_batch: cudaMalloc failed for a repeated plan's fixed-point tables");
         return MHC_ENOMEM;
       }
-      fx_layout(p, reinterpret_cast<char*>(b.own_fx[k]), &desc[k].fx);
+      fx_layout(p, b.own_fx[k], &desc[k].fx);
     }
     if (repeat && desc[k].snk_orig) {
       if (!b.own_kbuf[k]) {
@@ -418,7 +418,7 @@ void destroy(mhc_batch_s* b) {
     if (p) cudaFree(p);
   for (void* p : b->own_kguard)
     if (p) cudaFree(p);
-  for (void* p : b->own_fx)
+  for (char* p : b->own_fx)
     if (p) cudaFree(p);
   if (b->cap) cudaStreamDestroy(b->cap);
   if (b->side) cudaStreamDestroy(b->side);
@@ -466,11 +466,7 @@ mhc_status mhc_batch_create(mhc_batch_t* out, int32_t count, const mhc_plan_t* p
     fx::Tables t;
     const size_t bytes = p.dev.fx || !fx_pays(p) ? 0 : fx_layout(p, nullptr, &t);
     if (bytes == 0 || fx_own + bytes > kMaxFxBytes) continue;
-    if (cudaMalloc(&b->own_fx[k], bytes) != cudaSuccess) {
-      b->own_fx[k] = nullptr;
-      cudaGetLastError();
-      break;
-    }
+    if (!fx_alloc(p, &b->own_fx[k])) break;
     fx_own += bytes;
   }
   std::vector<int64_t> kpref(1, 0), nfam, fxpref(1, 0);

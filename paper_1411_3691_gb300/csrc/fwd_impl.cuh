@@ -573,8 +573,8 @@ static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S
 }
 
 // One work item (family W x sink tile) by the whole thread block; the block's sum goes
-// to *partial.  Shared by the per-plan launch and the persistent batched launch.  FX: the plan has
-// fixed-point tables; else the FP64 path alone.  CW: the weights may be complex.
+// to *partial.  Shared by the per-plan launch and the persistent batched launch.  FX: the call takes the
+// fixed-point path (dev::fx_on); else the FP64 path alone.  CW: the weights may be complex.
 template <int NCMAX, bool FX, bool CW>
 __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, double2* smem,
                                          double2* partial) {
@@ -977,7 +977,8 @@ __device__ __forceinline__ void fold_partials(const FwdArgs& a, double2* smem) {
 // FX: the call has fixed-point tables, or complex weights; else the kernel holds the FP64 path for
 // real weights alone (n <= 32: for both).  512 x 512 terms of n = 3: 55 us per call, and 64 us when it
 // also carried the complex weights, converted solves for the refactors and a launch for the partials'
-// sum.  The FX kernel keeps the FP64 path apart, as a copy of its own.
+// sum.  The FX kernel keeps the FP64 path apart, as a copy of its own, for plans without tables
+// and for propagators that are not flat.
 template <int NCMAX, bool FX>
 __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) {
   extern __shared__ double2 smem[];
@@ -986,7 +987,7 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) 
   const int W = a.fam_order ? a.fam_order[pos] : (int)pos;
   const int tile = (int)(item % a.n_tiles);
   if constexpr (FX) {
-    if (a.fx.nf > 0)
+    if (dev::fx_on(a))
       fwd_item<NCMAX, true, true>(a, W, tile, smem, &a.partials[item]);
     else
       fwd_item<NCMAX, false, true>(a, W, tile, smem, &a.partials[item]);
@@ -1106,7 +1107,7 @@ __device__ __forceinline__ void kfac_one(const FwdArgs& a, int64_t t, int64_t n_
   }
 #define MHC_KF(N)                                                                         \
   case N:                                                                                 \
-    g = rho == 1 ? dev::kfac_block<N, N, 1>(S, L, N, arow, scol, K, a.kp, a.fx.nf > 0)    \
+    g = rho == 1 ? dev::kfac_block<N, N, 1>(S, L, N, arow, scol, K, a.kp, dev::fx_on(a))    \
                  : dev::kfac_block<N, N, (N >= 2 ? 2 : 1)>(S, L, N, arow, scol, K, a.kp, false); \
     break;
   switch (n) {
@@ -1344,7 +1345,7 @@ __device__ __forceinline__ void kfac_group_one(const FwdArgs& a, int64_t t) {
   else if (sig == 2)
     gd = dev::group_kfac_block12<KG::G>(S, L, n, arow, scol, K, a.kp, g, gm, Bs, Ps);
   else
-    gd = dev::group_kfac_block<KG::G>(S, L, n, rho, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps, NCMAX, a.fx.nf > 0);
+    gd = dev::group_kfac_block<KG::G>(S, L, n, rho, arow, scol, K, a.kp, g, gm, Bs, Ws, Ps, NCMAX, dev::fx_on(a));
   if (g == 0) a.kguard[t] = gd ? 1 : 0;
 }
 
@@ -1422,7 +1423,7 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) batch_kernel(const FwdArgs* 
     const BatchItem bi = items[it];
     const FwdArgs& a = desc[bi.corr];
     double2* partial = &partials[part_off[bi.corr] + (int64_t)bi.W * a.n_tiles + bi.tile];
-    if (NCMAX <= 18 && a.fx.nf > 0)
+    if (NCMAX <= 18 && dev::fx_on(a))
       fwd::fwd_item<NCMAX, (NCMAX <= 18), false>(a, bi.W, bi.tile, smem, partial);
     else
       fwd::fwd_item<NCMAX, false, false>(a, bi.W, bi.tile, smem, partial);

@@ -76,6 +76,9 @@ struct FwdArgs {
 
 namespace dev {
 
+// does the call take the fixed-point path: its plan has tables, and its propagators are flat
+__device__ __forceinline__ bool fx_on(const FwdArgs& a) { return a.fx.nf > 0 && a.fx.state[0] != 0; }
+
 // Per-(n, rank) dispatch to the register-resident specialisations (n <= 6) or the generic
 // runtime-n routine with arrays sized for the n class NCMAX.
 template <int NCMAX>

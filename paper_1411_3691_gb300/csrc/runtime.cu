@@ -107,6 +107,8 @@ size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
     if (p.n_f[f] == 0) continue;
     if (t->f0 < 0) t->f0 = f;
     t->nf++;
+    t->used[f] = reinterpret_cast<const int*>(take((size_t)p.L_f[f] * sizeof(int)));
+    t->scan[f] = reinterpret_cast<const int4*>(take((size_t)p.L_f[f] * sizeof(int4)));
     t->s[f] = reinterpret_cast<const int4*>(take((size_t)p.L_f[f] * p.L_f[f] * sizeof(int4)));
     t->sc[f] = reinterpret_cast<const int4*>(take((size_t)p.L_f[f] * p.L_f[f] * sizeof(int4)));
     t->cexp[f] = reinterpret_cast<const int*>(take((size_t)p.L_f[f] * sizeof(int)));
@@ -118,7 +120,38 @@ size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
   t->ws = reinterpret_cast<const int4*>(take((size_t)p.n_src * p.L_f[t->f0] * sizeof(int4)));
   t->shift = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
   t->fexp = reinterpret_cast<const int*>(take((size_t)p.n_fam * sizeof(int)));
+  t->state = reinterpret_cast<int*>(take(2 * sizeof(int)));
   return off;
+}
+
+// Allocates a plan's tables and writes what does not change between calls; false (and nothing
+// allocated): no memory for them.
+bool fx_alloc(const Plan& p, char** base) {
+  fx::Tables t;
+  const size_t bytes = fx_layout(p, nullptr, &t);
+  if (cudaMalloc(base, bytes) != cudaSuccess) {
+    *base = nullptr;
+    cudaGetLastError();
+    return false;
+  }
+  fx_layout(p, *base, &t);
+  bool ok = cudaMemset(t.state, 0, 2 * sizeof(int)) == cudaSuccess;
+  for (int f = 0; f < p.F; f++) {
+    if (p.n_f[f] == 0) continue;
+    std::vector<int> used(p.L_f[f], 0);
+    for (int side = 0; side < 2; side++) {
+      const std::vector<int32_t>& lab = side ? p.labels_snk : p.labels_src;
+      for (size_t i = 0; i < lab.size(); i += p.Tn)
+        for (int q = 0; q < p.n_f[f]; q++) used[lab[i + p.off_f[f] + q]] |= 1 << side;
+    }
+    ok = ok && cudaMemcpy(const_cast<int*>(t.used[f]), used.data(), used.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess;
+  }
+  if (!ok) {
+    cudaFree(*base);
+    *base = nullptr;
+    cudaGetLastError();
+  }
+  return ok;
 }
 
 mhc_status ensure_device(Plan& p) {
@@ -222,10 +255,7 @@ mhc_status ensure_device(Plan& p) {
   {
     fx::Tables t;
     const size_t bytes = fx_warps(p) >= kMinFxWarps && fx_pays(p) ? fx_layout(p, nullptr, &t) : 0;
-    if (bytes > 0 && bytes <= kMaxFxBytes && cudaMalloc(&d.fx, bytes) != cudaSuccess) {
-      d.fx = nullptr;  // the FP64 dots need no tables
-      cudaGetLastError();
-    }
+    if (bytes > 0 && bytes <= kMaxFxBytes) fx_alloc(p, &d.fx);  // without: the FP64 path
   }
   if ((st = upload<double>(&d.reduce, nullptr, 2 * kReduceMaxBlocks + 2)) != MHC_OK) return st;
   MHC_CUDA(cudaMemset(d.reduce, 0, (2 * kReduceMaxBlocks + 2) * sizeof(double)));
@@ -359,7 +389,12 @@ mhc_status mhc_forward_info(mhc_plan_t plan, mhc_forward_path* out, mhc_stream_t
   fx::Tables t;
   *out = mhc_forward_path();
   out->tables = p.dev.fx ? 1 : 0;
-  out->tables_used = out->tables;
+  if (p.dev.fx) {
+    fx_layout(p, p.dev.fx, &t);
+    int flat = 0;
+    MHC_CUDA(cudaMemcpy(&flat, t.state, sizeof(int), cudaMemcpyDeviceToHost));
+    out->tables_used = flat;
+  }
   out->table_bytes = p.dev.fx ? (int64_t)fx_layout(p, nullptr, &t) : 0;
   out->folded_sum = forward_folds(p.dev.n_items, p.dev.tile) ? 1 : 0;
   const int kfac = p.dev.two_sided ? 1 + (p.max_n > 6 ? 1 : 0) : 0;

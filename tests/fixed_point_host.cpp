@@ -2,7 +2,8 @@
 // long double, beside the FP64 path's (csrc/device.cuh: kfac_block, kapply, member_det).  Prints: blocks,
 // those refused, sinks, those refused, and the accepted solves' largest error by their largest entry,
 // median and maximum, then the same for FP64; determinants accepted, left to the FP64 path, and the
-// accepted ones' relative error, median and maximum, then the same for FP64.
+// accepted ones' relative error, median and maximum, then the same for FP64; whether the propagator is
+// flat (a call on others takes the FP64 path throughout).
 // usage: fixed_point_host n pattern spread kp kc [seed]
 //   pattern: rows | cols | both: scaled by random powers of two over 2^spread; decay: by
 //   2^-spread per step between 12-label sites; onerow, onecol: one label in eight scaled by 2^-spread;
@@ -91,18 +92,25 @@ int main(int argc, char** argv) {
       S[(size_t)a * L + b] = {(N(g) + (a == b ? (n == 18 ? 3 : 2) : 0)) * f, N(g) * f};
     }
   std::vector<int> rexp(L), cexp(L);
+  fx::Scan scan;
   for (int l = 0; l < L; l++) {
-    int er = -4096, ec = -4096;
+    int er = -4096, ec = -4096, small = 0, total = 0;
     for (int k = 0; k < L; k++) {
-      er = max(er, dev::expo(S[(size_t)l * L + k]));
+      if (used[k]) er = max(er, dev::expo(S[(size_t)l * L + k]));
       ec = max(ec, dev::expo(S[(size_t)k * L + l]));
     }
     rexp[l] = er + 1;
     cexp[l] = ec + 1;
+    for (int k = 0; k < L; k++) {
+      total += used[k];
+      small += used[k] && fx::small_entry(S[(size_t)l * L + k], rexp[l]);
+    }
+    scan.row(rexp[l], small, total);
+    if (used[l]) scan.column(cexp[l]);
   }
   std::vector<double> efx, e64, dfx, d64;
   long blocks = 0, brefused = 0, sinks = 0, srefused = 0, accepted = 0, left = 0;
-  for (int t = 0; t < (n > 9 ? 800 : 3000); t++) {
+  for (int t = 0; t < (n > 9 ? 500 : 1500); t++) {
     std::vector<int> p(L);
     for (int i = 0; i < L; i++) p[i] = i;
     std::shuffle(p.begin(), p.end(), g);
@@ -194,6 +202,6 @@ int main(int argc, char** argv) {
   printf("%ld %ld %ld %ld %.3e %.3e %.3e %.3e ", blocks, brefused, sinks, srefused, a, b, c, d);
   stat(dfx, &a, &b);
   stat(d64, &c, &d);
-  printf("%ld %ld %.3e %.3e %.3e %.3e\n", accepted, left, a, b, c, d);
+  printf("%ld %ld %.3e %.3e %.3e %.3e %d\n", accepted, left, a, b, c, d, (int)scan.flat());
   return 0;
 }

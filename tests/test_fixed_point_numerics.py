@@ -45,7 +45,22 @@ def test_determinants(host, n, pattern, spread, guard):
     """An accepted determinant: a value of 2^-7 of the scale is off by a few units of 2^-56 of it, 2^-46 at
     the most; beyond that as the solves, four times FP64's error and sixteen in the extremes."""
     out = host(n, pattern, spread, 13 if guard == 10 else 4096, guard)
-    accepted, left, med, worst, med64, worst64 = out[8:]
+    accepted, left, med, worst, med64, worst64 = out[8:14]
     assert med <= 4 * med64 + 2.0 ** -49 and worst <= 16 * worst64 + 2.0 ** -46
     if spread == 0:
         assert left <= 0.005 * accepted
+
+
+@pytest.mark.parametrize("pattern, spread, flat", [
+    ("rows", 0, 1), ("rows", 1, None), ("rows", 2, None), ("rows", 3, 0), ("rows", 30, 0), ("cols", 2, None), ("cols", 3, 0),
+    ("cols", 20, 0), ("both", 2, None), ("both", 3, 0), ("decay", 1, None), ("decay", 3, 0), ("decay", 8, 0), ("onerow", 4, 0),
+    ("onecol", 4, 0), ("flip", 8, 0), ("unused", 3, 1), ("unused", 40, 1)])
+@pytest.mark.parametrize("n", [4, 6, 12, 18])
+def test_flat_propagators(host, n, pattern, spread, flat):
+    """What the scan lets pass is as good in fixed point as in FP64: three times its error at most, eight in
+    the extremes (the maxima of some 10 000 determinants); rows or columns over 2^3 do not pass."""
+    out = host(n, pattern, spread, 13, 10)
+    accepted, left, med, worst, med64, worst64, is_flat = out[8:]
+    assert flat is None or is_flat == flat
+    if is_flat:
+        assert accepted > 0 and med <= 3 * med64 and worst <= 8 * worst64

@@ -30,15 +30,15 @@ def make(n, seed, diag=2.0, **kw):
     return wl.make_workload("path", n, L, SRC, SNK, seed=seed, diag=diag, **kw)
 
 
-def run(M, w, tables, one_sided=0):
-    """The plan's C; tables: whether it has to hold the fixed-point tables."""
+def run(M, w, tables, one_sided=0, flat=True):
+    """The plan's C; tables: whether it has to hold the fixed-point tables; flat: and to use them."""
     opts = M.default_opts()
     opts.one_sided = one_sided
     plan = M.Plan.from_workload(w, opts)
     S = [torch.from_numpy(np.ascontiguousarray(s)).cuda() for s in w.S]
     out = plan.correlator(S).cpu().numpy()
     info = plan.forward_info()
-    assert info["tables"] == int(tables), info
+    assert info["tables"] == int(tables) and info["tables_used"] == int(tables and flat), info
     code = M.mhc_get_status_code(plan.handle)
     plan.close()
     return out, code
@@ -93,5 +93,5 @@ def test_forward_info(M):
 def test_nonfinite_entries_are_reported(M, value):
     w = make([4, 4], 24)
     w.S[0][int(w.labels_src[0, 0])] = value
-    _, code = run(M, w, True)
+    _, code = run(M, w, True, flat=False)
     assert code == M.MHC_ENONFINITE

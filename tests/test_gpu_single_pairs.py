@@ -149,3 +149,62 @@ def test_smallest_values(M, n, tau_child):
             ref = run.exact(terms[0], j)
             assert abs(run.C({terms[0]: 1.0}, {j: 1.0}) - ref) <= 1e-12 * abs(ref)
     run.plan.close()
+
+
+def scaled(w, pattern, spread, seed=4):
+    """Propagators with rows, columns or both scaled by powers of two over 2^spread, or entries by
+    2^-spread per step between 12-label sites."""
+    rng = np.random.default_rng(seed)
+    out = []
+    for s in w.S:
+        L = s.shape[0]
+        r, c = (np.exp2(rng.integers(0, spread + 1, L)) for _ in range(2))
+        site = np.arange(L) // 12
+        f = {"rows": r[:, None], "cols": c[None, :], "both": r[:, None] * c[None, :],
+             "decay": np.exp2(-float(spread) * np.abs(site[:, None] - site[None, :]))}[pattern]
+        out.append(np.ascontiguousarray(s * f))
+    w.S = out
+    return w
+
+
+@pytest.mark.parametrize("tau", [1e-4, 1e-9, 1e-12])
+@pytest.mark.parametrize("pattern, spread", [("rows", 5), ("rows", 10), ("rows", 39), ("cols", 5), ("cols", 12), ("both", 8),
+                                             ("decay", 2)])
+@pytest.mark.parametrize("n", [[6, 5], [12, 10]])
+def test_propagators_that_are_not_flat(M, n, pattern, spread, tau):
+    """Rows, columns and entries of very different sizes, with pivot guards down to 1e-12: the call takes
+    the FP64 path, though the plan has tables, and keeps its accuracy."""
+    run = Runner(M, scaled(make(n, 80 + sum(n)), pattern, spread), tau_parent=tau)
+    run.C({}, {})
+    info = run.plan.forward_info()
+    assert info["tables"] == 1 and info["tables_used"] == 0
+    rng = np.random.default_rng(9)
+    for _ in range(25):
+        i, j = int(rng.integers(len(run.w.w_src))), int(rng.integers(len(run.w.w_snk)))
+        ref = run.exact(i, j)
+        assert abs(run.C({i: 1.0}, {j: 1.0}) - ref) <= 1e-12 * abs(ref)
+    run.plan.close()
+
+
+@pytest.mark.parametrize("n", [[6, 5], [12, 10]])
+def test_labels_that_no_term_has(M, n):
+    """Large entries, infinities and zeros in rows and columns that no term uses leave the call on the
+    fixed-point path, as accurate as without them."""
+    w = make(n, 90 + sum(n))
+    rng = np.random.default_rng(10)
+    for f, s in enumerate(w.S):
+        L = s.shape[0]
+        big = np.zeros((L + 9, L + 9), complex)
+        big[:L, :L] = s
+        big[:L, L:L + 3] = 2.0 ** 25 * rng.normal(size=(L, 3))
+        big[L:L + 3, :L] = 2.0 ** -25 * rng.normal(size=(3, L))
+        big[L + 3:L + 6, :], big[:, L + 3:L + 6] = np.inf, np.nan
+        w.S[f] = big
+    run = Runner(M, w)
+    run.C({}, {})
+    assert run.plan.forward_info()["tables_used"] == 1
+    for i in rng.integers(len(w.w_src), size=3):
+        for j in np.argsort(run.all_dets(i))[:4]:
+            ref = run.exact(i, j)
+            assert abs(run.C({i: 1.0}, {j: 1.0}) - ref) <= 1e-12 * abs(ref)
+    run.plan.close()

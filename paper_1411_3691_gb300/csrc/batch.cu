@@ -134,6 +134,7 @@ struct mhc_batch_s {
   // later entries; a plan too small for tables of its own gets them where the batch fills the chip
   std::vector<void*> own_kbuf, own_kguard;  // [count], null where the plan's own are used
   std::vector<char*> own_fx;
+  size_t fx_own = 0;              // bytes of own_fx, at most kMaxFxBytes; without memory: the FP64 path
   cudaStream_t side = nullptr;    // second branch: the class kernels run concurrently
   cudaEvent_t fork = nullptr, join = nullptr;
   std::vector<const void*> key;  // S and out pointers the graph was captured with
@@ -286,6 +287,13 @@ std::string class_key(const mhc_batch_s& b, int c) {
   return k;
 }
 
+// tables of its own for entry k, within the batch's limit
+void own_tables(mhc_batch_s& b, int k) {
+  fx::Tables t;
+  const size_t bytes = fx_layout(*b.plans[k], nullptr, &t);
+  if (bytes > 0 && b.fx_own + bytes <= kMaxFxBytes && fx_alloc(*b.plans[k], &b.own_fx[k])) b.fx_own += bytes;
+}
+
 mhc_status fill_descs(mhc_batch_s& b, const BatchShape& sh, const double* const* const* S,
                       std::vector<FwdArgs>& desc) {
   desc.resize(b.count);
@@ -299,14 +307,10 @@ mhc_status fill_descs(mhc_batch_s& b, const BatchShape& sh, const double* const*
     desc[k].n_tiles = sh.n_tiles[k];
     bool repeat = false;
     for (int k2 = 0; k2 < k; k2++) repeat |= b.plans[k2] == b.plans[k];
-    if (!p.dev.fx && b.own_fx[k]) {
-      fx_layout(p, b.own_fx[k], &desc[k].fx);
-    } else if (repeat && desc[k].fx.nf > 0) {
-      if (!b.own_fx[k] && !fx_alloc(p, &b.own_fx[k])) {
-        set_error("mhc_batch: cudaMalloc failed for a repeated plan's fixed-point tables");
-        return MHC_ENOMEM;
-      }
-      fx_layout(p, b.own_fx[k], &desc[k].fx);
+    if (repeat && p.dev.fx && !b.own_fx[k]) own_tables(b, k);
+    if (repeat || !p.dev.fx) {
+      desc[k].fx = fx::Tables();
+      if (b.own_fx[k]) fx_layout(p, b.own_fx[k], &desc[k].fx);
     }
     if (repeat && desc[k].snk_orig) {
       if (!b.own_kbuf[k]) {
@@ -459,16 +463,9 @@ mhc_status mhc_batch_create(mhc_batch_t* out, int32_t count, const mhc_plan_t* p
   // 16 correlators of 256 to 4096 terms a side, n = 3 to 18: 6.7 ms with them, 7.9 ms without
   b->own_fx.resize(count, nullptr);
   int64_t warps = 0;
-  size_t fx_own = 0;
   for (const Plan* p : b->plans) warps += fx_warps(*p);
-  for (int k = 0; k < count && warps >= kMinFxWarps; k++) {
-    const Plan& p = *b->plans[k];
-    fx::Tables t;
-    const size_t bytes = p.dev.fx || !fx_pays(p) ? 0 : fx_layout(p, nullptr, &t);
-    if (bytes == 0 || fx_own + bytes > kMaxFxBytes) continue;
-    if (!fx_alloc(p, &b->own_fx[k])) break;
-    fx_own += bytes;
-  }
+  for (int k = 0; k < count && warps >= kMinFxWarps; k++)
+    if (!b->plans[k]->dev.fx && fx_pays(*b->plans[k])) own_tables(*b, k);
   std::vector<int64_t> kpref(1, 0), nfam, fxpref(1, 0);
   for (int k = 0; k < count; k++) {
     const Plan& p = *b->plans[k];

@@ -123,12 +123,19 @@ cudaError_t launch_reduce(const FwdArgs& a, int64_t items, double* out, cudaStre
   return cudaGetLastError();
 }
 
+// In slices: pair_group_kernel has one block per 2, 4 or 8 (pair, flavour) units, and a grid holds
+// 2^31 - 1 blocks (eight flavours of n > 18: 2^29 pairs).  A slice fills the chip many times over.
+constexpr int64_t kPairSlice = (int64_t)1 << 22;
 cudaError_t launch_pairs(const FwdArgs& a, int ncmax, int64_t n_pairs, int64_t n_src,
                          const int64_t* ii, const int64_t* jj, const int32_t* src_member,
                          const int32_t* mem_family, double* dets, int32_t* path, cudaStream_t s) {
-  if (ncmax <= 8) return launch_pairs_nc8(a, n_pairs, n_src, ii, jj, src_member, mem_family, dets, path, s);
-  if (ncmax <= 18) return launch_pairs_nc18(a, n_pairs, n_src, ii, jj, src_member, mem_family, dets, path, s);
-  return launch_pairs_nc32(a, n_pairs, n_src, ii, jj, src_member, mem_family, dets, path, s);
+  const auto slice = ncmax <= 8 ? launch_pairs_nc8 : ncmax <= 18 ? launch_pairs_nc18 : launch_pairs_nc32;
+  for (int64_t p = 0; p < n_pairs; p += kPairSlice) {
+    const cudaError_t e = slice(a, n_pairs - p < kPairSlice ? n_pairs - p : kPairSlice, n_src, ii + p, jj + p, src_member,
+                                mem_family, dets + 2 * p * a.F, path ? path + p : nullptr, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace mhc

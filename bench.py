@@ -129,17 +129,10 @@ def forward_launches(plan, w, st) -> int:
     return kfac + fwd + 1
 
 
-def call_launches(plan, w, st) -> int:
-    """Kernel launches of one plain call: forward_launches, one more for the fixed-point tables
-    (plans of one or two flavours with n <= 18 and enough warps of work), one less where the
-    forward kernel's last block sums the partials itself (up to 16 per thread of a block)."""
-    n_fam, n_max = len(plan.families()["rank"]), max(w.n_f)
-    warps = n_fam * ((len(w.w_snk) + 31) // 32)
-    tables = (sum(n > 0 for n in w.n_f) in (1, 2) and n_max <= 18 and warps >= 2 * 12 * 152
-              and st["two_sided_blocks"] > 0 and (n_max > 8 or len(w.w_src) >= 4 * n_fam))
-    tile = 128 if n_max <= 8 else 64 if n_max <= 12 else 32
-    folded = n_fam * ((len(w.w_snk) + tile - 1) // tile) <= 16 * tile
-    return forward_launches(plan, w, st) + tables - folded
+def call_launches(plan) -> int:
+    """Kernel launches of one plain call, from the library: forward_launches, one more where the plan
+    has fixed-point tables, one less where the forward kernel's last block sums the partials itself."""
+    return plan.forward_info()["launches"]
 
 
 def max_over_ranks(x: float, pg, device) -> float:
@@ -411,7 +404,7 @@ def run_gpu(args):
     plan.status()
     C = [float(out[0].item()), float(out[1].item())]
 
-    launches = call_launches(plan, w, st)
+    launches = call_launches(plan)
     one_sided = rowdiff = configs = None
     if extras:
         one_sided = time_one_sided(mhc, w, S, out, flush, stream, ms_per_step, peak)
@@ -509,7 +502,7 @@ def time_config(mhc, w, flush, stream, peak, steps=20, opts=None):
     flops = st["flops_per_call"] + st["refactor_flops"] / steps
     res = {"workload": w.name, "ms_per_step": ms, "pairs_per_s": w.pairs / (ms * 1e-3),
            "tflops": flops / (ms * 1e-3) / 1e12, "frac_of_fp64_peak": flops / (ms * 1e-3) / 1e12 / peak,
-           "flops_per_step": flops, "gpu_launches_per_step": call_launches(plan, w, st)}
+           "flops_per_step": flops, "gpu_launches_per_step": call_launches(plan)}
     plan.close()
     return res
 

@@ -19,7 +19,7 @@ LIB_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIB_DIR, "libmhc.so")
 
 SOURCES = ["planner.cpp", "runtime.cu", "forward.cu", "fxprep.cu", "backward.cu", "batch.cu", "probe.cu", "noalloc.cu",
-           "fwd_fx_nc8.cu", "fwd_fx_nc18.cu"] + [f"{k}_nc{n}.cu" for k in ("fwd", "batch", "pair", "bwd") for n in (8, 18, 32)]
+           "fwd_fx_nc8.cu", "fwd_fx_nc18.cu", "fwd_cw_nc8.cu", "fwd_cw_nc18.cu"] + [f"{k}_nc{n}.cu" for k in ("fwd", "batch", "pair", "bwd") for n in (8, 18, 32)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr"]

@@ -5,7 +5,7 @@
 namespace mhc {
 
 cudaError_t launch_fwd_fx_nc18(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  return launch_fwd_nc<18, true>(a, tile, items, smem, s);
+  return launch_fwd_nc<18, true, false>(a, tile, items, smem, s);
 }
 
 }  // namespace mhc

@@ -5,7 +5,7 @@
 namespace mhc {
 
 cudaError_t launch_fwd_fx_nc8(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  return launch_fwd_nc<8, true>(a, tile, items, smem, s);
+  return launch_fwd_nc<8, true, false>(a, tile, items, smem, s);
 }
 
 }  // namespace mhc

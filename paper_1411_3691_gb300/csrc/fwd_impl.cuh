@@ -501,31 +501,11 @@ __device__ __forceinline__ fx::Val fx_det2(int n, const int4* __restrict__ r1, c
   return ok ? fx::Val{p.re - m.re, p.im - m.im} : fx::Val{0, 0};  // half the determinant
 }
 
-// Whether a member's products in a flavour come close to the scale (fx::accepted): rows r1 (and r2
-// against both null vectors: every one of the four dots) and this lane's solve.
-static __device__ __noinline__ bool fx_carries(int n, int rho, const int4* __restrict__ r1, const int4* __restrict__ r2,
-                                               const unsigned short* lab, const int4* Y, int T) {
-  int p11 = 0, p12 = 0, p21 = 0, p22 = 0;
-#pragma unroll 1
-  for (int q = 0; q < n; q++) {
-    const int o = lab[q * 32];
-    const int4 a = __ldg(r1 + o), z = Y[q * T];
-    p11 = max(p11, fx::product_magnitude(a, z));
-    if (rho == 2) {
-      const int4 b = __ldg(r2 + o), z2 = Y[(n + q) * T];
-      p12 = max(p12, fx::product_magnitude(a, z2));
-      p21 = max(p21, fx::product_magnitude(b, z));
-      p22 = max(p22, fx::product_magnitude(b, z2));
-    }
-  }
-  return (rho == 2 ? min(min(p11, p12), min(p21, p22)) : p11) >= fx::kCarries;
-}
-
 // One member's determinant in FP64 from a fixed-point solve, with the FP64 lemma guard: the pairs
 // whose fixed-point value is out of range, too small to be sure of, or near the guard.  The solve's
 // entries carry at least the accuracy of FP64 ones at their largest entry's scale, which is the guard's
 // scale; where every product is far below it and the determinant too, that is not enough, and the pair
-// is refactored (bounds as fx::accepted, with floor exponents).
+// is refactored (kFloorBits and kCarryBits, with floor exponents).
 static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S, int L, int n, int rho,
                                             const int32_t* __restrict__ lab, const int32_t* __restrict__ col,
                                             const int4* Y, int T, int e, dev::cd factor, int kc, bool* fail) {
@@ -570,6 +550,34 @@ static __device__ __noinline__ dev::cd fx_member64(const dev::cd* __restrict__ S
   const bool carried = min(p11, p12) >= eb + ez - fx::kCarryBits && min(p21, p22) >= e2 + ez - fx::kCarryBits;
   *fail = ed < es - kc || (ed < es - fx::kFloorBits2 && !carried);
   return d;
+}
+
+// A sum of products of two dots (of one dot with nf = 1) in FP64; e: the exponent of their scale, lf: the
+// lane's factors.
+__device__ __forceinline__ double2 fx_sum(const fx::Acc2& s, int nf, int e, double2 lf) {
+  double re, im;
+  if (nf == 1) {
+    re = (double)s.rp;
+    im = (double)s.ih;
+    e -= fx::kDotBits;
+  } else {
+    constexpr double k30 = 1073741824.0;
+    re = fma((double)s.hi_re(), k30, (double)s.lo_re());
+    im = fma((double)s.hi_im(), k30, (double)s.lo_im());
+    e += 30 - 2 * fx::kSplitBits;
+  }
+  return dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
+}
+// One member's product: a call, as the member loop needs it now and then only.
+static __device__ __noinline__ double2 fx_far(fx::Val u, fx::Val t, int nf, int e, double2 lf) {
+  fx::Acc2 s;
+  if (nf == 1) {
+    s.rp = u.re;
+    s.ih = u.im;
+  } else {
+    fx::mac(s, fx::split(u), fx::split(t));
+  }
+  return fx_sum(s, nf, e, lf);
 }
 
 // One work item (family W x sink tile) by the whole thread block; the block's sum goes
@@ -797,39 +805,21 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
   } else {
     // Sum of the members' products at the family's exponent, in integers: to FP64 every kFlush members.
     fx::Acc2 tot;
-    auto add = [&](const fx::Acc2& s, int d) {  // acc += s, d binades below that exponent
-      double re, im;
-      int e = a.fx.fexp[W] + le - d;
-      if (a.fx.nf == 1) {
-        re = (double)s.rp;
-        im = (double)s.ih;
-        e -= fx::kDotBits;
-      } else {
-        constexpr double k30 = 1073741824.0;
-        re = fma((double)s.hi_re(), k30, (double)s.lo_re());
-        im = fma((double)s.hi_im(), k30, (double)s.lo_im());
-        e += 30 - 2 * fx::kSplitBits;
-      }
-      const double2 v = dev::cmul(make_double2(fx::scale2(re, e), fx::scale2(im, e)), lf);
+    auto add = [&]() {
+      const double2 v = fx_sum(tot, a.fx.nf, a.fx.fexp[W] + le, lf);
       acc.x += v.x;
       acc.y += v.y;
+      tot = fx::Acc2();
     };
-    auto term = [&](fx::Acc2& s, fx::Val u, fx::Val t) {  // s += u t; u alone with one flavour
-      if (a.fx.nf == 1) {  // kFlush values below 2^60
-        s.rp += u.re;
-        s.ih += u.im;
-      } else {
-        fx::mac(s, fx::split(u), fx::split(t));
-      }
-    };
-    const int thr1 = fx::threshold(a.kc, 1), thr2 = fx::threshold(a.kc, 2);
-    const int sure1 = fx::accepted(a.kc, 1), sure2 = fx::accepted(a.kc, 2);
+    constexpr int kFloorN = NCMAX <= 8 ? 8 : 18;
+    const int thr1 = fx::accepted(kFloorN, a.kc, 1), thr2 = fx::accepted(kFloorN, a.kc, 2);
     // members four at a time (a step that they do not fill repeats the last one)
     constexpr int kN = 4;
     const int step = fxm ? kN : 1;
     for (int c = 0; c < kW; c += step) {
       unsigned slow = 15;  // bit k: this lane's pair with member c + k goes through FP64
       if (fxm) {
+        const unsigned ds = __ldg(a.fx.align + mem0 + c);
         fx::Val u[kN], t[kN];
         int at = 0;
         slow = 0;
@@ -837,7 +827,6 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           const int n = a.n_f[f], L = a.L_f[f];
           if (n == 0) continue;
           const int rho = a.fam_rank[(int64_t)W * a.F + f];
-          const unsigned before = slow;  // by an earlier flavour
           const unsigned short* lb = lab + a.yoff[f] * 32;
           const int4* Yf = reinterpret_cast<const int4*>(Y + (size_t)a.yoff[f] * T);
           fx::Val v[kN];
@@ -857,53 +846,49 @@ __device__ __forceinline__ void fwd_item(const FwdArgs& a, int W, int tile, doub
           } else {
             fx_dots<kN>(n, r, lb, Yf, T, v);
           }
-          const int thr = rho == 2 ? thr2 : thr1, sure = rho == 2 ? sure2 : sure1;
-          unsigned look = 0;  // values that the guard lets pass, but small: it depends on the products
+          const int thr = rho == 2 ? thr2 : thr1;
   #pragma unroll
           for (int k = 0; k < kN; k++) {
-            const int mag = fx::magnitude(v[k]);
-            const bool ok = fx::usable(mag, sure);
             u[k] = at == 0 ? v[k] : u[k];
             t[k] = v[k];
-            look |= (unsigned)(!ok && c + k < kW && fx::usable(mag, thr)) << k;
-            slow |= (unsigned)!ok << k;
-          }
-          for (unsigned todo = __reduce_or_sync(0xffffffffu, look); todo; todo &= todo - 1) {
-            const int k = __ffs(todo) - 1, m = mem0 + c + k;
-            const int32_t* mlab = a.mem_lab + ((int64_t)m * a.F + f) * MHC_MAX_RANK;
-            const int4* r1 = at == 0 ? a.fx.ws + (size_t)m * L : a.fx.s[f] + (size_t)mlab[0] * L;
-            const bool two = NCMAX >= 10 && rho == 2;
-            if (fx_carries(n, two ? 2 : 1, r1, a.fx.s[f] + (size_t)mlab[two ? 1 : 0] * L, lb, Yf, T))
-              slow &= ~(look & (1u << k) & ~before);
+            slow |= (unsigned)!fx::usable(fx::magnitude(v[k]), thr) << k;
           }
           at++;
         }
-        unsigned far = 0;  // members that their family's exponent would cost too many bits
+        unsigned far = 0;
+        if (ds & 0x80808080u) {
+  #pragma unroll
+          for (int k = 0; k < kN; k++) {
+            const unsigned d = (ds >> (8 * k)) & 255u;
+            far |= (unsigned)(d == fx::kFar) << k;
+            slow |= (unsigned)(d == fx::kOnlyFp64) << k;
+          }
+        }
   #pragma unroll
         for (int k = 0; k < kN; k++) {
-          const int d = __ldg(a.fx.shift + mem0 + min(c + k, kW - 1));
-          if (d == fx::kNever) slow |= 1u << k;
-          const bool use = c + k < kW && !((slow >> k) & 1) && fx::aligns(d, a.fx.nf);
-          far |= (unsigned)(c + k < kW && !fx::aligns(d, a.fx.nf) && d < fx::kMute) << k;
-          const int du = !use ? 0 : a.fx.nf == 1 ? d : d >> 1, dt = use ? d - du : 0;
-          term(tot, use ? fx::aligned(u[k], du) : fx::Val{0, 0}, fx::aligned(t[k], dt));
+          const unsigned d = (ds >> (8 * k)) & 255u;
+          const bool use = d < fx::kFar && !((slow >> k) & 1);
+          if (a.fx.nf == 1) {  // kFlush values below 2^60
+            const fx::Val x = fx::rounded(u[k], d & 31u);
+            tot.rp += use ? x.re : 0;
+            tot.ih += use ? x.im : 0;
+          } else {
+            const fx::Val x = d & 127u ? fx::aligned(u[k], d & 31u) : u[k];
+            fx::mac(tot, fx::split(use ? x : fx::Val{0, 0}), fx::split(t[k]));
+          }
         }
-        if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) {
-          add(tot, 0);
-          tot = fx::Acc2();
-        }
+        if (((c + kN) & (fx::kFlush - 1)) == 0 || c + kN >= kW) add();
         while (far) {
           const int k = __ffs(far) - 1;
           far &= far - 1;
-          const bool p = (slow >> k) & 1;
-          const fx::Val uk = k == 0 ? u[0] : k == 1 ? u[1] : k == 2 ? u[2] : u[3];
-          fx::Acc2 one;
-          term(one, p ? fx::Val{0, 0} : uk, k == 0 ? t[0] : k == 1 ? t[1] : k == 2 ? t[2] : t[3]);
-          add(one, __ldg(a.fx.shift + mem0 + c + k));
+          const fx::Val x = k == 0 ? u[0] : k == 1 ? u[1] : k == 2 ? u[2] : u[3];
+          const fx::Val y = k == 0 ? t[0] : k == 1 ? t[1] : k == 2 ? t[2] : t[3];
+          const double2 v = fx_far(x, y, a.fx.nf, a.fx.fexp[W] + le - __ldg(a.fx.below + mem0 + c + k), lf);
+          if (!((slow >> k) & 1)) acc = dev::cadd(acc, v);
         }
       }
-      // pairs out of the fixed-point range or near the lemma guard (every pair of a family or warp that
-      // the format does not take)
+      // pairs out of the fixed-point range or below its floor (every pair of a family or warp that the format
+      // does not take)
       slow &= (1u << min(step, kW - c)) - 1u;
       for (unsigned todo = __reduce_or_sync(0xffffffffu, slow); todo; todo &= todo - 1) {
         const int k = __ffs(todo) - 1;
@@ -974,13 +959,22 @@ __device__ __forceinline__ void fold_partials(const FwdArgs& a, double2* smem) {
 // Registers: the n <= 8 class keeps 168 (12 one-warp blocks per SM, or 3 blocks of its
 // 128-thread tile); the larger classes may use all 255, measured fastest for n = 18 (8 blocks
 // per SM against 9 at 216 and 10 at 200, whose spills cost more than the warps gain).
-// FX: the call has fixed-point tables, or complex weights; else the kernel holds the FP64 path for
+// FX: the plan has fixed-point tables, or the weights are complex; else the kernel holds the FP64 path for
 // real weights alone (n <= 32: for both).  512 x 512 terms of n = 3: 55 us per call, and 64 us when it
 // also carried the complex weights, converted solves for the refactors and a launch for the partials'
-// sum.  The FX kernel keeps the FP64 path apart, as a copy of its own, for plans without tables
-// and for propagators that are not flat.
-template <int NCMAX, bool FX>
-__global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) {
+// sum.  The FX kernels (CW: for complex weights, else real ones) keep the FP64 path apart, for plans without
+// tables and for propagators that are not flat: a copy of its own, for n <= 8 called, so that its registers
+// stay out of the other's (4096 x 4096 terms of n = 6: 1177 us, 1200 us inlined; n = 9, 7 with families of
+// three 1983 us, 1895 us inlined).  The arguments stay in constant memory (__grid_constant__): calls take
+// their address, for which every thread had copied all 1.4 KB of them (n = 9, 7: 2185 us; n = 18, 4096 x 4096
+// terms 9.8 ms, 9.3 ms without the copy).
+template <int NCMAX, bool CW>
+__device__ __noinline__ void fwd_item_fp64(const FwdArgs& a, int W, int tile, double2* partial) {
+  extern __shared__ double2 smem[];
+  fwd_item<NCMAX, false, CW>(a, W, tile, smem, partial);
+}
+template <int NCMAX, bool FX, bool CW>
+__global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const __grid_constant__ FwdArgs a) {
   extern __shared__ double2 smem[];
   const int64_t item = a.item0 + blockIdx.x;
   const int64_t pos = item / a.n_tiles;
@@ -988,11 +982,13 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const FwdArgs a) 
   const int tile = (int)(item % a.n_tiles);
   if constexpr (FX) {
     if (dev::fx_on(a))
-      fwd_item<NCMAX, true, true>(a, W, tile, smem, &a.partials[item]);
+      fwd_item<NCMAX, true, CW>(a, W, tile, smem, &a.partials[item]);
+    else if (NCMAX <= 8)
+      fwd_item_fp64<NCMAX, CW>(a, W, tile, &a.partials[item]);
     else
-      fwd_item<NCMAX, false, true>(a, W, tile, smem, &a.partials[item]);
+      fwd_item<NCMAX, false, CW>(a, W, tile, smem, &a.partials[item]);
   } else {
-    fwd_item<NCMAX, false, (NCMAX > 18)>(a, W, tile, smem, &a.partials[item]);
+    fwd_item<NCMAX, false, CW>(a, W, tile, smem, &a.partials[item]);
   }
   if (a.fold_items > 0) fold_partials(a, smem);
 }
@@ -1453,12 +1449,12 @@ int batch_occupancy_nc(int T, size_t smem) {
   return nb > 0 ? nb : 1;
 }
 
-template <int NCMAX, bool FX>
+template <int NCMAX, bool FX, bool CW>
 cudaError_t launch_fwd_nc(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(fwd::fwd_kernel<NCMAX, FX>,
+  cudaError_t e = cudaFuncSetAttribute(fwd::fwd_kernel<NCMAX, FX, CW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fwd::fwd_kernel<NCMAX, FX><<<(unsigned)items, tile, smem, s>>>(a);
+  fwd::fwd_kernel<NCMAX, FX, CW><<<(unsigned)items, tile, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -5,7 +5,9 @@
 namespace mhc {
 
 cudaError_t launch_fwd_nc18(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  return a.fx.nf > 0 || a.w_src_im ? launch_fwd_fx_nc18(a, tile, items, smem, s) : launch_fwd_nc<18, false>(a, tile, items, smem, s);
+  if (a.w_src_im) return launch_fwd_cw_nc18(a, tile, items, smem, s);
+  if (a.fx.nf > 0) return launch_fwd_fx_nc18(a, tile, items, smem, s);
+  return launch_fwd_nc<18, false, false>(a, tile, items, smem, s);
 }
 
 cudaError_t launch_kfac_nc18(const FwdArgs& a, int64_t n_fam, cudaStream_t s) {

@@ -5,7 +5,7 @@
 namespace mhc {
 
 cudaError_t launch_fwd_nc32(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s) {
-  return launch_fwd_nc<32, false>(a, tile, items, smem, s);
+  return launch_fwd_nc<32, false, true>(a, tile, items, smem, s);
 }
 
 cudaError_t launch_kfac_nc32(const FwdArgs& a, int64_t n_fam, cudaStream_t s) {

@@ -13,10 +13,9 @@
 // 2^52 per product against 2^111 for the vectors' scale in a dot.  A dot is off by less than
 // (2 n) 2^-56 |g|max |y|max then.  That is a quarter of what an FP64 chain may be off by when its
 // largest product has that size, and more than FP64's error when all products are far smaller.  So a
-// dot well below the scale is used only after a look at the products (accepted, below), and one below
-// 2^-kc of it (kc: the lemma guard's exponent) or above eight times it never: the FP64 path forms that
-// determinant again and applies its own guard, so which pairs are refactored does not depend on this
-// arithmetic.  (Random blocks of n = 6 to 18: the median dot is 2^-1.7 of the scale, one in a thousand
+// dot below a floor (accepted, below), below 2^-kc of the scale (kc: the lemma guard's exponent) or above
+// eight times it is not used: the FP64 path forms that determinant again and applies its own guard, so
+// which pairs the guard has refactored does not depend on this arithmetic.  (Random blocks of n = 6 to 18: the median dot is 2^-1.7 of the scale, one in a thousand
 // lies above 2^0.6 to 2^1.)
 #pragma once
 
@@ -35,10 +34,11 @@ constexpr int kRowBits = 55;            // a propagator row: |entry| <= 2^55
 constexpr int kDotBits = 57;            // a dot: 2^57 stands for the product of the scales
 constexpr int kMaxHi = 1 << 28;         // high word of 2^60: a larger dot is not used
 constexpr int kMulHi = 1 << 27;         // high word of 2^59: the largest factor of mul
-constexpr int kNever = 0x7fffffff;      // a threshold that no value reaches; Tables::shift: the FP64
-                                        // path evaluates the member
-constexpr int kMute = 0x7ffffffe;       // Tables::shift: the member's weight is zero
-constexpr int kMaxAlign = 4;            // most bits of a dot that its family's common exponent may cost
+constexpr int kNever = 0x7fffffff;      // a threshold that no value reaches
+// Tables::align, other than the binades up to kMaxAlign: the member lies further below, adds nothing
+// (its weight is zero, or there is no such member), or is evaluated by the FP64 path
+enum : unsigned { kFar = 128, kMute = 129, kOnlyFp64 = 130 };
+constexpr int kMaxAlign = 8;            // most bits of a dot that its family's common exponent may cost
 constexpr int kFlush = 8;               // members per 64-bit sum of products (Acc2)
 constexpr int kMaxMembers = 64;
 
@@ -131,24 +131,21 @@ __device__ __forceinline__ int threshold(int kc, int rank) {
   return t >= 28 ? kNever : t <= 0 ? 1 : 1 << t;
 }
 
-// High word of the smallest |value| accepted by itself, whatever the guard allows.  A dot is off by a
-// few units of 2^57 2^-56 times the square root of n, so a value of 2^(57 - kFloorBits) by some 2^-48 of
-// itself (a two-row determinant has three bits more to give: its two dots are each off by as little).  A
-// smaller one may be a sum of large products that cancel, where FP64 is off as much: it is accepted
-// when the largest product is within kCarryBits binades of the scale.  Or every product is far below the
-// scale, as the row is large where the solve is small: then FP64 rounds each product at its own size,
-// and the FP64 path evaluates the pair.  On random blocks of n = 3 to 18 one dot in 700 lies below the
-// floor.
-constexpr int kFloorBits = 7;
-constexpr int kFloorBits2 = 10;  // of a two-row determinant, 2^56 for the scales
-constexpr int kCarryBits = 4;
-constexpr int kCarries = 1 << (kDotBits - kCarryBits - 32);
-__device__ __forceinline__ int accepted(int kc, int rank) {
-  return max(threshold(kc, rank), 1 << (rank == 1 ? kDotBits - 32 - kFloorBits : kDotBits - 1 - 32 - kFloorBits2));
-}
-// high word of the product of the larger components' high limbs, 2^57 for the scale
-__device__ __forceinline__ int product_magnitude(int4 a, int4 b) {
-  return (int)(madw(max(abs(a.x), abs(a.z)), max(abs(b.x), abs(b.z)), 0) >> 32);
+// High word of the smallest |value| that is used: the guard's threshold, and a floor that no guard lowers.  A
+// dot is off by a few units of 2^57 2^-56 times the square root of n, so a value of 2^(57 - kFloorBits)
+// by some 2^-46 of itself (2^-45 for n > 8); a two-row determinant's two dots are each off by as little.  A
+// smaller one may be a sum of large products that cancel, where FP64 is off as much, or all its products may
+// be far below the scale: the FP64 path tells (fx_member64).  Of the dots of random blocks one in 20 000 lies
+// below 2^-9 of the scale, one in 80 000 below 2^-10, where the default lemma guard sends it there anyway; an
+// evaluation takes its warp as long as 10 to 20 members in fixed point, and more for n > 8.  (4096 x 4096
+// terms of n = 6: floors of 2^-10, 2^-9, 2^-8 1095, 1112, 1150 us; small pairs queued for refactors, of which an
+// item has one at a time, 1360 to 1520 us.)
+constexpr int kFloorBits = 9, kFloorBitsLarge = 10;  // n <= 8; above
+constexpr int kFloorBits2 = 12;  // of a two-row determinant, 2^56 for the scales
+constexpr int kCarryBits = 4;    // a product this many binades below the scale still carries a small value
+__device__ __forceinline__ int accepted(int n, int kc, int rank) {
+  const int bits = rank == 2 ? 1 + kFloorBits2 : n <= 8 ? kFloorBits : kFloorBitsLarge;
+  return max(threshold(kc, rank), 1 << (kDotBits - 32 - bits));
 }
 
 // Products of two dots.  A dot's scale is an upper bound that it stays a few binades below: the product
@@ -161,13 +158,15 @@ __device__ __forceinline__ int4 split(Val v) {
   const int rh = (int)((v.re + (1ll << 30)) >> 31), ih = (int)((v.im + (1ll << 30)) >> 31);
   return make_int4(rh, (int)(v.re >> 1) - (rh << 30), ih, (int)(v.im >> 1) - (ih << 30));
 }
-// A member whose product lies d binades below its family's exponent: its two dots shifted by half of d
-// each, a single one by d.  Up to kMaxAlign a dot stays as accurate as FP64 would form it (2^-57 2^4 of the
-// scale, half a unit of it on average); a member further down is summed in FP64 by itself.
-__device__ __forceinline__ bool aligns(int d, int flavours) { return d <= flavours * kMaxAlign; }
-__device__ __forceinline__ Val aligned(Val v, int d) {
-  const long long half = (1ll << d) >> 1;
-  return Val{(v.re + half) >> d, (v.im + half) >> d};
+// A member whose product lies d binades below its family's exponent: its first dot in that exponent's units.
+// Beside the larger members' own errors the bits it loses are nothing; where those members vanish, kMaxAlign
+// leaves it 2^-49 of its scale.  A member further down (one in 100 with normal weights) is summed in
+// FP64 by itself.  The shift rounds down: its mean of half a unit is multiplied by the second dot, whose
+// phase it does not know; a single dot is rounded to the nearest instead.
+__device__ __forceinline__ Val aligned(Val v, int d) { return Val{v.re >> d, v.im >> d}; }
+__device__ __forceinline__ Val rounded(Val v, int d) {
+  const unsigned half = (1u << d) >> 1;
+  return aligned(Val{v.re + half, v.im + half}, d);
 }
 struct Acc2 : Acc {
   long long qp = 0, qn = 0, qi = 0;  // lo lo
@@ -424,8 +423,10 @@ struct Tables {
   int* state;                   // [0] 1: the propagators are flat (Scan), [1] rows scanned, 0 between calls
   const int4* ws;               // [members][L_f0] first flavour's first member row times the weight (as
                                 // it is where that is zero), with an exponent of its own
-  const int* shift;             // [members] binades by which the member's product scale lies below its
-                                // family's, or kMute, or kNever
+  const unsigned* align;        // [members] at a family's member 0, 4, 8 ...: a byte for it and the next
+                                // three, binades by which the member's product scale lies below its
+                                // family's, or kFar, kMute, kOnlyFp64
+  const int* below;             // [members] those binades of a kFar member
   const int* fexp;              // [W] exponent of the family's products: its largest member's
   int f0, nf;                   // first flavour with n_f > 0; flavours with n_f > 0 (0: no tables)
 };

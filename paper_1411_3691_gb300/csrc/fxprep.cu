@@ -18,7 +18,7 @@ namespace mhc {
 
 namespace {
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 512;  // a warp per member of a family of 16: one chain of loads each
 
 // exponent above every used entry of a row or column (largest binary exponent + 1); one warp
 __device__ __forceinline__ int row_exponent(const dev::cd* row, int pitch, int L, int lane, const int* used, int bit) {
@@ -133,18 +133,21 @@ __device__ void prep_family(const FwdArgs& a, int W) {
       if (a.n_f[f] == 0) continue;
       for (int t = 0; t < a.fam_rank[(int64_t)W * a.F + f]; t++) {
         const dev::cd* row = a.S[f] + (size_t)lab[f * MHC_MAX_RANK + t] * a.L_f[f];
-        const int e = row_exponent(row, 1, a.L_f[f], lane, a.fx.used[f], 2);
-        bad |= e > 1023 || e < -1000;
-        if (f == f0 && t == 0) {
-          for (int l = lane; l < L0; l += 32)
-            if (a.fx.used[f][l] & 2) e0 = max(e0, dev::expo(weighted(a, w, dev::ldS(row + l))));
-          e0 = __reduce_max_sync(0xffffffffu, e0) + 1;
-          bad |= e0 > 1023 || e0 < -1000;
-        } else {
-          r += e;
+        const bool first = f == f0 && t == 0;
+        int e = -4096;
+        for (int l = lane; l < a.L_f[f]; l += 32) {
+          if (!(a.fx.used[f][l] & 2)) continue;
+          const dev::cd z = dev::ldS(row + l);
+          e = max(e, dev::expo(z));
+          if (first) e0 = max(e0, dev::expo(weighted(a, w, z)));
         }
+        e = __reduce_max_sync(0xffffffffu, e) + 1;
+        bad |= e > 1023 || e < -1000;
+        if (!first) r += e;
       }
     }
+    e0 = __reduce_max_sync(0xffffffffu, e0) + 1;
+    bad |= e0 > 1023 || e0 < -1000;
     if (lane == 0) {
       ws[c] = w;
       e0s[c] = bad ? -100000 : e0;
@@ -155,12 +158,20 @@ __device__ void prep_family(const FwdArgs& a, int W) {
   int X = -100000;
   for (int c = 0; c < kW; c++)
     if (e0s[c] > -100000 && !is_zero(ws[c])) X = max(X, e0s[c] + rest[c]);
-  if (threadIdx.x == 0) const_cast<int*>(a.fx.fexp)[W] = X;
+  if (threadIdx.x == 0) {
+    const_cast<int*>(a.fx.fexp)[W] = X;
+    for (int c = kW; c & 3; c++)  // a step of four that the family does not fill
+      reinterpret_cast<unsigned char*>(const_cast<unsigned*>(a.fx.align + mem0 + (c & ~3)))[c & 3] = fx::kMute;
+  }
   for (int c = warp; c < kW; c += kThreads / 32) {
     const int m = mem0 + c;
     const bool bad = e0s[c] == -100000;
-    if (lane == 0)
-      const_cast<int*>(a.fx.shift)[m] = bad ? fx::kNever : is_zero(ws[c]) ? fx::kMute : X - e0s[c] - rest[c];
+    if (lane == 0) {
+      const int d = X - e0s[c] - rest[c];
+      const_cast<int*>(a.fx.below)[m] = d;
+      reinterpret_cast<unsigned char*>(const_cast<unsigned*>(a.fx.align + mem0 + (c & ~3)))[c & 3] =
+          bad ? fx::kOnlyFp64 : is_zero(ws[c]) ? fx::kMute : d > fx::kMaxAlign ? fx::kFar : d;
+    }
     const int32_t lab = a.mem_lab[((int64_t)m * a.F + f0) * MHC_MAX_RANK];
     const dev::cd* row = a.S[f0] + (size_t)lab * L0;
     int4* out = const_cast<int4*>(a.fx.ws) + (size_t)m * L0;

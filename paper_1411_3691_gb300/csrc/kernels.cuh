@@ -408,6 +408,8 @@ size_t forward_smem_bytes(int slots, int tile, int ncmax, bool tables);
   cudaError_t launch_kfac_batch_nc##NC(const FwdArgs* desc, const int64_t* kpref,            \
                                        const int64_t* nfam, int count, int64_t total,         \
                                        int big, cudaStream_t s);
+cudaError_t launch_fwd_cw_nc8(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
+cudaError_t launch_fwd_cw_nc18(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
 cudaError_t launch_fwd_fx_nc8(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
 cudaError_t launch_fwd_fx_nc18(const FwdArgs& a, int tile, int64_t items, size_t smem, cudaStream_t s);
 MHC_DECL_NC(8)

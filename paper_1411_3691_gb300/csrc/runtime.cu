@@ -118,7 +118,8 @@ size_t fx_layout(const Plan& p, char* base, fx::Tables* t) {
     return 0;
   }
   t->ws = reinterpret_cast<const int4*>(take((size_t)p.n_src * p.L_f[t->f0] * sizeof(int4)));
-  t->shift = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
+  t->align = reinterpret_cast<const unsigned*>(take((size_t)p.n_src * sizeof(unsigned)));
+  t->below = reinterpret_cast<const int*>(take((size_t)p.n_src * sizeof(int)));
   t->fexp = reinterpret_cast<const int*>(take((size_t)p.n_fam * sizeof(int)));
   t->state = reinterpret_cast<int*>(take(2 * sizeof(int)));
   return off;

@@ -165,15 +165,13 @@ int main(int argc, char** argv) {
         if (fail) continue;  // refactored
         fx::Acc s;
         std::vector<int4> row(n);
-        int largest = 0;
         for (int q = 0; q < n; q++) {
           row[q] = fx::quant(S[(size_t)m * L + c[q]], rexp[m], fx::kRowBits);
           fx::mac(s, row[q], y[q]);
-          largest = max(largest, fx::product_magnitude(row[q], y[q]));
         }
         const fx::Val v = fx::finish(s);
         const int mag = fx::magnitude(v);
-        if (!fx::usable(mag, fx::accepted(kc, 1)) && !(fx::usable(mag, fx::threshold(kc, 1)) && largest >= fx::kCarries)) {
+        if (!fx::usable(mag, fx::accepted(n, kc, 1))) {
           left++;
           continue;
         }

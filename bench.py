@@ -49,14 +49,14 @@ NOMINAL_FP64_TFLOPS = 2 * 152 * 2.07e9 * 2 / 1e12
 # dram__bytes_read.sum + dram__bytes_write.sum of every kernel of one forward call, from one
 # ncu capture of the current kernels.  The large nucleus holds 9.7 GB of block factors, too much
 # for a multi-metric capture, so its 1/8-per-side copy (--workload large_small: 1/64 of the pairs
-# and of the (family, sink family) blocks) was captured and the sum scaled by 64: 165.9 MB read
-# + 99.5 MB written per call of the copy (kfac_kernel, kfac_group_kernel, three fwd_kernel
-# launches, reduce_kernel).
+# and of the (family, sink family) blocks) was captured and the sum scaled by 64: 178.8 MB read
+# + 102.9 MB written per call of the copy (fxprep_kernel, kfac_kernel, kfac_group_kernel, three
+# fwd_kernel launches, reduce_kernel).
 TRAFFIC = {
-    "large": {"bytes": 269.78e6 * 64,
+    "large": {"bytes": 281.6e6 * 64,
               "source": "ncu dram__bytes_read + dram__bytes_write of every kernel of one call of the "
                         "1/8-per-side copy (--workload large_small), x 64"},
-    "he4": {"bytes": 108.71e6,
+    "he4": {"bytes": 126.4e6,
             "source": "ncu dram__bytes_read + dram__bytes_write of every kernel of one call"},
 }
 

@@ -317,7 +317,7 @@ mhc_status mhc_correlator_noalloc(mhc_plan_t plan, const double* const* S_f,
                                   double* out_dev, mhc_stream_t stream);
 
 /*
- * Per-pair determinants through the same update path (families, lemma, guards):
+ * Per-pair determinants by the update scheme (families, lemma, guards), in FP64:
  *   i_dev, j_dev : device int64 [n_pairs] source and sink term indices
  *   dets_dev     : device float64 [n_pairs][F][2], det of each flavour block in the
  *                  terms' own label order, written

@@ -1,12 +1,12 @@
-// fwd_impl.cuh -- forward correlator kernel and per-pair probe (templates; instantiated
-// once per n class by fwd_nc8.cu, fwd_nc18.cu and fwd_nc32.cu).
+// fwd_impl.cuh -- forward correlator kernel, block factors, batched kernel and per-pair probe
+// (templates; instantiated once per n class and kernel by fwd_*.cu, batch_nc*.cu and pair_nc*.cu).
 //
 // One thread block per work item (work family W, tile of `tile` sinks); one thread per
 // sink.  Per flavour a thread factorises the family's shared rows against its sink's
 // columns (shared_rows) and caches y = det(G) G^{-1} e_r in shared memory; then every
 // member of the family costs one O(n) dot product per flavour, Sec. 2.1: in fixed point on the
-// integer pipe (fx_dots, fx_det2), or in FP64 (member_det) where the fixed-point value is out of
-// its range or near the lemma guard.
+// integer pipe (fx_dots, fx_det2), or in FP64 (member_det) in calls without tables, on propagators that
+// do not suit them, and where a fixed-point value is out of its range, small, or near the lemma guard.
 // Two-sided blocks (a family against a sink family) take y from factors stored once per
 // block (kapply*).  Members whose lemma factor or whose family pivots fail the guards go
 // to a per-warp queue and are refactored from scratch 32 at a time -- pairs that share the
@@ -996,7 +996,7 @@ __global__ void __maxnreg__(NCMAX <= 8 ? 168 : 255) fwd_kernel(const __grid_cons
 // Flavours of a pair that pair_group_kernel takes: blocks that do not fit in a thread's registers.
 __device__ __forceinline__ bool pair_grouped(int n, int rho) { return n > 6 && rho <= 2; }
 
-// Per-pair determinants through the same update path (one thread per pair): the flavours with
+// Per-pair determinants by the update scheme in FP64 (one thread per pair): the flavours with
 // n <= 6 or more than two changed rows.
 template <int NCMAX>
 __global__ void __launch_bounds__(64) pair_kernel(const FwdArgs a, int64_t n_pairs, int64_t n_src,

@@ -172,7 +172,10 @@ void mhc_plan_opts_default(mhc_plan_opts* opts);
  * The plan is reusable across propagators S_f (Sec. 3: the graph and the dominating
  * set do not depend on the gauge configuration).  Its device tables are uploaded by
  * the first device call that uses it (a synchronous copy on the current device);
- * issue that first call outside any stream capture.  Repeated labels are allowed and
+ * issue that first call outside any stream capture.  Two-sided plans of one or two flavours with
+ * n_f <= 18 and enough terms keep fixed-point tables of the propagators there as well, at most
+ * 4 GiB and usually a few MB (mhc_forward_info); without memory for them, with opts->one_sided and
+ * on propagators that do not suit them their calls run in FP64.  Repeated labels are allowed and
  * give det = 0.  n_f = 0 makes flavour f a factor 1.
  * Errors: MHC_EINVAL (bad sizes or labels, null pointers), MHC_ENOMEM.
  */
